@@ -25,18 +25,28 @@ cudaError_t launch_chor_answer(const CUtensorMap &db_map, const CUtensorMap &qt_
                                uint32_t B, uint32_t qtw, uint32_t *out, int num_sms, int *status,
                                cudaStream_t stream, int form);
 
-// Four-Russians path (large batches): box shape of its database map.
-constexpr uint32_t kChorM4TileWords = 64;
-constexpr uint32_t kChorM4BandRows = 64;
+// Tensor-core path (chor_gemm.cu): units of 256 rows x 16 words, up to 128 queries per pass.
+constexpr uint32_t kChorGemmUnitRows = 256;
+constexpr uint32_t kChorGemmUnitWords = 16;
+constexpr uint32_t kChorGemmMaxBatch = 128;
+// Rows per launch: bounds the expanded queries (64 bytes per row) and, far below 2^22, the counts.
+constexpr uint64_t kChorGemmRows = 1ull << 18;
+// Bytes of expanded queries for B queries of `units` units.
+constexpr uint64_t chor_gemm_query_bytes(uint32_t B, uint32_t units) { return 128ull * B * units; }
 
-// Q (B x qw words) -> QS (qw x 256 words): word k of query b at QS[k * 256 + b];
-// the buffer must hold roundup(qw, 2) x 256 words (a band reads two query words).
-cudaError_t launch_chor_words(const uint32_t *Q, uint64_t qw, uint32_t B, uint64_t r, uint32_t *QS, int num_sms,
-                              cudaStream_t stream);
+cudaError_t prepare_chor_gemm_kernels();
+// Query rows of a tile (32, 64 or 128) for B queries: the box height of q_map.
+uint32_t chor_gemm_n(uint32_t B);
 
-// out (B x W words, zeroed by the caller) ^= the responses of B <= 256 queries;
-// db_map covers the database {W, r} words with box {64, 64}.
-cudaError_t launch_chor_m4rm(const CUtensorMap &db_map, const uint32_t *QS, uint64_t r, uint32_t W, uint32_t B,
-                             uint32_t *out, int num_sms, int *status, cudaStream_t stream);
+// Q (B x qw words) -> QF: the bits of rows [row0, row0 + 256 units) as e2m1 ones, B rows of
+// 128 * units bytes; row0 a multiple of 32.
+cudaError_t launch_chor_nibbles(const uint32_t *Q, uint64_t qw, uint32_t B, uint64_t row0, uint32_t units, uint32_t *QF,
+                                cudaStream_t stream);
+
+// out (B x W words, zeroed by the caller) ^= the responses of B <= 128 queries over the rows
+// [row0, row0 + 256 units); db_map covers the database {W, r} words with box {16, 256} and 64-byte swizzle, q_map QF
+// {128 units, B} bytes with box {128, chor_gemm_n(B)} and 128-byte swizzle.
+cudaError_t launch_chor_gemm(const CUtensorMap &db_map, const CUtensorMap &q_map, uint64_t row0, uint32_t units,
+                             uint32_t W, uint32_t B, uint32_t *out, int num_sms, int *status, cudaStream_t stream);
 
 }  // namespace qpadl

@@ -94,16 +94,25 @@ struct qpadl_chor {
     const uint32_t *db = nullptr;    // caller-owned, rows x W words
     int device = 0;
     int num_sms = 0;
-    uint32_t *qt = nullptr;          // selector scratch: rows x 8 words or ceil(rows/32) x 256 words
+    uint32_t *qt = nullptr;          // selector scratch: rows x 8 words, or expanded queries (chor_gemm.cu)
     int *d_status = nullptr;
     uint64_t owned_bytes = 0;
-    uint32_t m4rm_min_batch = 48;    // batches from this size take the four-Russians kernel
+    uint32_t large_min_batch = 48;   // QPADL_CHOR_OPT_M4RM_MIN_BATCH: batches from this size take the tensor cores
+    bool large_set = false;          // ... set by the caller (else chor_large_batch)
     int scan_form = -1;              // QPADL_CHOR_OPT_SCAN_FORM (-1: by batch size)
 };
 
 namespace {
 
 constexpr int kMaxN = 16384;
+// Smallest Chor batch on the tensor cores for records of W words, unless the caller chose one.  Their
+// time hardly depends on the batch up to 64 queries; the scan's grows with it and its column tiles
+// are 1024 words wide (one query; a narrower record leaves their threads idle).  Measured, scan
+// against tensor cores: 16 words (2^20 rows of 4: 536 against 83 us; 200,000 of 16: 111 / 20), 256
+// words (60,000 rows) 41 / 26 us at one query; 768 words (2^18 rows) 148 / 187 us at one, 159 / 189
+// at 2, 195 / 189 at 3; 8192 words (32,768 rows) 241 / 251 at 8 and 356 / 251 at 9.
+uint32_t chor_large_batch(uint32_t W) { return W < 512 ? 1u : (W < 1024 ? 3u : 9u); }
+uint32_t chor_units(uint64_t rows) { return static_cast<uint32_t>((rows + kChorGemmUnitRows - 1) / kChorGemmUnitRows); }
 // Goldberg sums stay exact (|centred sum| < 2^31, unsigned sum < 2^32) below this many columns
 constexpr uint64_t kGoldbergMaxCols = 65792;
 
@@ -161,6 +170,7 @@ int prepare_device(int dev) {
     QPADL_CU(prepare_limb_gemm_u8_kernels());
     QPADL_CU(prepare_client_kernels());
     QPADL_CU(prepare_chor_kernels());
+    QPADL_CU(prepare_chor_gemm_kernels());
     prepared[dev] = true;
     return QPADL_OK;
 }
@@ -1209,7 +1219,10 @@ int qpadl_chor_setup(uint64_t rows, uint64_t bits, const uint32_t *db_dev, qpadl
         return fail(QPADL_ECUDA);
     int rc = prepare_device(h->device);
     if (rc != QPADL_OK) return fail(rc);
-    const uint64_t qt_bytes = 4ull * std::max<uint64_t>(rows * 8, (h->qw + 1) / 2 * 2 * kChorMaxBatch);
+    // selector bits of the scans, or one launch's expanded queries of the tensor-core path
+    const uint64_t block_rows = std::min<uint64_t>(rows, kChorGemmRows);
+    const uint64_t qt_bytes =
+        std::max<uint64_t>(32 * rows, chor_gemm_query_bytes(kChorGemmMaxBatch, chor_units(block_rows)));
     if (cudaMalloc(reinterpret_cast<void **>(&h->qt), qt_bytes) != cudaSuccess ||
         cudaMalloc(reinterpret_cast<void **>(&h->d_status), 16) != cudaSuccess) {
         cudaGetLastError();
@@ -1222,6 +1235,33 @@ int qpadl_chor_setup(uint64_t rows, uint64_t bits, const uint32_t *db_dev, qpadl
     return QPADL_OK;
 }
 
+}  // extern "C"
+
+namespace {
+
+// Up to 128 queries on the tensor cores, kChorGemmRows rows at a time (the scratch holds one such
+// block's expanded queries; the launches of a stream follow one another).
+int chor_answer_gemm(qpadl_chor *h, const uint32_t *Q, uint32_t B, uint32_t *out, cudaStream_t s) {
+    const uint32_t W = h->words;
+    CUtensorMap db_map, q_map;
+    if (!encode_2d(&db_map, CU_TENSOR_MAP_DATA_TYPE_UINT32, h->db, W, h->rows, 4ull * W, kChorGemmUnitWords,
+                   kChorGemmUnitRows, CU_TENSOR_MAP_SWIZZLE_64B))
+        return QPADL_ECUDA;
+    for (uint64_t r0 = 0; r0 < h->rows; r0 += kChorGemmRows) {
+        const uint32_t units = chor_units(std::min(h->rows - r0, kChorGemmRows));
+        QPADL_CU(launch_chor_nibbles(Q, h->qw, B, r0, units, h->qt, s));
+        if (!encode_2d(&q_map, CU_TENSOR_MAP_DATA_TYPE_UINT8, h->qt, 128ull * units, B, 128ull * units, 128,
+                       chor_gemm_n(B), CU_TENSOR_MAP_SWIZZLE_128B))
+            return QPADL_ECUDA;
+        QPADL_CU(launch_chor_gemm(db_map, q_map, r0, units, W, B, out, h->num_sms, h->d_status, s));
+    }
+    return QPADL_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
 int qpadl_chor_answer_batch(qpadl_chor *h, const uint32_t *Q_dev, uint32_t B, uint32_t *out_dev,
                             qpadl_stream_t stream) {
     if (!h || !Q_dev || !out_dev || B == 0) return QPADL_EINVAL;
@@ -1231,16 +1271,13 @@ int qpadl_chor_answer_batch(qpadl_chor *h, const uint32_t *Q_dev, uint32_t B, ui
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const uint64_t W = h->words;
     QPADL_CU(cudaMemsetAsync(out_dev, 0, 4ull * W * B, s));
-    for (uint32_t b0 = 0; b0 < B; b0 += kChorMaxBatch) {
-        const uint32_t Bc = std::min(B - b0, kChorMaxBatch);
-        if (Bc >= h->m4rm_min_batch) {
-            QPADL_CU(launch_chor_words(Q_dev + (uint64_t)b0 * h->qw, h->qw, Bc, h->rows, h->qt, h->num_sms, s));
-            CUtensorMap db_map;
-            if (!encode_2d(&db_map, CU_TENSOR_MAP_DATA_TYPE_UINT32, h->db, W, h->rows, W * 4, kChorM4TileWords,
-                           kChorM4BandRows, CU_TENSOR_MAP_SWIZZLE_NONE))
-                return QPADL_ECUDA;
-            QPADL_CU(launch_chor_m4rm(db_map, h->qt, h->rows, static_cast<uint32_t>(W), Bc,
-                                      out_dev + (uint64_t)b0 * W, h->num_sms, h->d_status, s));
+    const uint32_t large = h->large_set || h->scan_form >= 0 ? h->large_min_batch : chor_large_batch(h->words);
+    for (uint32_t b0 = 0, Bc; b0 < B; b0 += Bc) {
+        Bc = std::min(B - b0, kChorMaxBatch);
+        if (Bc >= large) {
+            Bc = std::min(Bc, kChorGemmMaxBatch);
+            int rc = chor_answer_gemm(h, Q_dev + (uint64_t)b0 * h->qw, Bc, out_dev + (uint64_t)b0 * W, s);
+            if (rc != QPADL_OK) return rc;
             continue;
         }
         uint32_t tw = 0, rb = 0, boxw = 0, qtw = 0;
@@ -1266,7 +1303,8 @@ int qpadl_chor_set_option(qpadl_chor *h, int option, int64_t value) {
     switch (option) {
         case QPADL_CHOR_OPT_M4RM_MIN_BATCH:
             if (value < 1 || value > (int64_t)kChorMaxBatch + 1) return QPADL_EINVAL;
-            h->m4rm_min_batch = static_cast<uint32_t>(value);
+            h->large_min_batch = static_cast<uint32_t>(value);
+            h->large_set = true;
             return QPADL_OK;
         case QPADL_CHOR_OPT_SCAN_FORM:
             if (value < -1 || value > 3) return QPADL_EINVAL;
@@ -1279,7 +1317,7 @@ int qpadl_chor_set_option(qpadl_chor *h, int option, int64_t value) {
 int qpadl_chor_get_option(qpadl_chor *h, int option, int64_t *value) {
     if (!h || !value) return QPADL_EINVAL;
     switch (option) {
-        case QPADL_CHOR_OPT_M4RM_MIN_BATCH: *value = h->m4rm_min_batch; return QPADL_OK;
+        case QPADL_CHOR_OPT_M4RM_MIN_BATCH: *value = h->large_min_batch; return QPADL_OK;
         case QPADL_CHOR_OPT_SCAN_FORM: *value = h->scan_form; return QPADL_OK;
         default: return QPADL_EINVAL;
     }

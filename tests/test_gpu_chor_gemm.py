@@ -1,0 +1,54 @@
+"""Chor Response on the tensor cores at the edges of its tiles: rows around a unit of 256 and around
+the 2^18 rows of one launch, words around a column tile of 16, batches around 32, 64 and 128 query
+tiles; all-ones databases and queries (the largest counts); the default choice of kernel by record
+length.  Every answer equals the oracle's bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2510_03631_gb300 import inputs, pir
+
+pytestmark = pytest.mark.gpu
+
+
+def _dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a, dtype=np.uint32).view(np.int32).reshape(-1)).cuda()
+
+
+def _check(rows, bits, B, DB, Q, min_batch):
+    h = pir.qpadl_chor_setup(rows, bits, _dev(DB))
+    if min_batch:
+        pir.qpadl_chor_set_option(h, pir.QPADL_CHOR_OPT_M4RM_MIN_BATCH, min_batch)
+    out = torch.empty(B * h.words, dtype=torch.int32, device="cuda")
+    pir.qpadl_chor_answer_batch(h, _dev(Q), out)
+    assert pir.qpadl_chor_status(h) == pir.QPADL_OK
+    exp = oracle.chor_answer(DB, rows, Q, threads=oracle.max_threads())
+    assert np.array_equal(pir.as_u32(out).reshape(B, h.words), exp)
+    h.close()
+
+
+@pytest.mark.parametrize("rows", [1, 31, 255, 256, 257, 1025])
+@pytest.mark.parametrize("bits", [128, 512, 640, 4096 + 128])
+@pytest.mark.parametrize("B", [1, 32, 33, 64, 65, 128, 129])
+def test_tile_edges(rows, bits, B):
+    _check(rows, bits, B, inputs.chor_db(rows, bits, seed=rows + bits), inputs.chor_queries(B, rows, seed=rows * 3 + B), 1)
+
+
+@pytest.mark.parametrize("rows,B", [((1 << 18) - 1, 2), (1 << 18, 40), ((1 << 18) + 300, 70)])
+def test_rows_of_one_launch(rows, B):
+    _check(rows, 128, B, inputs.chor_db(rows, 128, seed=1), inputs.chor_queries(B, rows, seed=2), 1)
+
+
+@pytest.mark.parametrize("rows,B", [(257, 33), (1 << 18, 3), (262143, 65)])
+def test_largest_counts(rows, B):
+    DB = np.full((rows, 4), 0xFFFFFFFF, np.uint32)
+    Q = np.full((B, (rows + 31) // 32), 0xFFFFFFFF, np.uint32)
+    _check(rows, 128, B, DB, Q, 1)
+
+
+@pytest.mark.parametrize("bits", [511 * 32 // 128 * 128, 512 * 32, 1024 * 32])
+@pytest.mark.parametrize("B", [1, 2, 3, 8, 9, 137])
+def test_default_choice(bits, B):
+    rows = 300
+    _check(rows, bits, B, inputs.chor_db(rows, bits, seed=bits), inputs.chor_queries(B, rows, seed=B), None)
