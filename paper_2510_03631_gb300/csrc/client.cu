@@ -13,8 +13,8 @@
 // registers, and the kernel overlaps its start with the end of the kernel
 // before it (programmatic dependent launch); other n use one warp per row
 // and a shared-memory copy of the secret.
-// Batches are u32 GEMMs (Y = X * W^T over Z_{2^32}) on the CUDA cores with
-// 8x8 register blocking.
+// Batches are u32 GEMMs (Y = X * W^T over Z_{2^32}) on the CUDA cores in
+// panels of 32 rows whose warps split K.
 #include <cstdint>
 #include <mutex>
 
@@ -200,6 +200,18 @@ __global__ void __launch_bounds__(kMvThreads, 1)
 // device; read and cleared by client_status_take).
 static __device__ int g_client_status;
 
+template <int TC, class Epi>
+__global__ void u32_panel_kernel(const uint32_t *__restrict__ X, uint64_t M, const uint32_t *__restrict__ W,
+                                 uint32_t N, uint32_t K, uint32_t n_tiles, int vec, Epi epi);
+template <int TC>
+constexpr int panel_smem_bytes();
+
+template <int TC, class Epi>
+static cudaError_t set_panel_attr() {
+    return cudaFuncSetAttribute(u32_panel_kernel<TC, Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                panel_smem_bytes<TC>());
+}
+
 template <class Epi>
 static cudaError_t set_matvec_attrs() {
     cudaError_t e = cudaFuncSetAttribute(matvec_kernel<Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, 16384 * 4);
@@ -212,6 +224,11 @@ static cudaError_t set_matvec_attrs() {
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(matvec_tma_kernel<16, Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  MvCfg<16>::kSmemBytes);
+    if (e == cudaSuccess) e = set_panel_attr<1, Epi>();
+    if (e == cudaSuccess) e = set_panel_attr<2, Epi>();
+    if (e == cudaSuccess) e = set_panel_attr<4, Epi>();
+    if (e == cudaSuccess) e = set_panel_attr<6, Epi>();
+    if (e == cudaSuccess) e = set_panel_attr<8, Epi>();
     return e;
 }
 
@@ -268,69 +285,155 @@ static cudaError_t launch_matvec(const uint32_t *X, uint64_t rows, uint32_t n, c
     return cudaGetLastError();
 }
 
-// Y[i][b] = sum_k X[i][k] * W[b][k]  (mod 2^32), X: M x K, W: N x K, both
-// row-major; 128 x 128 output tile per block, 8 x 8 per thread.
-constexpr int kGT = 128, kGK = 8;
-template <class Epi>
-__global__ void __launch_bounds__(256) u32_gemm_nt_kernel(const uint32_t *__restrict__ X, uint64_t M,
-                                                          const uint32_t *__restrict__ W, uint32_t N, uint32_t K,
-                                                          Epi epi) {
-    __shared__ uint32_t xs[kGK][kGT];
-    __shared__ uint32_t ws[kGK][kGT];
-    const uint64_t i0 = (uint64_t)blockIdx.x * kGT;
-    const uint32_t b0 = blockIdx.y * kGT;
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    uint32_t acc[8][8];
-#pragma unroll
-    for (int a = 0; a < 8; ++a)
-#pragma unroll
-        for (int c = 0; c < 8; ++c) acc[a][c] = 0u;
-    // loader mapping: 256 threads x 4 elements = one 128 x 8 tile
-    const int lr = threadIdx.x / 2;            // tile row 0..127
-    const int lk = (threadIdx.x % 2) * 4;      // k offset 0 or 4
-    for (uint32_t k0 = 0; k0 < K; k0 += kGK) {
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const uint32_t k = k0 + lk + t;
-            const uint64_t i = i0 + lr;
-            const uint32_t b = b0 + lr;
-            xs[lk + t][lr] = (i < M && k < K) ? X[i * K + k] : 0u;
-            ws[lk + t][lr] = (b < N && k < K) ? W[(uint64_t)b * K + k] : 0u;
+// Y[i][b] = sum_k X[i][k] * W[b][k]  (mod 2^32), X: M x K, W: N x K, both row-major, for the
+// handle-free batch calls (a few to a few hundred vectors, no scratch).
+//
+// A CTA makes a panel of 32 rows x 4 TC vectors.  Its eight warps split K: slabs of 128 columns of
+// both operands stream through a three-stage cp.async ring and warp w takes columns 16 w .. 16 w + 15
+// of every slab, each lane a 4 x TC register block (rows lane / 4 + 8 a, vectors lane % 4 + 4 c).
+// Shared rows are 132 words apart, so the eight rows of one 16-byte read lie in distinct banks.  The
+// eight partial panels meet in shared memory once, at the end.  Short panels rather than 128 x 128
+// tiles because M is often only a few thousand and N a few dozen: 5003 rows still make 157 CTAs, and
+// a panel does no work for absent vectors beyond rounding N up to 4 TC.  Bound by HBM up to about 8
+// vectors, by the integer multiply rate above.  7001 x 630 by 24 vectors: 19 us, the same by
+// 128 x 128 tiles without a K split about 155 us (55 CTAs, five sixths of the columns absent).
+constexpr int kPanelRows = 32, kPanelK = 128, kPanelLd = kPanelK + 4, kPanelStages = 3, kPanelThreads = 256;
+constexpr int kPanelRedLd = 40;   // row stride of the partial sums: lanes (r, c) land in banks r + 8 c
+
+template <int TC>
+constexpr int panel_smem_bytes() {
+    return kPanelStages * (kPanelRows + 4 * TC) * kPanelLd * 4;
+}
+
+__device__ __forceinline__ void cp_async_zfill(uint32_t dst, const void *src, int bytes, bool valid) {
+    const int n = valid ? bytes : 0;
+    if (bytes == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
+    else if (bytes == 8)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
+}
+
+// Slab [k0, k0 + 128) of the panel's rows of X and W, VEC words per copy (K % VEC == 0 and both
+// operands VEC-word aligned); rows past the end and columns past K are zero.
+template <int TC, int VEC>
+__device__ __forceinline__ void panel_load(uint32_t *buf, const uint32_t *__restrict__ X, uint64_t M, uint64_t i0,
+                                           const uint32_t *__restrict__ W, uint32_t N, uint32_t b0, uint32_t K,
+                                           uint32_t k0) {
+    constexpr int PIECES = kPanelK / VEC, ROWS = kPanelRows + 4 * TC;
+#pragma unroll 4
+    for (int e = threadIdx.x; e < ROWS * PIECES; e += kPanelThreads) {
+        const int r = e / PIECES, c = (e % PIECES) * VEC;
+        const uint32_t k = k0 + c;
+        const bool mat = r < kPanelRows;
+        const uint64_t row = mat ? i0 + r : (uint64_t)b0 + (r - kPanelRows);
+        const bool valid = k < K && row < (mat ? M : (uint64_t)N);
+        const uint32_t *base = mat ? X : W;
+        cp_async_zfill(smem_addr(buf + r * kPanelLd + c), valid ? base + row * K + k : base, 4 * VEC, valid);
+    }
+}
+
+template <int TC, class Epi>
+__global__ void __launch_bounds__(kPanelThreads, 2)
+    u32_panel_kernel(const uint32_t *__restrict__ X, uint64_t M, const uint32_t *__restrict__ W, uint32_t N,
+                     uint32_t K, uint32_t n_tiles, int vec, Epi epi) {
+    extern __shared__ __align__(16) uint32_t panel_smem[];
+    constexpr int ROWS = kPanelRows + 4 * TC;
+    const uint64_t i0 = (uint64_t)(blockIdx.x / n_tiles) * kPanelRows;   // the panels of one row block run together
+    const uint32_t b0 = (blockIdx.x % n_tiles) * (4 * TC);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rg = lane >> 2, cg = lane & 3;
+    const uint32_t slabs = (K + kPanelK - 1) / kPanelK;
+    auto load = [&](uint32_t s) {
+        if (s < slabs) {
+            uint32_t *buf = panel_smem + (s % kPanelStages) * ROWS * kPanelLd;
+            if (vec == 4) panel_load<TC, 4>(buf, X, M, i0, W, N, b0, K, s * kPanelK);
+            else if (vec == 2) panel_load<TC, 2>(buf, X, M, i0, W, N, b0, K, s * kPanelK);
+            else panel_load<TC, 1>(buf, X, M, i0, W, N, b0, K, s * kPanelK);
         }
-        __syncthreads();
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    uint32_t acc[4][TC];
 #pragma unroll
-        for (int kk = 0; kk < kGK; ++kk) {
-            uint32_t xa[8], wb[8];
+    for (int a = 0; a < 4; ++a)
 #pragma unroll
-            for (int a = 0; a < 8; ++a) xa[a] = xs[kk][ty + 16 * a];
+        for (int c = 0; c < TC; ++c) acc[a][c] = 0u;
+    for (int s = 0; s < kPanelStages - 1; ++s) load(s);
+    for (uint32_t s = 0; s < slabs; ++s) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(kPanelStages - 2) : "memory");
+        __syncthreads();   // slab s is here, and every warp is done with the slab that load(s + 2) replaces
+        load(s + kPanelStages - 1);
+        const uint32_t *buf = panel_smem + (s % kPanelStages) * ROWS * kPanelLd + 16 * warp;
+        const uint32_t *xs = buf + rg * kPanelLd, *ws = buf + (kPanelRows + cg) * kPanelLd;
+#pragma unroll 2
+        for (int kk = 0; kk < 4; ++kk) {
+            uint4 x[4];
 #pragma unroll
-            for (int c = 0; c < 8; ++c) wb[c] = ws[kk][tx + 16 * c];
+            for (int a = 0; a < 4; ++a) x[a] = *reinterpret_cast<const uint4 *>(xs + 8 * a * kPanelLd + 4 * kk);
 #pragma unroll
-            for (int a = 0; a < 8; ++a)
+            for (int c = 0; c < TC; ++c) {
+                const uint4 w = *reinterpret_cast<const uint4 *>(ws + 4 * c * kPanelLd + 4 * kk);
 #pragma unroll
-                for (int c = 0; c < 8; ++c) acc[a][c] += xa[a] * wb[c];
+                for (int a = 0; a < 4; ++a)
+                    acc[a][c] += x[a].x * w.x + x[a].y * w.y + x[a].z * w.z + x[a].w * w.w;
+            }
         }
-        __syncthreads();
+    }
+    __syncthreads();   // the ring is done: its space takes the partial panels
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int c = 0; c < TC; ++c)
+            panel_smem[(warp * 4 * TC + cg + 4 * c) * kPanelRedLd + rg + 8 * a] = acc[a][c];
+    __syncthreads();
+    // thread (warp, lane): row i0 + lane of vectors b0 + warp, b0 + warp + 8, ...; all loads before any store
+    constexpr int OUT = (4 * TC + 7) / 8;
+    const uint64_t i = i0 + lane;
+    uint32_t pre_v[OUT];
+#pragma unroll
+    for (int o = 0; o < OUT; ++o) {
+        const uint32_t b = warp + 8 * o;
+        pre_v[o] = (b < 4 * TC && i < M && b0 + b < N) ? epi.pre(i, b0 + b) : 0u;
     }
 #pragma unroll
-    for (int a = 0; a < 8; ++a) {
-        const uint64_t i = i0 + ty + 16 * a;
-        if (i >= M) continue;
-        uint32_t pre_v[8];   // all loads of the row's outputs before any of its stores
+    for (int o = 0; o < OUT; ++o) {
+        const uint32_t b = warp + 8 * o;
+        if (b >= 4 * TC || i >= M || b0 + b >= N) continue;
+        uint32_t sum = 0;
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            const uint32_t b = b0 + tx + 16 * c;
-            pre_v[c] = b < N ? epi.pre(i, b) : 0u;
-        }
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            const uint32_t b = b0 + tx + 16 * c;
-            if (b < N) epi.put(i, b, acc[a][c], pre_v[c]);
-        }
+        for (int w = 0; w < 8; ++w) sum += panel_smem[(w * 4 * TC + b) * kPanelRedLd + lane];
+        epi.put(i, b0 + b, sum, pre_v[o]);
     }
 }
 
 // ------------------------------------------------------------------ host side
+template <int TC, class Epi>
+static cudaError_t launch_panel_t(const uint32_t *X, uint64_t M, const uint32_t *W, uint32_t N, uint32_t K, int vec,
+                                  const Epi &epi, cudaStream_t stream) {
+    const uint64_t n_tiles = ((uint64_t)N + 4 * TC - 1) / (4 * TC);
+    const uint64_t grid = (M + kPanelRows - 1) / kPanelRows * n_tiles;
+    if (grid >= (1ull << 31)) return cudaErrorInvalidValue;   // more than 2^39 outputs
+    u32_panel_kernel<TC, Epi><<<static_cast<unsigned>(grid), kPanelThreads, panel_smem_bytes<TC>(), stream>>>(
+        X, M, W, N, K, static_cast<uint32_t>(n_tiles), vec, epi);
+    return cudaGetLastError();
+}
+
+// The fewest panels of at most 32 vectors, each as narrow as covers the batch.
+template <class Epi>
+static cudaError_t launch_panel(const uint32_t *X, uint64_t M, const uint32_t *W, uint32_t N, uint32_t K,
+                                const Epi &epi, cudaStream_t stream) {
+    if (!client_status_word()) return cudaErrorUnknown;   // this device's kernel attributes
+    const uintptr_t at = reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(W);
+    const int vec = (K % 4 == 0 && at % 16 == 0) ? 4 : ((K % 2 == 0 && at % 8 == 0) ? 2 : 1);
+    const uint32_t tiles = (N - 1) / 32 + 1, per = (N - 1) / tiles + 1;
+    if (per <= 4) return launch_panel_t<1>(X, M, W, N, K, vec, epi, stream);
+    if (per <= 8) return launch_panel_t<2>(X, M, W, N, K, vec, epi, stream);
+    if (per <= 16) return launch_panel_t<4>(X, M, W, N, K, vec, epi, stream);
+    if (per <= 24) return launch_panel_t<6>(X, M, W, N, K, vec, epi, stream);
+    return launch_panel_t<8>(X, M, W, N, K, vec, epi, stream);
+}
+
 cudaError_t launch_gen_a(uint64_t seed, uint64_t C, uint32_t n, uint32_t *A, int num_sms, cudaStream_t stream) {
     gen_a_kernel<<<num_sms * 8, 256, 0, stream>>>(seed, C * n, A);
     return cudaGetLastError();
@@ -345,9 +448,7 @@ cudaError_t launch_query(const uint32_t *A, uint64_t C, uint32_t n, const uint32
 cudaError_t launch_query_batch(const uint32_t *A, uint64_t C, uint32_t n, const uint32_t *S, const int32_t *E,
                                const uint32_t *cols, uint32_t B, uint32_t delta, uint32_t *Q, cudaStream_t stream) {
     QueryEpi epi{E, C, cols, 0, delta, Q, C};
-    dim3 grid(static_cast<unsigned>((C + kGT - 1) / kGT), (B + kGT - 1) / kGT);
-    u32_gemm_nt_kernel<QueryEpi><<<grid, 256, 0, stream>>>(A, C, S, B, n, epi);
-    return cudaGetLastError();
+    return launch_panel(A, C, S, B, n, epi, stream);
 }
 
 cudaError_t launch_recover(const uint32_t *ans, const uint32_t *H, uint64_t R, uint32_t n, const uint32_t *s,
@@ -359,9 +460,7 @@ cudaError_t launch_recover(const uint32_t *ans, const uint32_t *H, uint64_t R, u
 cudaError_t launch_recover_batch(const uint32_t *ans, const uint32_t *H, uint64_t R, uint32_t n, const uint32_t *S,
                                  uint32_t B, uint32_t shift, uint8_t *out, cudaStream_t stream) {
     RecoverEpi epi{ans, R, shift, out, R};
-    dim3 grid(static_cast<unsigned>((R + kGT - 1) / kGT), (B + kGT - 1) / kGT);
-    u32_gemm_nt_kernel<RecoverEpi><<<grid, 256, 0, stream>>>(H, R, S, B, n, epi);
-    return cudaGetLastError();
+    return launch_panel(H, R, S, B, n, epi, stream);
 }
 
 cudaError_t prepare_client_kernels() { return client_status_word() ? cudaSuccess : cudaErrorUnknown; }
