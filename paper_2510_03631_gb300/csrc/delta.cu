@@ -14,15 +14,13 @@
 // Response, Recover and hint run on it unchanged.  A client that recovers
 // block j decodes it on its own by prefix sums.
 //
-//   delta_width_kernel   largest within-block difference: a warp per block,
-//                        a warp max, one atomic max per warp
-//   delta_encode_kernel  a CTA per 128 blocks x 64 differences: the entries
-//                        staged in shared memory (read run by run), the
-//                        database rows written 128 bytes at a time (four
-//                        columns per 32-bit store when aligned)
-//   delta_decode_kernel  one CTA per recovered block: per-thread runs of
-//                        differences, a CTA-wide exclusive scan of the run
-//                        totals, then each run's prefix sums
+//   delta_width_kernel   largest within-block difference: four entries per 16-byte
+//                        load over the entries in order, a CTA max, one atomic max
+//   delta_encode_kernel  a CTA per 128 blocks x 128 positions: four entries of four
+//                        blocks per thread, packed into row words in registers and
+//                        turned through shared memory into 128-byte row segments
+//   delta_decode_kernel  one CTA per recovered block: eight entries per thread,
+//                        a CTA-wide scan of their sums, 16-byte stores
 #include <cstdint>
 #include <mutex>
 
@@ -36,126 +34,231 @@ __device__ __forceinline__ uint32_t entry_at(const uint32_t *__restrict__ x, uin
     return x[k < n ? k : n - 1];
 }
 
-// One warp per block (grid-stride over blocks), lanes striding over its differences.
-__global__ void delta_width_kernel(const uint32_t *__restrict__ x, uint64_t n, uint64_t E, uint64_t C,
-                                   uint32_t *__restrict__ dmax) {
+// Largest within-block difference.  Thread t of the grid takes the four entries 4 t .. 4 t + 3, then
+// strides; its place in the block advances by a constant, so no iteration divides.  Four independent
+// 16-byte loads per thread are in flight; the entry before a thread's four comes from its neighbour
+// lane.  HBM-bound: each entry is read once.  2^26 entries: 50 us, a warp striding over one block at a
+// time 86; eight loads per thread are no faster.
+constexpr int kWidthThreads = 256;
+__global__ void __launch_bounds__(kWidthThreads) delta_width_kernel(const uint32_t *__restrict__ x, uint64_t n,
+                                                                    uint64_t E, int vec,
+                                                                    uint32_t *__restrict__ dmax) {
     const int lane = threadIdx.x & 31;
-    const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
+    const uint64_t stride = 4ull * gridDim.x * kWidthThreads;
+    const uint64_t base = 4ull * ((uint64_t)blockIdx.x * kWidthThreads + threadIdx.x);
+    const uint64_t step = stride % E;
+    uint64_t place = base % E;   // of entry k in its block
     uint32_t m = 0;
-    for (uint64_t j = (uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); j < C; j += warps)
-        for (uint64_t i = 1 + lane; i < E; i += 32) {
-            const uint32_t d = entry_at(x, n, j * E + i) - entry_at(x, n, j * E + i - 1);
-            m = d > m ? d : m;
+    constexpr int U = 4;
+    for (uint64_t k0 = base; k0 - 4ull * lane < n; k0 += U * stride) {   // warp-uniform
+        uint32_t v[U][4], before[U];
+        if (vec && k0 + 4ull * (32 - lane) + (U - 1) * stride <= n) {   // the warp's loads all in range
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const uint4 w = *reinterpret_cast<const uint4 *>(x + k0 + u * stride);
+                v[u][0] = w.x, v[u][1] = w.y, v[u][2] = w.z, v[u][3] = w.w;
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) before[u] = lane == 0 && k0 + u > 0 ? x[k0 + u * stride - 1] : 0u;
+        } else {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const uint64_t k = k0 + u * stride;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) v[u][q] = entry_at(x, n, k + q);
+                before[u] = lane == 0 && k > 0 ? entry_at(x, n, k - 1) : 0u;
+            }
         }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            uint32_t prev = __shfl_up_sync(0xffffffffu, v[u][3], 1);
+            if (lane == 0) prev = before[u];
+            uint64_t p = place;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {   // entries past n - 1 repeat it: difference 0
+                const uint32_t d = p == 0 ? 0u : v[u][q] - prev;
+                m = d > m ? d : m;
+                prev = v[u][q];
+                if (++p == E) p = 0;
+            }
+            place += step;
+            if (place >= E) place -= E;
+        }
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         const uint32_t other = __shfl_xor_sync(0xffffffffu, m, o);
         m = other > m ? other : m;
     }
-    if (lane == 0 && m) atomicMax(dmax, m);
+    __shared__ uint32_t wm[kWidthThreads / 32];
+    if (lane == 0) wm[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < kWidthThreads / 32; ++w) m = wm[w] > m ? wm[w] : m;
+        if (m) atomicMax(dmax, m);
+    }
 }
 
-// A CTA writes the rows of kEncCols consecutive blocks (columns) that hold
-// differences kEncEntries * blockIdx.y + 1 .. + kEncEntries (and the CTAs with
-// blockIdx.y == 0 also the 4 rows of the first entries).  The entries it needs
-// are read run by run (consecutive entries of one block are contiguous) into
-// shared memory, so both the reads and the row writes are coalesced.
+// A CTA writes the rows of 128 consecutive blocks (columns) that hold positions kEncPos y ..
+// kEncPos y + 127 (position 0: the four rows of the first entry).  Lane l of a warp takes positions
+// 4 l .. 4 l + 3 of four neighbouring columns: four 16-byte loads, 512 contiguous bytes a warp and
+// column.  Byte b of the four columns' differences makes one row word; the words are turned through
+// shared memory (word index xor lane: no bank conflicts either way) so that a warp writes one row's
+// 128 bytes at a time.  HBM-bound: each entry is read once, each digit written once.  2^26 entries in
+// blocks of 8192, one byte: 56 us (6.0 TB/s), 117 with the entries staged in shared memory by single
+// words; with a range check before each load instead of once per CTA, which makes every load wait for the
+// one before it, 150.
 constexpr int kEncCols = 128;     // columns per CTA: each database row segment is 128 bytes
-constexpr int kEncEntries = 64;   // differences per block per CTA
+constexpr int kEncPos = 128;      // positions per block per CTA
+constexpr uint32_t kMaxEncodeEntries = 4194241;   // longest block the encoder takes
 constexpr int kEncThreads = 256;
+constexpr int kEncQuads = kEncCols / 4 / (kEncThreads / 32);   // column quads per warp
 
 __global__ void __launch_bounds__(kEncThreads) delta_encode_kernel(const uint32_t *__restrict__ x, uint64_t n,
-                                                                   uint64_t E, uint32_t w, uint64_t C,
+                                                                   uint64_t E, uint32_t w, uint64_t C, int vec,
                                                                    uint8_t *__restrict__ db) {
-    __shared__ uint32_t ent[kEncCols][kEncEntries + 1];   // entries i0 - 1 .. i0 + kEncEntries - 1
+    __shared__ uint32_t tile[kEncPos * (kEncCols / 4)];   // word of quad c, position p at 32 p + (c ^ (p / 4))
     const uint64_t j0 = (uint64_t)blockIdx.x * kEncCols;
-    const uint64_t i0 = 1 + (uint64_t)blockIdx.y * kEncEntries;   // first difference of this CTA
-    const uint64_t ncols = C - j0 < (uint64_t)kEncCols ? C - j0 : (uint64_t)kEncCols;
-    const uint64_t i1 = i0 + kEncEntries < E ? i0 + kEncEntries : E;   // differences [i0, i1)
-    // stage entries (block j0 + c, positions i0 - 1 .. i1 - 1): consecutive threads take
-    // consecutive entries of one block's run, and each thread issues its loads independently
-    const uint32_t nt = static_cast<uint32_t>(i1 - i0) + 1;
-    const uint32_t nload = static_cast<uint32_t>(ncols) * nt;
-#pragma unroll 4
-    for (uint32_t f = threadIdx.x; f < nload; f += kEncThreads) {
-        const uint32_t c = f / nt, t = f - c * nt;
-        ent[c][t] = entry_at(x, n, (j0 + c) * E + i0 - 1 + t);
-    }
-    __syncthreads();
-    // rows of this CTA's differences: row 4 + (i - 1) w + b, column j0 + c; threads run over
-    // (row, column) with the column fastest
-    const uint32_t rows = (nt - 1) * w;   // at most 64 x 4 rows: 32-bit index math below
-    const uint64_t row0 = 4 + (i0 - 1) * w;
-    // four columns per thread in one 32-bit store when every row segment is 4-byte aligned
-    const bool quad = (C % 4 == 0) && (ncols % 4 == 0) && ((reinterpret_cast<uintptr_t>(db) & 3u) == 0);
-    if (quad) {
-        constexpr uint32_t kQuads = kEncCols / 4;
-        for (uint32_t t = threadIdx.x; t < rows * kQuads; t += kEncThreads) {
-            const uint32_t r = t / kQuads, c = 4 * (t % kQuads);
-            if (c >= ncols) continue;
-            const uint32_t di = r / w;   // difference i0 + di
-            const uint32_t sh = 8u * (r - di * w);
-            uint32_t v = 0;
+    const uint64_t p0 = (uint64_t)blockIdx.y * kEncPos;
+    const uint32_t ncols = static_cast<uint32_t>(C - j0 < (uint64_t)kEncCols ? C - j0 : (uint64_t)kEncCols);
+    const uint32_t npos = static_cast<uint32_t>(E - p0 < (uint64_t)kEncPos ? E - p0 : (uint64_t)kEncPos);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint32_t d[kEncQuads][4][4];   // entries, then differences [quad][column][position]
+    uint32_t prev[kEncQuads][4];   // lane 0: the entry before its four (none before position 0)
+    const bool inside = vec && ncols == (uint32_t)kEncCols && npos == (uint32_t)kEncPos &&
+                        (j0 + kEncCols - 1) * E + p0 + kEncPos <= n;
+    if (inside) {   // all of a thread's loads go out before the first is used
+        const uint32_t *src = x + (j0 + 4u * warp) * E + p0 + 4u * lane;
 #pragma unroll
-            for (uint32_t k = 0; k < 4; ++k)
-                v |= (((ent[c + k][di + 1] - ent[c + k][di]) >> sh) & 255u) << (8u * k);
-            *reinterpret_cast<uint32_t *>(db + (row0 + r) * C + j0 + c) = v;
-        }
+        for (int u = 0; u < kEncQuads; ++u)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const uint4 q = *reinterpret_cast<const uint4 *>(src + (32u * u + c) * E);
+                d[u][c][0] = q.x, d[u][c][1] = q.y, d[u][c][2] = q.z, d[u][c][3] = q.w;
+            }
+#pragma unroll
+        for (int u = 0; u < kEncQuads; ++u)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) prev[u][c] = lane == 0 && p0 > 0 ? *(src + (32u * u + c) * E - 1) : 0u;
     } else {
-        for (uint32_t t = threadIdx.x; t < rows * kEncCols; t += kEncThreads) {
-            const uint32_t r = t / kEncCols, c = t % kEncCols;
-            if (c >= ncols) continue;
-            const uint32_t di = r / w;   // difference i0 + di
-            const uint32_t b = r - di * w;
-            const uint32_t d = ent[c][di + 1] - ent[c][di];
-            db[(row0 + r) * C + j0 + c] = static_cast<uint8_t>(d >> (8u * b));
-        }
+#pragma unroll
+        for (int u = 0; u < kEncQuads; ++u)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const uint32_t col = 4u * (warp + 8 * u) + c;
+                const uint64_t k = (j0 + col) * E + p0 + 4u * lane;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) d[u][c][q] = col < ncols ? entry_at(x, n, k + q) : 0u;
+                prev[u][c] = col < ncols && lane == 0 && p0 > 0 ? entry_at(x, n, k - 1) : 0u;
+            }
     }
-    if (blockIdx.y == 0) {   // the first entry of each block in full
-        for (uint64_t t = threadIdx.x; t < 4 * (uint64_t)kEncCols; t += kEncThreads) {
-            const uint64_t r = t / kEncCols, c = t % kEncCols;
-            if (c < ncols) db[r * C + j0 + c] = static_cast<uint8_t>(ent[c][0] >> (8u * r));
+#pragma unroll
+    for (int u = 0; u < kEncQuads; ++u)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const uint32_t up = __shfl_up_sync(0xffffffffu, d[u][c][3], 1);
+            d[u][c][3] -= d[u][c][2];
+            d[u][c][2] -= d[u][c][1];
+            d[u][c][1] -= d[u][c][0];
+            d[u][c][0] -= lane > 0 ? up : prev[u][c];   // position 0: the entry itself
         }
+    const bool words = (C % 4 == 0) && ((reinterpret_cast<uintptr_t>(db) & 3u) == 0);
+    const uint32_t quad_cols = ncols - (4u * lane < ncols ? 4u * lane : ncols);   // columns of this lane's row word
+    for (uint32_t b = 0; b < 4; ++b) {
+        if (b >= w && p0 != 0) break;   // bytes past w: only the first entries' rows
+        const uint32_t lo = b | ((b + 4) << 4);   // byte b of each of two words
+#pragma unroll
+        for (int u = 0; u < kEncQuads; ++u)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const uint32_t a = __byte_perm(d[u][0][q], d[u][1][q], lo), c = __byte_perm(d[u][2][q], d[u][3][q], lo);
+                tile[(4 * lane + q) * 32 + ((warp + 8 * u) ^ lane)] = __byte_perm(a, c, 0x5410);
+            }
+        __syncthreads();
+        const uint32_t last = b < w ? npos : 1u;
+        for (uint32_t p = warp; p < last; p += kEncThreads / 32) {
+            const uint32_t v = tile[p * 32 + (lane ^ (p >> 2))];
+            const uint64_t pos = p0 + p;
+            const uint64_t row = pos == 0 ? b : 4 + (pos - 1) * w + b;
+            uint8_t *dst = db + row * C + j0 + 4u * lane;
+            if (words) {
+                if (quad_cols) *reinterpret_cast<uint32_t *>(dst) = v;   // C % 4 == 0: whole words
+            } else {
+#pragma unroll
+                for (uint32_t c = 0; c < 4; ++c)
+                    if (c < quad_cols) dst[c] = static_cast<uint8_t>(v >> (8 * c));
+            }
+        }
+        __syncthreads();
     }
 }
 
-constexpr int kDecodeThreads = 256;
+// Block b: digits b * Rp .. (4-byte first entry, then E - 1 differences of W bytes) -> out b * E ..
+// Thread t takes positions 8 t .. 8 t + 7 of a run of 8192 (its digits are independent loads of
+// adjacent bytes), a two-level shuffle scan gives the sum before them, and the runs of a longer
+// block follow one another with the last sum carried.  64 blocks of 8192: 4.2 us, 12.1 with each thread
+// adding up a run of 32 bytes of its own.
+constexpr int kDecodeThreads = 1024;
+constexpr int kDecodeRun = 8;
 
-// Block b: digits b * Rp .. (4-byte first entry, then E - 1 differences of w bytes) -> out b * E ..
+template <int W>
 __global__ void __launch_bounds__(kDecodeThreads) delta_decode_kernel(const uint8_t *__restrict__ digits, uint64_t E,
-                                                                      uint32_t w, uint64_t Rp,
+                                                                      uint64_t Rp, int vec,
                                                                       uint32_t *__restrict__ out) {
-    __shared__ uint32_t part[kDecodeThreads];
+    __shared__ uint32_t part[2][kDecodeThreads / 32];
     const uint8_t *dg = digits + (uint64_t)blockIdx.x * Rp;
     uint32_t *o = out + (uint64_t)blockIdx.x * E;
-    const uint64_t nd = E - 1;                                       // differences in the block
-    const uint64_t run = (nd + kDecodeThreads - 1) / kDecodeThreads;  // differences per thread
-    const uint64_t i0 = (uint64_t)threadIdx.x * run;
-    const uint64_t i1 = i0 + run < nd ? i0 + run : nd;
-    auto diff = [&](uint64_t i) {   // difference i (0-based) of the block
-        const uint8_t *p = dg + 4 + i * w;
-        uint32_t d = 0;
-        for (uint32_t b = 0; b < w; ++b) d |= static_cast<uint32_t>(p[b]) << (8u * b);
-        return d;
-    };
-    uint32_t sum = 0;
-    for (uint64_t i = i0; i < i1; ++i) sum += diff(i);
-    part[threadIdx.x] = sum;
-    __syncthreads();
-    // inclusive scan of the run totals (Hillis-Steele over 256 values)
-    for (int off = 1; off < kDecodeThreads; off <<= 1) {
-        const uint32_t add = threadIdx.x >= static_cast<unsigned>(off) ? part[threadIdx.x - off] : 0u;
-        __syncthreads();
-        part[threadIdx.x] += add;
-        __syncthreads();
-    }
-    const uint32_t first = static_cast<uint32_t>(dg[0]) | (static_cast<uint32_t>(dg[1]) << 8) |
-                           (static_cast<uint32_t>(dg[2]) << 16) | (static_cast<uint32_t>(dg[3]) << 24);
-    uint32_t v = first + (threadIdx.x ? part[threadIdx.x - 1] : 0u);
-    if (threadIdx.x == 0) o[0] = first;
-    for (uint64_t i = i0; i < i1; ++i) {
-        v += diff(i);
-        o[i + 1] = v;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint32_t carry = 0;
+    int turn = 0;
+    for (uint64_t e0 = 0; e0 < E; e0 += kDecodeThreads * kDecodeRun, turn ^= 1) {
+        const uint64_t t0 = e0 + (uint64_t)threadIdx.x * kDecodeRun;
+        uint32_t v[kDecodeRun];
+#pragma unroll
+        for (int i = 0; i < kDecodeRun; ++i) {
+            const uint64_t t = t0 + i;
+            v[i] = 0u;
+            if (t < E) {
+                if (t == 0) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) v[i] |= static_cast<uint32_t>(dg[k]) << (8 * k);
+                } else {
+                    const uint8_t *p = dg + 4 + (t - 1) * W;
+#pragma unroll
+                    for (int k = 0; k < W; ++k) v[i] |= static_cast<uint32_t>(p[k]) << (8 * k);
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 1; i < kDecodeRun; ++i) v[i] += v[i - 1];
+        uint32_t sum = v[kDecodeRun - 1];   // inclusive over the warp, then over the CTA
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const uint32_t a = __shfl_up_sync(0xffffffffu, sum, off);
+            if (lane >= off) sum += a;
+        }
+        if (lane == 31) part[turn][warp] = sum;
+        __syncthreads();   // the other buffer's readers are done before this one is written again
+        uint32_t ps = part[turn][lane];
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const uint32_t a = __shfl_up_sync(0xffffffffu, ps, off);
+            if (lane >= off) ps += a;
+        }
+        const uint32_t total = __shfl_sync(0xffffffffu, ps, 31);
+        const uint32_t warps_before = __shfl_sync(0xffffffffu, ps, (warp + 31) & 31);   // unused in warp 0
+        const uint32_t before = carry + (warp ? warps_before : 0u) + sum - v[kDecodeRun - 1];
+        carry += total;
+        if (vec && t0 + kDecodeRun <= E) {
+#pragma unroll
+            for (int i = 0; i < kDecodeRun; i += 4)
+                *reinterpret_cast<uint4 *>(o + t0 + i) =
+                    make_uint4(before + v[i], before + v[i + 1], before + v[i + 2], before + v[i + 3]);
+        } else {
+#pragma unroll
+            for (int i = 0; i < kDecodeRun; ++i)
+                if (t0 + i < E) o[t0 + i] = before + v[i];
+        }
     }
 }
 
@@ -188,14 +291,16 @@ int qpadl_pir_delta_width(const uint32_t *entries_dev, uint64_t n, uint32_t E, u
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const int sms = num_sms_current();
     if (sms <= 0) return QPADL_ECUDA;
-    const uint64_t C = (n + E - 1) / E;
+    const int vec = (reinterpret_cast<uintptr_t>(entries_dev) & 15u) == 0;
+    const uint64_t want = (n + 16 * kWidthThreads - 1) / (16 * kWidthThreads);   // 16 entries per thread and pass
+    const unsigned grid = static_cast<unsigned>(want < (uint64_t)sms * 4 ? want : (uint64_t)sms * 4);
     std::lock_guard<std::mutex> guard(g_width_mu);
     uint32_t *dmax = nullptr;
     if (cudaGetSymbolAddress(reinterpret_cast<void **>(&dmax), g_width_word) != cudaSuccess) return QPADL_ECUDA;
     uint32_t h = 0;
     bool ok = cudaMemsetAsync(dmax, 0, sizeof(uint32_t), s) == cudaSuccess;
     if (ok) {
-        delta_width_kernel<<<sms * 8, 256, 0, s>>>(entries_dev, n, E, C, dmax);
+        delta_width_kernel<<<grid, kWidthThreads, 0, s>>>(entries_dev, n, E, vec, dmax);
         ok = cudaGetLastError() == cudaSuccess;
     }
     ok = ok && cudaMemcpyAsync(&h, dmax, sizeof(uint32_t), cudaMemcpyDeviceToHost, s) == cudaSuccess;
@@ -210,14 +315,12 @@ int qpadl_pir_delta_width(const uint32_t *entries_dev, uint64_t n, uint32_t E, u
 int qpadl_pir_delta_encode(const uint32_t *entries_dev, uint64_t n, uint32_t E, uint32_t w, uint8_t *db_dev,
                            qpadl_stream_t stream) {
     if (!entries_dev || !db_dev || !delta_shape_ok(n, E, w)) return QPADL_EINVAL;
-    const int sms = num_sms_current();
-    if (sms <= 0) return QPADL_ECUDA;
-    (void)sms;
     const uint64_t C = (n + E - 1) / E;
-    const uint64_t ytiles = E > 1 ? (E - 1 + kEncEntries - 1) / kEncEntries : 1;
-    if (ytiles > 65535) return QPADL_EINVAL;   // blocks of more than 4 million entries
-    const dim3 grid(static_cast<unsigned>((C + kEncCols - 1) / kEncCols), static_cast<unsigned>(ytiles));
-    delta_encode_kernel<<<grid, kEncThreads, 0, reinterpret_cast<cudaStream_t>(stream)>>>(entries_dev, n, E, w, C,
+    if (E > kMaxEncodeEntries) return QPADL_EINVAL;
+    const int vec = (E % 4 == 0) && (reinterpret_cast<uintptr_t>(entries_dev) & 15u) == 0;
+    const dim3 grid(static_cast<unsigned>((C + kEncCols - 1) / kEncCols),
+                    static_cast<unsigned>((E + kEncPos - 1) / kEncPos));
+    delta_encode_kernel<<<grid, kEncThreads, 0, reinterpret_cast<cudaStream_t>(stream)>>>(entries_dev, n, E, w, C, vec,
                                                                                           db_dev);
     return cudaGetLastError() == cudaSuccess ? QPADL_OK : QPADL_ECUDA;
 }
@@ -226,8 +329,10 @@ int qpadl_pir_delta_decode(const uint8_t *digits_dev, uint32_t B, uint32_t E, ui
                            qpadl_stream_t stream) {
     if (!digits_dev || !entries_dev || B == 0 || !delta_shape_ok(E, E, w)) return QPADL_EINVAL;
     const uint64_t Rp = 4 + (uint64_t)w * (E - 1);
-    delta_decode_kernel<<<B, kDecodeThreads, 0, reinterpret_cast<cudaStream_t>(stream)>>>(digits_dev, E, w, Rp,
-                                                                                          entries_dev);
+    const int vec = (E % 4 == 0) && (reinterpret_cast<uintptr_t>(entries_dev) & 15u) == 0;
+    const auto kernel = w == 1 ? delta_decode_kernel<1>
+                               : (w == 2 ? delta_decode_kernel<2> : (w == 3 ? delta_decode_kernel<3> : delta_decode_kernel<4>));
+    kernel<<<B, kDecodeThreads, 0, reinterpret_cast<cudaStream_t>(stream)>>>(digits_dev, E, Rp, vec, entries_dev);
     return cudaGetLastError() == cudaSuccess ? QPADL_OK : QPADL_ECUDA;
 }
 
