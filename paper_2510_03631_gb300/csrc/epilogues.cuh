@@ -131,6 +131,11 @@ struct ModPEpi {
     __device__ __forceinline__ void store(uint64_t i, uint32_t b, uint32_t r) const {
         out[i * ld_m + (uint64_t)b * ld_b] = r;
     }
+    // the residue of one CTA's part of the element (split tiles; the output starts at zero and is
+    // reduced mod p afterwards)
+    __device__ __forceinline__ void add(uint64_t i, uint32_t b, uint32_t r) const {
+        atomicAdd(out + i * ld_m + (uint64_t)b * ld_b, r);
+    }
     __device__ __forceinline__ void operator()(uint64_t i, uint32_t b, uint32_t dot) const { put(i, b, dot, 0u); }
 };
 

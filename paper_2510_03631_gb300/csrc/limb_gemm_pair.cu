@@ -49,18 +49,20 @@
 //
 // Schedule.  Whole pair tiles go round-robin to the clusters.  A plain store may split its last
 // wave stream-K style (PairPieceIter: clusters grouped by vector tile so the clusters on one row
-// tile read its rows together), the split pieces adding into a zeroed output.
+// tile read its rows together), the split pieces adding into a zeroed output.  A Z_p store may cut
+// every tile into chunk ranges whose residues add up, reduced mod p by one more pass.
 //
 // One-row mode (ModPEpi: Z_p vectors as single centred fp16 rows, 256-wide tiles).  The running
 // sums stay in TMEM: after every 512-deep chunk the epilogue replaces its accumulator buffer by
 // small representatives of the sums mod p, and the MMA accumulates the chunk after next on top;
-// the last two buffers are combined mod p at the end of the tile.
+// the last two buffers are combined mod p at the end of the tile (of the piece, when it is split).
 #include <cstdint>
 #include <type_traits>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include "epilogues.cuh"
+#include "limb_gemm.cuh"
 #include "limb_gemm_pair.cuh"
 #include "ptx.cuh"
 
@@ -102,16 +104,22 @@ __device__ __forceinline__ bool drain_wait_p(uint64_t *bar, uint32_t parity) {
 // split by chunks (stream-K), so the last wave ends evenly: the first tail_parts * n_tiles
 // clusters form n_tiles groups, group n takes vector tile n of every tail row tile, and cluster p
 // of each group takes the same contiguous share of the (row tile, chunk) units, so the n_tiles
-// clusters that read one row tile's rows still read them together.
+// that read one row tile's rows still read them together.
+//
+// With ksplit > 1 every tile is cut into ksplit chunk ranges instead, dealt round-robin range by
+// range (unit i: range i / tiles of tile i % tiles), so the clusters that run together read the
+// same columns of the vector operand.
 struct PairPiece {
     uint32_t t, c0, c1;
 };
 struct PairPieceIter {
-    uint32_t t, step, n, u, u_end;
-    __device__ __forceinline__ PairPieceIter(uint32_t tiles, uint32_t dp_tiles, uint32_t n_tiles, uint32_t nchunks,
-                                             uint32_t tail_parts, uint32_t part, uint32_t nparts) {
+    uint32_t t, step, n, u, u_end, tiles, ksplit;
+    __device__ __forceinline__ PairPieceIter(uint32_t tiles_, uint32_t dp_tiles, uint32_t n_tiles, uint32_t nchunks,
+                                             uint32_t tail_parts, uint32_t ksplit_, uint32_t part, uint32_t nparts) {
         t = part;
         step = nparts;
+        tiles = tiles_;
+        ksplit = ksplit_;
         n = part % n_tiles;
         u = u_end = 0;
         const uint32_t p = part / n_tiles;
@@ -122,6 +130,14 @@ struct PairPieceIter {
         }
     }
     __device__ __forceinline__ bool next(PairPiece &pc, uint32_t dp_tiles, uint32_t n_tiles, uint32_t nchunks) {
+        if (ksplit > 1) {
+            const uint32_t s = t / tiles;
+            if (s >= ksplit) return false;
+            pc = PairPiece{t % tiles, static_cast<uint32_t>((uint64_t)s * nchunks / ksplit),
+                           static_cast<uint32_t>((uint64_t)(s + 1) * nchunks / ksplit)};
+            t += step;
+            return true;
+        }
         if (t < dp_tiles) {
             pc = PairPiece{t, 0u, nchunks};
             t += step;
@@ -142,7 +158,8 @@ template <int BN, class Epi, bool PLANED>
 __global__ void __launch_bounds__(kPThreads, 1)
     limb_gemm_pair_kernel(const __grid_constant__ CUtensorMap a_map, const __grid_constant__ PairBMaps bm, Epi epi,
                           uint32_t M, uint32_t NV, uint32_t KB, uint32_t ckb, uint32_t plane_chunks,
-                          uint32_t dp_tiles_arg, uint32_t tail_parts, int *__restrict__ status) {
+                          uint32_t dp_tiles_arg, uint32_t tail_parts, uint32_t ksplit,
+                          int *__restrict__ status) {
     using Cfg = PairCfg<BN>;
     static_assert(BN == 64 || BN == 128 || BN == 256, "tile width");
     static_assert(!PLANED || BN >= 128, "a planed shift group needs N/2 >= 16 rows per CTA");
@@ -201,10 +218,12 @@ __global__ void __launch_bounds__(kPThreads, 1)
     const uint32_t tiles = m_tiles * n_tiles;
     const uint32_t cluster = blockIdx.x >> 1, nclusters = gridDim.x >> 1;   // clusters are CTAs 2c, 2c + 1
     const uint32_t nchunks = (KB + ckb - 1) / ckb;
-    // only a plain store takes split tiles (their pieces add into a zeroed output)
-    constexpr bool kSplit = std::is_same<Epi, StoreEpi>::value;
+    // split tiles: the pieces of a plain store, or the residues of a Z_p tile's pieces, add into a
+    // zeroed output
+    constexpr bool kSplit = std::is_same<Epi, StoreEpi>::value || std::is_same<Epi, ModPEpi>::value;
     const uint32_t dp_tiles = kSplit && dp_tiles_arg < tiles ? dp_tiles_arg : tiles;
     const uint32_t tparts = dp_tiles < tiles ? tail_parts : 0u;
+    const uint32_t ks = kSplit ? ksplit : 1u;
     bool failed = false;
     auto fail_both = [&]() {
         failed = true;
@@ -225,7 +244,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
             }
             const uint32_t kpp = PLANED ? ckb * plane_chunks : KB;   // k-steps per limb plane
             uint32_t it = 0, st = 0, ph = 0;
-            PairPieceIter pit(tiles, dp_tiles, n_tiles, nchunks, tparts, cluster, nclusters);
+            PairPieceIter pit(tiles, dp_tiles, n_tiles, nchunks, tparts, ks, cluster, nclusters);
             PairPiece pc;
             while (!failed && pit.next(pc, dp_tiles, n_tiles, nchunks)) {
                 const uint32_t t = pc.t;
@@ -277,7 +296,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
             uint32_t ci = 0, st = 0, ph = 0;
             const uint32_t kpp = PLANED ? ckb * plane_chunks : KB;
             bool issued = false;
-            PairPieceIter pit(tiles, dp_tiles, n_tiles, nchunks, tparts, cluster, nclusters);
+            PairPieceIter pit(tiles, dp_tiles, n_tiles, nchunks, tparts, ks, cluster, nclusters);
             PairPiece pc;
             while (!failed && pit.next(pc, dp_tiles, n_tiles, nchunks)) {
                 const uint32_t kb0 = pc.c0 * ckb, kb1 = pc.c1 * ckb < KB ? pc.c1 * ckb : KB;
@@ -309,7 +328,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
 #pragma unroll
                         for (int k = 0; k < kPK / 16; ++k)
                             umma_f16_pair(d_tmem, adesc + 2u * k, bdesc + 2u * k, idesc,
-                                          (kc != 0 || k != 0 || (TMEMSUM && kb >= 2u * ckb)) ? 1u : 0u);
+                                          (kc != 0 || k != 0 || (TMEMSUM && kb >= kb0 + 2u * ckb)) ? 1u : 0u);
                         umma_commit_pair(&empty[st], 3);
                         if (last_of_chunk) umma_commit_pair(&acc_full[ci & 1u], 3);
                     }
@@ -339,12 +358,13 @@ __global__ void __launch_bounds__(kPThreads, 1)
         const uint32_t quarter = static_cast<uint32_t>(warp & 3);
         const uint32_t lane_addr = (quarter * 32u) << 16;
         uint32_t ci = 0;
-        PairPieceIter pit(tiles, dp_tiles, n_tiles, nchunks, tparts, cluster, nclusters);
+        PairPieceIter pit(tiles, dp_tiles, n_tiles, nchunks, tparts, ks, cluster, nclusters);
         PairPiece pc;
         while (!failed && pit.next(pc, dp_tiles, n_tiles, nchunks)) {
             const uint32_t t = pc.t;
             const uint32_t row = (t / n_tiles) * 2 * kPM + rank * kPM + quarter * 32u + static_cast<uint32_t>(lane);
             const uint32_t v0 = (t % n_tiles) * QPT;
+            const bool whole = pc.c0 == 0 && pc.c1 == nchunks;   // no other cluster works on this tile
             constexpr int RUN = TMEMSUM ? 1 : QPT;   // running sums kept in registers
             uint32_t run[RUN];
 #pragma unroll
@@ -367,7 +387,8 @@ __global__ void __launch_bounds__(kPThreads, 1)
                 const uint32_t acc = tmem_base + lane_addr + buf * BN;
                 if constexpr (TMEMSUM) {
                     const float pf = static_cast<float>(epi.p), inv = 1.0f / pf;
-                    if (c + 1 < nchunks) {
+                    const bool two = pc.c1 - pc.c0 >= 2;   // the piece used both buffers
+                    if (c + 1 < pc.c1) {
                         // replace this buffer's running sums by small representatives of their
                         // residues mod p: q = x / p rounded to an integer through the 1.5 * 2^23
                         // rounding constant, r = x - q p with |r| <= 1.5 p; q p and r are integers
@@ -392,7 +413,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
                             }
                         }
                         tmem_wait_st();
-                        if (c + 2 < nchunks) {
+                        if (c + 2 < pc.c1) {
                             tc_fence_before();
                             __syncwarp();
                             if (lane == 0) mbar_arrive_cluster(acc_empty_c + 8u * buf);
@@ -410,13 +431,13 @@ __global__ void __launch_bounds__(kPThreads, 1)
                     for (int j = 0; j < BN / 32; ++j) {
                         uint32_t v[32], w[32];
                         tmem_ld32(acc + 32u * j, v);
-                        if (nchunks >= 2) tmem_ld32(oth + 32u * j, w);
+                        if (two) tmem_ld32(oth + 32u * j, w);
                         tmem_wait_ld();
 #pragma unroll
                         for (int q = 0; q < 32; ++q) {
                             float x = __uint_as_float(v[q]);
                             x = __fmaf_rn(-__fsub_rn(__fmaf_rn(x, inv, kRound), kRound), pf, x);
-                            if (nchunks >= 2) {
+                            if (two) {
                                 float y = __uint_as_float(w[q]);
                                 y = __fmaf_rn(-__fsub_rn(__fmaf_rn(y, inv, kRound), kRound), pf, y);
                                 x = __fadd_rn(x, y);
@@ -425,14 +446,17 @@ __global__ void __launch_bounds__(kPThreads, 1)
                             if (r < 0.0f) r = __fadd_rn(r, pf);
                             if (r >= pf) r = __fsub_rn(r, pf);
                             const uint32_t vi = v0 + 32u * j + q;
-                            if (row < M && vi < NV) epi.store(row, vi, static_cast<uint32_t>(r));
+                            if (row < M && vi < NV) {
+                                if (whole) epi.store(row, vi, static_cast<uint32_t>(r));
+                                else epi.add(row, vi, static_cast<uint32_t>(r));
+                            }
                         }
                     }
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) {
                         mbar_arrive_cluster(acc_empty_c + 8u * buf);
-                        if (nchunks >= 2) mbar_arrive_cluster(acc_empty_c + 8u * (buf ^ 1u));
+                        if (two) mbar_arrive_cluster(acc_empty_c + 8u * (buf ^ 1u));
                     }
                     continue;
                 } else if constexpr (PLANED) {
@@ -493,7 +517,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
             if (failed) break;
             if constexpr (TMEMSUM) continue;   // the last chunk already wrote the tile
             if constexpr (kSplit) {
-                if (row < M && !(pc.c0 == 0 && pc.c1 == nchunks)) {
+                if (row < M && !whole) {
                     // part of a split tile: exact, since addition mod 2^32 commutes
 #pragma unroll
                     for (int q = 0; q < QPT; ++q)
@@ -648,6 +672,28 @@ static bool pair_split_schedule(uint64_t tiles, uint64_t n_tiles, uint32_t nchun
     return true;
 }
 
+// Chunk ranges per tile of a Z_p launch: the fewest that bring its tiles (or ranges) within 2% of the
+// best fill of whole waves on `pairs` clusters, when that saves at least 8%.  A tile of such a
+// launch does a quarter of a 4-limb tile's work per byte of D and reads the vector rows (134 MB at
+// 1024 x 65536, more than L2 holds beside D) once per row tile, so all clusters must stay on the same
+// columns: stream-K shares, which spread the clusters over all of K, read them from DRAM for every row
+// tile.  3072 rows, 1024 vectors of 65536 entries, 48 tiles on 76 pairs: whole tiles 290 us, stream-K
+// shares 331, three ranges 250 (and 12 for zeroing and the last mod p).
+static uint32_t field_ksplit(uint64_t tiles, uint32_t nchunks, uint64_t pairs) {
+    if (pairs == 0) return 1;
+    auto fill = [&](uint64_t s) {
+        const uint64_t waves = (tiles * s + pairs - 1) / pairs;
+        return static_cast<double>(tiles * s) / static_cast<double>(waves * pairs);
+    };
+    const uint32_t most = nchunks / 4 < 8 ? nchunks / 4 : 8;   // ranges of at least four chunks
+    double best = fill(1);
+    for (uint32_t s = 2; s <= most; ++s) best = fill(s) > best ? fill(s) : best;
+    if (fill(1) > 0.92 * best) return 1;
+    for (uint32_t s = 2; s <= most; ++s)
+        if (fill(s) >= 0.98 * best) return s;
+    return 1;
+}
+
 template <int BN, class Epi, bool PLANED>
 static cudaError_t launch_pair_t(const CUtensorMap &a_map, const PairBMaps &bm, const Epi &epi, uint32_t M,
                                  uint32_t NV, uint32_t KB, uint32_t ckb, uint32_t plane_chunks, int num_sms,
@@ -659,9 +705,10 @@ static cudaError_t launch_pair_t(const CUtensorMap &a_map, const PairBMaps &bm, 
     const uint64_t pairs = static_cast<uint64_t>(resident_pairs<BN, Epi, PLANED>(num_sms));
     uint64_t clusters = tiles < pairs ? tiles : pairs;
     uint32_t dp = 0xffffffffu, tail_parts = 0;
+    uint32_t ksplit = 1;
+    // split tiles add into the output, so it is zeroed first; only a dense output (every
+    // element of the M x NV block, in either order) can be zeroed in one piece
     if constexpr (std::is_same<Epi, StoreEpi>::value) {
-        // split tiles add into the output, so it is zeroed first; only a dense output (every
-        // element of the M x NV block, in either order) can be zeroed in one piece
         const bool dense = (epi.ld_m == 1 && epi.ld_b == M) || (epi.ld_b == 1 && epi.ld_m == NV);
         uint64_t c2 = clusters;
         uint32_t dp2 = 0, tp2 = 0;
@@ -673,11 +720,25 @@ static cudaError_t launch_pair_t(const CUtensorMap &a_map, const PairBMaps &bm, 
             tail_parts = tp2;
         }
     }
+    if constexpr (std::is_same<Epi, ModPEpi>::value) {
+        if (epi.ld_m == 1 && epi.ld_b == M) ksplit = field_ksplit(tiles, (KB + ckb - 1) / ckb, pairs);
+        if (ksplit > 1) {
+            const cudaError_t e = cudaMemsetAsync(epi.out, 0, 4ull * M * NV, stream);
+            if (e != cudaSuccess) return e;
+            clusters = tiles * ksplit < pairs ? tiles * ksplit : pairs;
+        }
+    }
     if (clusters == 0) return cudaSuccess;
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = pair_config<BN>(static_cast<unsigned>(clusters), stream, attr);
-    return cudaLaunchKernelEx(&cfg, limb_gemm_pair_kernel<BN, Epi, PLANED>, a_map, bm, epi, M, NV, KB, ckb,
-                              plane_chunks, dp, tail_parts, status);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, limb_gemm_pair_kernel<BN, Epi, PLANED>, a_map, bm, epi, M, NV, KB,
+                                             ckb, plane_chunks, dp, tail_parts, ksplit, status);
+    if constexpr (std::is_same<Epi, ModPEpi>::value) {
+        // the residues of a tile's ranges were added up (at most 8 * 256): now mod p
+        if (ksplit > 1 && e == cudaSuccess)
+            return launch_mod_p(epi.out, (uint64_t)M * NV, static_cast<uint32_t>(epi.p), num_sms, stream);
+    }
+    return e;
 }
 
 template <class Epi>

@@ -131,3 +131,16 @@ def test_full_size_sampled_rows(cuda, B):
     exp = oracle.goldberg_answer(np.ascontiguousarray(D[rows]), Q, p, threads=oracle.max_threads())
     assert np.array_equal(got[:, rows], exp)
     h.close()
+
+
+# 256-wide pair tiles split between clusters: pieces of one, two and more 512-deep chunks, a ragged
+# last chunk, several vector tiles
+@pytest.mark.parametrize("R,C,p,B", [(300, 5000, 257, 130), (2500, 3000, 251, 600), (3072, 2561, 31, 513),
+                                     (520, 60000, 257, 300)])
+def test_split_tiles_match_oracle(cuda, R, C, p, B):
+    D = _db(R, C, p, seed=R + B)
+    Q = (inputs.uniform_u32(B * C, seed=B + p, tag=inputs.TAG_MISC) % p).reshape(B, C)
+    h = pir.qpadl_goldberg_setup(R, C, p, torch.from_numpy(D).cuda())
+    got = _answer(h, Q, 1, 0)
+    assert np.array_equal(got, oracle.goldberg_answer(D, Q, p, threads=oracle.max_threads()))
+    h.close()
