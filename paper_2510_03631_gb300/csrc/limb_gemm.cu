@@ -497,7 +497,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
 // D (uint8, R x C) -> D16 (fp16, R x pitch), digits as exact small integers.
 // One block per row at a time; 16 digits per thread step when rows are aligned.
 __global__ void db_to_f16_kernel(const uint8_t *__restrict__ D, uint64_t R, uint64_t C, __half *__restrict__ D16,
-                                 uint64_t pitch) {
+                                 uint64_t pitch, int centre) {
     const bool vec = (C % 16 == 0) && ((reinterpret_cast<uintptr_t>(D) & 15u) == 0) && (pitch % 8 == 0);
     for (uint64_t i = blockIdx.x; i < R; i += gridDim.x) {
         const uint8_t *src = D + i * C;
@@ -509,8 +509,9 @@ __global__ void db_to_f16_kernel(const uint8_t *__restrict__ D, uint64_t R, uint
                 uint32_t h[8];
 #pragma unroll
                 for (int t = 0; t < 4; ++t) {
-                    const __half2 lo = __halves2half2(__ushort2half_rn(ws[t] & 255u), __ushort2half_rn((ws[t] >> 8) & 255u));
-                    const __half2 hi = __halves2half2(__ushort2half_rn((ws[t] >> 16) & 255u), __ushort2half_rn(ws[t] >> 24));
+                    auto digit = [&](int k) { return __int2half_rn(static_cast<int>((ws[t] >> (8 * k)) & 255u) - centre); };
+                    const __half2 lo = __halves2half2(digit(0), digit(1));
+                    const __half2 hi = __halves2half2(digit(2), digit(3));
                     h[2 * t] = *reinterpret_cast<const uint32_t *>(&lo);
                     h[2 * t + 1] = *reinterpret_cast<const uint32_t *>(&hi);
                 }
@@ -520,7 +521,7 @@ __global__ void db_to_f16_kernel(const uint8_t *__restrict__ D, uint64_t R, uint
             }
         } else {
             for (uint64_t j = threadIdx.x; j < C; j += blockDim.x)
-                dst[j] = __ushort2half_rn(static_cast<unsigned short>(src[j]));
+                dst[j] = __int2half_rn(static_cast<int>(src[j]) - centre);
         }
     }
 }
@@ -817,7 +818,7 @@ static cudaError_t launch_epi(int bn, const CUtensorMap &a_map, const CUtensorMa
 cudaError_t launch_limb_gemm(int bn, const CUtensorMap &a_map, const CUtensorMap &b_map, uint32_t *out,
                              uint64_t ld_m, uint64_t ld_b, uint32_t M, uint32_t NV, uint64_t K, int num_sms,
                              int *status, cudaStream_t stream) {
-    return launch_epi(bn, a_map, b_map, StoreEpi{out, ld_m, ld_b}, M, NV, K, 0, num_sms, status, stream);
+    return launch_epi(bn, a_map, b_map, StoreEpi{out, ld_m, ld_b, nullptr, 0u}, M, NV, K, 0, num_sms, status, stream);
 }
 
 cudaError_t launch_limb_gemm_query(int bn, const CUtensorMap &a_map, const CUtensorMap &b_map, const QueryNoiseEpi &epi,
@@ -850,10 +851,10 @@ cudaError_t launch_limb_gemm_modp(int bn, const CUtensorMap &a_map, const CUtens
     return launch_epi(bn, a_map, b_map, epi, M, NV, K, 0, num_sms, status, stream);
 }
 
-cudaError_t launch_db_to_f16(const uint8_t *D, uint64_t R, uint64_t C, __half *D16, uint64_t pitch, int num_sms,
-                             cudaStream_t stream) {
+cudaError_t launch_db_to_f16(const uint8_t *D, uint64_t R, uint64_t C, __half *D16, uint64_t pitch, int centre,
+                             int num_sms, cudaStream_t stream) {
     const uint64_t blocks = R < (uint64_t)num_sms * 8 ? R : (uint64_t)num_sms * 8;
-    db_to_f16_kernel<<<static_cast<unsigned>(blocks), 256, 0, stream>>>(D, R, C, D16, pitch);
+    db_to_f16_kernel<<<static_cast<unsigned>(blocks), 256, 0, stream>>>(D, R, C, D16, pitch, centre);
     return cudaGetLastError();
 }
 

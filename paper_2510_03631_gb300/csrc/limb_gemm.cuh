@@ -50,8 +50,9 @@ cudaError_t launch_mod_p(uint32_t *x, uint64_t n, uint32_t p, int num_sms, cudaS
 // x[i] = (x[i] as a signed 32-bit integer) mod p, in [0, p).
 cudaError_t launch_mod_p_signed(uint32_t *x, uint64_t n, uint32_t p, int num_sms, cudaStream_t stream);
 
-cudaError_t launch_db_to_f16(const uint8_t *D, uint64_t R, uint64_t C, __half *D16, uint64_t pitch, int num_sms,
-                             cudaStream_t stream);
+// The digits minus `centre` as fp16.
+cudaError_t launch_db_to_f16(const uint8_t *D, uint64_t R, uint64_t C, __half *D16, uint64_t pitch, int centre,
+                             int num_sms, cudaStream_t stream);
 // Limbs of NV vectors (vector v at X + v * x_ld) into L (limb k of vector v in row 4 v + k).
 // When `zero` is given, the same launch also zeroes zero_words words there (the output block of a
 // uint8-digit GEMM launched right after it as its programmatic dependent).

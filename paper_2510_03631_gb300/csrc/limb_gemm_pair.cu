@@ -12,10 +12,10 @@
 //
 // Exactness is that of limb_gemm.cu: balanced byte limbs in fp16, drained to
 // int32 after every exact chunk and recombined as sum_k 2^{8k} s_k in uint32
-// arithmetic.  The chunk depth follows the products' bound: digits times limbs
-// (Response, hint; magnitude <= 255 * 128) take 512-deep chunks, whose sums
-// stay below 2^24; limbs times limbs (client Query/Recover; magnitude <= 2^14)
-// take 1024-deep chunks, whose partial sums never exceed 2^24 in magnitude.
+// arithmetic.  The chunk depth follows the products' bound: digits times
+// centred field elements (magnitude <= 255 * 128) take 512-deep chunks, whose sums
+// stay below 2^24; limbs, or digits centred to d - 128, times limbs (client Query/Recover; Response;
+// magnitude <= 2^14) take 1024-deep chunks, whose partial sums never exceed 2^24 in magnitude.
 // Every integer of magnitude <= 2^24 is an fp32 value, so no partial sum is
 // ever rounded either way.
 //
@@ -521,7 +521,8 @@ __global__ void __launch_bounds__(kPThreads, 1)
                     // part of a split tile: exact, since addition mod 2^32 commutes
 #pragma unroll
                     for (int q = 0; q < QPT; ++q)
-                        if (v0 + q < NV) epi.add(row, v0 + q, run[q]);
+                        if (v0 + q < NV)   // the first piece of a tile adds what centred digits leave out
+                            epi.add(row, v0 + q, run[q] + (pc.c0 == 0 ? epi.pre(row, v0 + q) : 0u));
                     continue;
                 }
             }
@@ -575,8 +576,6 @@ static cudaError_t set_pair_attr() {
 
 cudaError_t prepare_limb_gemm_pair_kernels() {
     cudaError_t e;
-    if ((e = set_pair_attr<64, StoreEpi, false>()) != cudaSuccess) return e;
-    if ((e = set_pair_attr<128, StoreEpi, false>()) != cudaSuccess) return e;
     if ((e = set_pair_attr<256, StoreEpi, false>()) != cudaSuccess) return e;
     if ((e = set_pair_attr<64, QueryNoiseEpi, false>()) != cudaSuccess) return e;
     if ((e = set_pair_attr<128, QueryNoiseEpi, false>()) != cudaSuccess) return e;
@@ -635,10 +634,14 @@ static int resident_pairs(int num_sms) {
     return n;
 }
 
-// k-steps (64 deep) per exact chunk: 8 for digits times limbs (StoreEpi), 16 for limbs times limbs.
+// k-steps (64 deep) per exact chunk: 8 for digits times centred field elements, 16 for limbs or centred
+// digits times limbs.  A split launch deals chunks, so the plain store takes 16 only from 32768 columns
+// up (32768 x 32768, 192 vectors: 875 -> 816 us); with fewer its shares would be too coarse (4096 x 4096,
+// 160 vectors: 32 us with 8, 36 with 16).
+static uint32_t store_chunk_kb(uint32_t KB) { return KB >= 512 ? 16u : 8u; }
 template <class Epi>
 constexpr uint32_t pair_chunk_kb() {
-    return (std::is_same<Epi, StoreEpi>::value || std::is_same<Epi, ModPEpi>::value) ? 8u : 16u;
+    return std::is_same<Epi, ModPEpi>::value ? 8u : 16u;
 }
 
 // Schedule of a plain-store launch over `tiles` pair tiles (n_tiles per row tile, nchunks exact
@@ -752,7 +755,11 @@ static cudaError_t launch_pair_epi(int bn, const CUtensorMap &a_map, const PairB
         return launch_pair_t<256, Epi, false>(a_map, bm, epi, M, NV, KB, pair_chunk_kb<Epi>(), 0, num_sms, status,
                                              stream);
     } else {
-        if (plane_chunks == 0) {
+        if constexpr (std::is_same<Epi, StoreEpi>::value) {   // 256-wide plain tiles only
+            if (bn != 256 || plane_chunks != 0) return cudaErrorInvalidValue;
+            return launch_pair_t<256, Epi, false>(a_map, bm, epi, M, NV, KB, store_chunk_kb(KB), 0, num_sms, status,
+                                                 stream);
+        } else if (plane_chunks == 0) {
             constexpr uint32_t ckb = pair_chunk_kb<Epi>();
             switch (bn) {
                 case 64:
@@ -783,10 +790,22 @@ static cudaError_t launch_pair_epi(int bn, const CUtensorMap &a_map, const PairB
     }
 }
 
-cudaError_t launch_limb_gemm_pair(int bn, const CUtensorMap &a_map, const PairBMaps &bm, uint32_t *out,
-                                  uint64_t ld_m, uint64_t ld_b, uint32_t M, uint32_t NV, uint64_t K, int num_sms,
-                                  int *status, cudaStream_t stream) {
-    return launch_pair_epi(bn, a_map, bm, StoreEpi{out, ld_m, ld_b}, M, NV, K, 0, num_sms, status, stream);
+cudaError_t launch_limb_gemm_pair(const CUtensorMap &a_map, const PairBMaps &bm, const uint32_t *sums, uint32_t centre,
+                                  uint32_t *out, uint64_t ld_m, uint64_t ld_b, uint32_t M, uint32_t NV, uint64_t K,
+                                  int num_sms, int *status, cudaStream_t stream) {
+    return launch_pair_epi(256, a_map, bm, StoreEpi{out, ld_m, ld_b, sums, centre}, M, NV, K, 0, num_sms, status, stream);
+}
+
+double limb_gemm_pair_waves(uint32_t M, uint32_t NV, uint64_t K, int num_sms) {
+    const uint64_t n_tiles = ((uint64_t)NV + 63) / 64, tiles = ((uint64_t)M + 2 * kPM - 1) / (2 * kPM) * n_tiles;
+    const uint32_t KB = static_cast<uint32_t>((K + kPK - 1) / kPK), ckb = store_chunk_kb(KB);
+    const uint64_t pairs = static_cast<uint64_t>(resident_pairs<256, StoreEpi, false>(num_sms));
+    uint64_t clusters = 0;
+    uint32_t dp = 0, tail = 0;
+    if (pairs == 0) return 0.0;
+    if (pair_split_schedule(tiles, n_tiles, (KB + ckb - 1) / ckb, pairs, &clusters, &dp, &tail))
+        return static_cast<double>(dp) / pairs + static_cast<double>(tiles - dp) / (tail * n_tiles);
+    return static_cast<double>((tiles + pairs - 1) / pairs);
 }
 
 cudaError_t launch_limb_gemm_pair_query(int bn, const CUtensorMap &a_map, const PairBMaps &bm,

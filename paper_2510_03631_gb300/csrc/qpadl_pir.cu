@@ -19,6 +19,7 @@
 #include "client.cuh"
 #include "limb_gemm.cuh"
 #include "limb_gemm_pair.cuh"
+#include "limb_gemm_tri.cuh"
 #include "limb_gemm_u8.cuh"
 #include "internal.cuh"
 #include "qpadl_pir.h"
@@ -49,9 +50,10 @@ struct qpadl_db {
     uint32_t u8_max_batch = 64;      // QPADL_OPT_U8_MAX_BATCH
     int u8_kstep = 0;                // QPADL_OPT_U8_KSTEP (0 = per tile width default)
     int pair_gemm = 1;               // QPADL_OPT_PAIR_GEMM
-    __half *d16 = nullptr;           // digits as fp16, R x pitch
+    __half *d16 = nullptr;           // digits as fp16, R x pitch (single-SM tiles, Z_p)
+    __half *d16c = nullptr;          // digits minus 128 as fp16, R x pitch (three-limb pair tiles)
     uint64_t pitch = 0;              // roundup(C, 8)
-    CUtensorMap a_map;
+    CUtensorMap a_map, ac_map;       // over d16, d16c
     __half *limbs = nullptr;         // limb scratch
     uint64_t limbs_bytes = 0;
     // host-buffer calls
@@ -167,6 +169,7 @@ int prepare_device(int dev) {
     QPADL_CU(prepare_stream_kernels());
     QPADL_CU(prepare_limb_gemm_kernels());
     QPADL_CU(prepare_limb_gemm_pair_kernels());
+    QPADL_CU(prepare_limb_gemm_tri_kernels());
     QPADL_CU(prepare_limb_gemm_u8_kernels());
     QPADL_CU(prepare_client_kernels());
     QPADL_CU(prepare_chor_kernels());
@@ -222,17 +225,30 @@ void dev_free(qpadl_db *db, void *p, uint64_t bytes) {
     }
 }
 
-int ensure_tensor_copy(qpadl_db *db, cudaStream_t stream) {
-    if (db->d16) return QPADL_OK;
+// An fp16 copy of the digits minus `centre`, and its tensor map.
+int build_f16_copy(qpadl_db *db, __half **copy, CUtensorMap *map, int centre, cudaStream_t stream) {
+    if (*copy) return QPADL_OK;
     const uint64_t R = db->prm.rows, C = db->prm.cols;
-    const uint64_t bytes = R * db->pitch * 2;
-    int rc = dev_alloc(db, reinterpret_cast<void **>(&db->d16), bytes);
+    int rc = dev_alloc(db, reinterpret_cast<void **>(copy), R * db->pitch * 2);
     if (rc != QPADL_OK) return rc;
-    QPADL_CU(launch_db_to_f16(db->db, R, C, db->d16, db->pitch, db->num_sms, stream));
-    if (!encode_2d(&db->a_map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, db->d16, C, R, db->pitch * 2, kLimbBoxK,
-                   kLimbBoxM, CU_TENSOR_MAP_SWIZZLE_128B))
+    QPADL_CU(launch_db_to_f16(db->db, R, C, *copy, db->pitch, centre, db->num_sms, stream));
+    if (!encode_2d(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, *copy, C, R, db->pitch * 2, kLimbBoxK, kLimbBoxM,
+                   CU_TENSOR_MAP_SWIZZLE_128B))
         return QPADL_ECUDA;
     return QPADL_OK;
+}
+
+int ensure_tensor_copy(qpadl_db *db, cudaStream_t stream) {
+    return build_f16_copy(db, &db->d16, &db->a_map, 0, stream);
+}
+
+// Whether batches beyond the uint8-digit GEMM run on three-limb pair tiles (else on single SMs).
+bool use_tri(const qpadl_db *db) { return db->pair_gemm && db->num_sms >= 2; }
+
+// The fp16 copy that batches of this handle read.
+int ensure_batch_copy(qpadl_db *db, cudaStream_t stream) {
+    return use_tri(db) ? build_f16_copy(db, &db->d16c, &db->ac_map, kTriCentre, stream)
+                       : ensure_tensor_copy(db, stream);
 }
 
 int ensure_limbs(qpadl_db *db, uint64_t bytes) {
@@ -257,21 +273,31 @@ int set_device(const qpadl_db *db) {
     return QPADL_OK;
 }
 
-// out[i * ld_m + v * ld_b] = D * X[v] for NV vectors given as fp16 limbs at `limbs`
-// (4 NV rows of db->pitch elements), on CTA pairs or single SMs (QPADL_OPT_PAIR_GEMM)
-int run_limb_gemm_at(qpadl_db *db, const __half *limbs, uint32_t NV, uint32_t *out, uint64_t ld_m, uint64_t ld_b,
-                     cudaStream_t stream) {
-    if (db->pair_gemm && db->num_sms >= 2) {
-        const int bn = limb_gemm_pair_bn_for(NV);
-        PairBMaps bm;
-        std::memset(&bm, 0, sizeof(bm));
-        if (!encode_2d(&bm.m[0], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, limbs, db->prm.cols, 4ull * NV, db->pitch * 2,
-                       kLimbBoxK, pair_b_box_rows(bn, false, 0), CU_TENSOR_MAP_SWIZZLE_128B))
-            return QPADL_ECUDA;
-        QPADL_CU(launch_limb_gemm_pair(bn, db->a_map, bm, out, ld_m, ld_b, static_cast<uint32_t>(db->prm.rows), NV,
-                                       db->prm.cols, db->num_sms, db->d_status, stream));
-        return QPADL_OK;
-    }
+// out[i * ld_m + v * ld_b] = D * X[v] for NV vectors given as limbs at `limbs`: three limbs and the
+// vectors' sums (launch_vec_limbs_tri) for pair tiles over d16c, or (run_limb_gemm) four, 4 NV rows of
+// db->pitch elements, for single-SM tiles over d16
+int run_tri_gemm(qpadl_db *db, const __half *limbs, uint32_t NV, uint32_t *out, uint64_t ld_m, uint64_t ld_b,
+                 uint32_t ranges, cudaStream_t stream) {
+    const uint64_t C = db->prm.cols;
+    CUtensorMap b_map;   // (column, vector, limb): a box is one CTA's 32 vectors x 3 limbs
+    auto fn = encode_fn();
+    cuuint64_t dims[3] = {C, NV, 3};
+    cuuint64_t strides[2] = {6 * db->pitch, 2 * db->pitch};
+    cuuint32_t box[3] = {kLimbBoxK, kTriGroup, 3};
+    cuuint32_t estr[3] = {1, 1, 1};
+    if (!fn || fn(&b_map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<__half *>(limbs), dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return QPADL_ECUDA;
+    const uint32_t *sums = reinterpret_cast<const uint32_t *>(reinterpret_cast<const uint8_t *>(limbs) +
+                                                              tri_sums_offset(NV, db->pitch));
+    QPADL_CU(launch_limb_gemm_tri(db->ac_map, b_map, sums, out, ld_m, ld_b, static_cast<uint32_t>(db->prm.rows), NV, C,
+                                  ranges, db->num_sms, db->d_status, stream));
+    return QPADL_OK;
+}
+
+int run_limb_gemm(qpadl_db *db, const __half *limbs, uint32_t NV, uint32_t *out, uint64_t ld_m, uint64_t ld_b,
+                  cudaStream_t stream) {
     const int bn = limb_gemm_bn_for(NV);
     CUtensorMap b_map;
     if (!encode_2d(&b_map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, limbs, db->prm.cols, 4ull * NV, db->pitch * 2,
@@ -282,8 +308,49 @@ int run_limb_gemm_at(qpadl_db *db, const __half *limbs, uint32_t NV, uint32_t *o
     return QPADL_OK;
 }
 
-int run_limb_gemm(qpadl_db *db, uint32_t NV, uint32_t *out, uint64_t ld_m, uint64_t ld_b, cudaStream_t stream) {
-    return run_limb_gemm_at(db, db->limbs, NV, out, ld_m, ld_b, stream);
+// Whether a batch on pair tiles takes four byte limbs instead of three: only with an odd number of
+// 64-vector halves, where the three-limb tiles (two halves, or three for 3 and 5) leave a half empty
+// or the last wave uneven.  Both times are in units of 256 rows x 64 vectors; a three-limb unit takes 0.93 of a
+// four-limb one, and 1.08 times that in tiles of three.  Measured, four limbs against three
+// (us): 32768 x 32768, 160 vectors 793 / 873, 192 816 / 915, 448 1927 / 2053; 8192 x 32768, 192
+// 242 / 277, 320 499 / 464, 448 493 / 563; 2000 x 30000, 320 157 / 134.
+bool four_limbs(const qpadl_db *db, uint32_t B) {
+    const uint32_t halves = (B - 1) / 64 + 1, M = static_cast<uint32_t>(db->prm.rows);
+    if (halves < 3 || halves % 2 == 0) return false;
+    const double four = limb_gemm_pair_waves(M, B, db->prm.cols, db->num_sms) * 1.07;
+    const double three = limb_gemm_tri_waves(M, B, db->prm.cols, db->num_sms) * (halves <= 5 ? 1.08 : 1.0);
+    return four < three;
+}
+
+// Limb scratch of a batch of B (at most 4096): four limbs and a word per query.
+uint64_t limb_bytes(const qpadl_db *db, uint32_t B) { return 8ull * B * db->pitch + 4ull * B; }
+
+// Answers of B queries (at most 4096) on an fp16 copy that exists, their limbs made at `limbs`
+// (8 B pitch bytes, or limb_bytes where four limbs on pair tiles are allowed).
+int answer_f16(qpadl_db *db, const uint32_t *Q, uint32_t B, uint32_t *ans, __half *limbs, bool tri, bool allow_four,
+               cudaStream_t stream) {
+    const uint64_t C = db->prm.cols, R = db->prm.rows;
+    if (tri && allow_four && four_limbs(db, B)) {
+        QPADL_CU(launch_vec_limbs_four(Q, C, B, C, limbs, db->pitch, stream));
+        PairBMaps bm;
+        std::memset(&bm, 0, sizeof(bm));
+        if (!encode_2d(&bm.m[0], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, limbs, C, 4ull * B, db->pitch * 2, kLimbBoxK,
+                       pair_b_box_rows(256, false, 0), CU_TENSOR_MAP_SWIZZLE_128B))
+            return QPADL_ECUDA;
+        const uint32_t *sums = reinterpret_cast<const uint32_t *>(reinterpret_cast<const uint8_t *>(limbs) +
+                                                                  four_sums_offset(B, db->pitch));
+        QPADL_CU(launch_limb_gemm_pair(db->ac_map, bm, sums, kTriCentre, ans, 1, R, static_cast<uint32_t>(R), B, C,
+                                       db->num_sms, db->d_status, stream));
+        return QPADL_OK;
+    }
+    if (tri) {
+        const uint32_t ranges = limb_gemm_tri_ranges(static_cast<uint32_t>(R), B, C, 1, R, db->num_sms);
+        // one launch makes the limbs and zeroes the answers that ranges add to
+        QPADL_CU(launch_vec_limbs_tri(Q, C, B, C, limbs, db->pitch, ranges > 1 ? ans : nullptr, (uint64_t)B * R, stream));
+        return run_tri_gemm(db, limbs, B, ans, 1, R, ranges, stream);
+    }
+    QPADL_CU(launch_vec_limbs(Q, C, B, C, limbs, db->pitch, db->num_sms, stream));
+    return run_limb_gemm(db, limbs, B, ans, 1, R, stream);
 }
 
 int answer_stream_group(qpadl_db *db, const uint32_t *Q, uint32_t nq, uint32_t *ans, cudaStream_t stream) {
@@ -429,17 +496,16 @@ int answer_tensor_u8(qpadl_db *db, const uint32_t *Q, uint32_t B, uint32_t *ans,
 
 int answer_tensor(qpadl_db *db, const uint32_t *Q, uint32_t B, uint32_t *ans, cudaStream_t stream) {
     if (db->u8_ok && B <= db->u8_max_batch) return answer_tensor_u8(db, Q, B, ans, stream);
-    int rc = ensure_tensor_copy(db, stream);
+    int rc = ensure_batch_copy(db, stream);
     if (rc != QPADL_OK) return rc;
     // chunks of at most 4096 queries bound the limb scratch (8 bytes per query per column)
     constexpr uint32_t kChunk = 4096;
-    rc = ensure_limbs(db, 8ull * std::min(B, kChunk) * db->pitch);
+    rc = ensure_limbs(db, limb_bytes(db, std::min(B, kChunk)));
     if (rc != QPADL_OK) return rc;
     const uint64_t C = db->prm.cols, R = db->prm.rows;
     for (uint32_t b0 = 0; b0 < B; b0 += kChunk) {
         const uint32_t Bc = std::min(B - b0, kChunk);
-        QPADL_CU(launch_vec_limbs(Q + (uint64_t)b0 * C, C, Bc, C, db->limbs, db->pitch, db->num_sms, stream));
-        rc = run_limb_gemm(db, Bc, ans + (uint64_t)b0 * R, 1, R, stream);
+        rc = answer_f16(db, Q + (uint64_t)b0 * C, Bc, ans + (uint64_t)b0 * R, db->limbs, use_tri(db), true, stream);
         if (rc != QPADL_OK) return rc;
     }
     return QPADL_OK;
@@ -454,7 +520,7 @@ uint64_t db_limb_pitch(const qpadl_db *db) { return db->pitch; }
 int db_num_sms(const qpadl_db *db) { return db->num_sms; }
 int *db_status_word(qpadl_db *db) { return db->d_status; }
 int db_prepare_u8(qpadl_db *db, cudaStream_t stream) { return ensure_blocked(db, stream); }
-int db_prepare_f16(qpadl_db *db, cudaStream_t stream) { return ensure_tensor_copy(db, stream); }
+int db_prepare_f16(qpadl_db *db, cudaStream_t stream) { return ensure_batch_copy(db, stream); }
 bool db_pair_gemm(const qpadl_db *db) { return db->pair_gemm && db->num_sms >= 2; }
 
 int db_fill_u8_group(qpadl_db *db, GroupedGemmArgs &args, int g, const __half *limbs, uint32_t NV, uint32_t *out,
@@ -481,10 +547,10 @@ int db_fill_u8_group(qpadl_db *db, GroupedGemmArgs &args, int g, const __half *l
 
 int db_answer_f16_ws(qpadl_db *db, const uint32_t *Q, uint32_t B, uint32_t *ans, __half *limbs,
                      cudaStream_t stream) {
-    if (!db->d16) return QPADL_EINVAL;
-    const uint64_t C = db->prm.cols, R = db->prm.rows;
-    QPADL_CU(launch_vec_limbs(Q, C, B, C, limbs, db->pitch, db->num_sms, stream));
-    return run_limb_gemm_at(db, limbs, B, ans, 1, R, stream);
+    // the copy that was prepared, even if the handle's tile option has changed since
+    const bool tri = db->d16c && (use_tri(db) || !db->d16);
+    if (!tri && !db->d16) return QPADL_EINVAL;
+    return answer_f16(db, Q, B, ans, limbs, tri, false, stream);   // the workspace has no room for the sums of four
 }
 
 int db_answer_one_noscratch(qpadl_db *db, const uint32_t *q, uint32_t *ans, cudaStream_t stream) {
@@ -609,7 +675,7 @@ int qpadl_pir_setup(const qpadl_params *prm, const uint8_t *db_dev, qpadl_stream
     if ((rc = dev_alloc(db, reinterpret_cast<void **>(&db->stage_q), C * 4)) != QPADL_OK) return fail(rc);
     if ((rc = dev_alloc(db, reinterpret_cast<void **>(&db->stage_ans), R * 4)) != QPADL_OK) return fail(rc);
     if (prm->flags & QPADL_SETUP_TENSOR_COPY) {
-        if ((rc = ensure_tensor_copy(db, s)) != QPADL_OK) return fail(rc);
+        if ((rc = ensure_batch_copy(db, s)) != QPADL_OK) return fail(rc);
     }
     *out = db;
     return QPADL_OK;
@@ -624,6 +690,7 @@ int qpadl_pir_destroy(qpadl_db *db) {
     dev_free(db, db->d_status, 16);
     dev_free(db, db->qpack, 4 * db->pack_words * 4);
     dev_free(db, db->d16, db->prm.rows * db->pitch * 2);
+    dev_free(db, db->d16c, db->prm.rows * db->pitch * 2);
     dev_free(db, db->blk, db->blk_bytes);
     dev_free(db, db->limbs, db->limbs_bytes);
     dev_free(db, db->stage_q, db->prm.cols * 4);
@@ -671,7 +738,7 @@ int qpadl_pir_reserve(qpadl_db *db, uint32_t max_batch, qpadl_stream_t stream) {
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     if (max_batch >= db->tensor_min_batch) {
         if (!(db->u8_ok && max_batch <= db->u8_max_batch)) {
-            int rc = ensure_tensor_copy(db, s);
+            int rc = ensure_batch_copy(db, s);
             if (rc != QPADL_OK) return rc;
         }
         if (db->u8_ok && db->u8_max_batch >= db->tensor_min_batch) {
@@ -679,7 +746,7 @@ int qpadl_pir_reserve(qpadl_db *db, uint32_t max_batch, qpadl_stream_t stream) {
             if (rc != QPADL_OK) return rc;
         }
         // the batched paths work in chunks of at most 4096 queries
-        int rc = ensure_limbs(db, 8ull * std::min<uint32_t>(max_batch, 4096u) * db->pitch);
+        int rc = ensure_limbs(db, limb_bytes(db, std::min<uint32_t>(max_batch, 4096u)));
         if (rc != QPADL_OK) return rc;
     }
     QPADL_CU(cudaStreamSynchronize(s));
@@ -703,12 +770,19 @@ int qpadl_pir_hint(qpadl_db *db, const uint32_t *A_dev, uint32_t *H_dev, qpadl_s
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const uint32_t n = db->prm.n;
     const bool u8 = db->u8_ok && n <= db->u8_max_batch;   // the lean layout keeps no fp16 copy
-    int rc = u8 ? ensure_blocked(db, s) : ensure_tensor_copy(db, s);
+    int rc = u8 ? ensure_blocked(db, s) : ensure_batch_copy(db, s);
     if (rc != QPADL_OK) return rc;
     rc = ensure_limbs(db, 8ull * n * db->pitch);
     if (rc != QPADL_OK) return rc;
+    if (!u8 && use_tri(db)) {
+        const uint64_t R = db->prm.rows;
+        const uint32_t ranges = limb_gemm_tri_ranges(static_cast<uint32_t>(R), n, db->prm.cols, n, 1, db->num_sms);
+        if (ranges > 1) QPADL_CU(cudaMemsetAsync(H_dev, 0, 4ull * n * R, s));
+        QPADL_CU(launch_mat_col_limbs_tri(A_dev, db->prm.cols, n, db->limbs, db->pitch, s));
+        return run_tri_gemm(db, db->limbs, n, H_dev, n, 1, ranges, s);
+    }
     QPADL_CU(launch_mat_col_limbs(A_dev, db->prm.cols, n, db->limbs, db->pitch, s));
-    return u8 ? run_u8_gemm(db, n, H_dev, n, 1, s) : run_limb_gemm(db, n, H_dev, n, 1, s);
+    return u8 ? run_u8_gemm(db, n, H_dev, n, 1, s) : run_limb_gemm(db, db->limbs, n, H_dev, n, 1, s);
 }
 
 int qpadl_pir_query(const qpadl_params *prm, const uint32_t *A_dev, const uint32_t *s_dev, const int32_t *e_dev,
