@@ -37,6 +37,7 @@ struct qpadl_db {
     bool stream_ok = false;          // C % 16 == 0 and D 16-byte aligned
     int stream_chunk = 2048;         // digits per row per stage (QPADL_OPT_STREAM_CHUNK)
     int stream_raw = 0;              // QPADL_OPT_STREAM_RAW
+    bool stream_raw_set = false;     // ... chosen by the caller or the tuner
     uint32_t tensor_min_batch = 3;   // QPADL_OPT_TENSOR_MIN_BATCH
     bool stream_maps = false;        // C % 256 == 0: 3-D tensor maps below are valid
     CUtensorMap stream_map[4];       // box {256, cch/256, 8} for cch = 512 << i
@@ -107,6 +108,11 @@ struct qpadl_chor {
 namespace {
 
 constexpr int kMaxN = 16384;
+// Largest database whose one query, or two, are packed in the streaming kernel by default, and its widest
+// rows (every CTA packs the whole query).  Separate pack launch against one launch, back to back (us): 1024 x
+// 1024 10.5 / 8.4 (two queries 11.4 / 9.0), 2048 x 2048 10.6 / 8.6 (10.9 / 9.4), 4096 x 4096 10.5 / 8.5 (12.2 /
+// 12.5), 6144 x 6144 12.4 / 12.4 (16.5 / 20.6), 8192 x 8192 14.4 / 16.5.
+constexpr uint64_t kRawCells = 16ull << 20, kRawCells2 = 4ull << 20, kRawCols = 4096;
 // Smallest Chor batch on the tensor cores for records of W words, unless the caller chose one.  Their
 // time hardly depends on the batch up to 64 queries; the scan's grows with it and its column tiles
 // are 1024 words wide (one query; a narrower record leaves their threads idle).  Measured, scan
@@ -372,28 +378,33 @@ int answer_stream_group(qpadl_db *db, const uint32_t *Q, uint32_t nq, uint32_t *
 int raw2_chunk(const qpadl_db *db) { return db->stream_chunk == 2048 ? 2048 : 1024; }
 
 int answer_two_raw(qpadl_db *db, const uint32_t *Q, uint64_t q_ld, uint32_t *ans, uint64_t ans_ld,
-                   cudaStream_t stream) {
+                   cudaStream_t stream, bool pdl = true) {
     const uint64_t C = db->prm.cols, R = db->prm.rows;
     const int cch = raw2_chunk(db);
     int mi = 0;
     while ((512 << mi) < cch) ++mi;
     const CUtensorMap *map = db->stream_maps ? &db->stream_map[mi] : nullptr;
     QPADL_CU(launch_stream_answer_raw2(cch, map, db->db, static_cast<uint32_t>(R), static_cast<uint32_t>(C), Q, q_ld,
-                                       ans, ans_ld, db->num_sms, db->d_status, stream));
+                                       ans, ans_ld, db->num_sms, db->d_status, stream, pdl));
     return QPADL_OK;
 }
 
 int answer_streaming(qpadl_db *db, const uint32_t *Q, uint32_t B, uint32_t *ans, cudaStream_t stream) {
     const uint64_t C = db->prm.cols, R = db->prm.rows;
-    if (db->stream_ok && B == 2 && db->stream_raw && aligned16(Q))
-        return answer_two_raw(db, Q, C, ans, R, stream);   // both queries in one pass, no scratch
-    if (db->stream_ok && B == 1 && db->stream_raw && aligned16(Q)) {
+    // Unless the caller chose, a small database's one or two queries are packed in the streaming kernel as well:
+    // one launch instead of two.  It is an ordinary launch there: as a programmatic dependent it would read the
+    // database before the kernel before it ends, which may be the one that writes it (the separate pack
+    // launch keeps that order for larger ones, and its cost is lost in the scan).
+    const bool small = !db->stream_raw_set && C <= kRawCols && R * C <= (B == 1 ? kRawCells : kRawCells2);
+    const bool raw = db->stream_ok && (db->stream_raw || small) && aligned16(Q);
+    if (raw && B == 2) return answer_two_raw(db, Q, C, ans, R, stream, !small);   // both queries in one pass, no scratch
+    if (raw && B == 1) {
         // one query: the streaming kernel packs its limbs itself (one launch, no scratch)
         int mi = 0;
         while ((512 << mi) < db->stream_chunk) ++mi;
         const CUtensorMap *map = db->stream_maps ? &db->stream_map[mi] : nullptr;
         QPADL_CU(launch_stream_answer_raw(db->stream_chunk, map, db->db, static_cast<uint32_t>(R),
-                                          static_cast<uint32_t>(C), Q, ans, db->num_sms, db->d_status, stream));
+                                          static_cast<uint32_t>(C), Q, ans, db->num_sms, db->d_status, stream, !small));
         return QPADL_OK;
     }
     if (!db->stream_ok) {
@@ -852,6 +863,7 @@ int qpadl_pir_set_option(qpadl_db *db, int option, int64_t value) {
         case QPADL_OPT_STREAM_RAW:
             if (value != 0 && value != 1) return QPADL_EINVAL;
             db->stream_raw = static_cast<int>(value);
+            db->stream_raw_set = true;
             return QPADL_OK;
         case QPADL_OPT_U8_MAX_BATCH:
             if (value < 0 || value > (1ll << 30)) return QPADL_EINVAL;
@@ -919,6 +931,7 @@ int qpadl_pir_autotune(qpadl_db *db, uint32_t max_batch, qpadl_stream_t stream, 
             if (!db->stream_ok || !stream_config_valid(1, chunks[ci])) continue;
             db->stream_chunk = chunks[ci];
             db->stream_raw = raw;
+            db->stream_raw_set = true;
             const double ms = time_calls([&] { return answer_streaming(db, Q, 1, A, s); }, s, kReps);
             rep.single_ms[ci][raw] = ms;
             if (ms > 0 && ms < best) {
@@ -930,6 +943,7 @@ int qpadl_pir_autotune(qpadl_db *db, uint32_t max_batch, qpadl_stream_t stream, 
     }
     db->stream_chunk = best_chunk;
     db->stream_raw = best_raw;
+    db->stream_raw_set = true;
     // 2. small batches: digit-tile depth of the uint8 GEMM, then the streaming/tensor crossover
     rep.tuned_batch = BT;
     if (max_batch >= 2) {

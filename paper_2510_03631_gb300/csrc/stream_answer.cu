@@ -395,11 +395,11 @@ cudaError_t launch_pack_query(const uint32_t *q, uint64_t q_ld, uint32_t C, uint
     return cudaGetLastError();
 }
 
-// Launch with programmatic dependent launch allowed (see the kernel comment).
+// Launch with programmatic dependent launch allowed (see the kernel comment), or as an ordinary launch.
 template <int NQ, int CCH, int QM, class Epi>
 static cudaError_t launch_cfg(const CUtensorMap *map, const uint8_t *D, uint32_t R, uint32_t C,
                               const uint32_t *qsrc, uint64_t pack_ld, const Epi &epi, int grid, int *status,
-                              cudaStream_t stream) {
+                              cudaStream_t stream, bool pdl = true) {
     CUtensorMap m;
     if (map) m = *map;
     else std::memset(&m, 0, sizeof(m));
@@ -412,7 +412,7 @@ static cudaError_t launch_cfg(const CUtensorMap *map, const uint8_t *D, uint32_t
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = pdl ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, stream_answer_kernel<NQ, CCH, QM, Epi>, m, map ? 1 : 0, D, R, C, qsrc, pack_ld,
                               epi, status);
 }
@@ -441,26 +441,27 @@ cudaError_t launch_stream_answer(int nq, int cch, const CUtensorMap *map, const 
 
 cudaError_t launch_stream_answer_raw(int cch, const CUtensorMap *map, const uint8_t *D, uint32_t R, uint32_t C,
                                      const uint32_t *q, uint32_t *ans, int num_sms, int *status,
-                                     cudaStream_t stream) {
+                                     cudaStream_t stream, bool pdl) {
     const int grid = stream_grid(R, num_sms);
     const AnswerEpi epi{ans, 0};
     switch (cch) {
-        case 512: return launch_cfg<1, 512, kQRaw>(map, D, R, C, q, 0, epi, grid, status, stream);
-        case 1024: return launch_cfg<1, 1024, kQRaw>(map, D, R, C, q, 0, epi, grid, status, stream);
-        case 2048: return launch_cfg<1, 2048, kQRaw>(map, D, R, C, q, 0, epi, grid, status, stream);
-        case 4096: return launch_cfg<1, 4096, kQRaw>(map, D, R, C, q, 0, epi, grid, status, stream);
+        case 512: return launch_cfg<1, 512, kQRaw>(map, D, R, C, q, 0, epi, grid, status, stream, pdl);
+        case 1024: return launch_cfg<1, 1024, kQRaw>(map, D, R, C, q, 0, epi, grid, status, stream, pdl);
+        case 2048: return launch_cfg<1, 2048, kQRaw>(map, D, R, C, q, 0, epi, grid, status, stream, pdl);
+        case 4096: return launch_cfg<1, 4096, kQRaw>(map, D, R, C, q, 0, epi, grid, status, stream, pdl);
         default: return cudaErrorInvalidValue;
     }
 }
 
 cudaError_t launch_stream_answer_raw2(int cch, const CUtensorMap *map, const uint8_t *D, uint32_t R, uint32_t C,
                                       const uint32_t *q, uint64_t q_ld, uint32_t *ans, uint64_t ans_ld, int num_sms,
-                                      int *status, cudaStream_t stream) {
+                                      int *status, cudaStream_t stream,
+                                      bool pdl) {
     const int grid = stream_grid(R, num_sms);
     const AnswerEpi epi{ans, ans_ld};
     switch (cch) {
-        case 1024: return launch_cfg<2, 1024, kQRaw>(map, D, R, C, q, q_ld, epi, grid, status, stream);
-        case 2048: return launch_cfg<2, 2048, kQRaw>(map, D, R, C, q, q_ld, epi, grid, status, stream);
+        case 1024: return launch_cfg<2, 1024, kQRaw>(map, D, R, C, q, q_ld, epi, grid, status, stream, pdl);
+        case 2048: return launch_cfg<2, 2048, kQRaw>(map, D, R, C, q, q_ld, epi, grid, status, stream, pdl);
         default: return cudaErrorInvalidValue;
     }
 }
