@@ -433,22 +433,35 @@ __global__ void __launch_bounds__(kPThreads, 1)
                         tmem_ld32(acc + 32u * j, v);
                         if (two) tmem_ld32(oth + 32u * j, w);
                         tmem_wait_ld();
+                        auto cut = [&](uint32_t b) {
+                            const float x = __uint_as_float(b);
+                            return __fmaf_rn(-__fsub_rn(__fmaf_rn(x, inv, kRound), kRound), pf, x);
+                        };
+                        float x[32];
+#pragma unroll
+                        for (int q = 0; q < 32; ++q) x[q] = cut(v[q]);
+                        if (two) {
+#pragma unroll
+                            for (int q = 0; q < 32; ++q) x[q] = __fadd_rn(x[q], cut(w[q]));
+                        }
 #pragma unroll
                         for (int q = 0; q < 32; ++q) {
-                            float x = __uint_as_float(v[q]);
-                            x = __fmaf_rn(-__fsub_rn(__fmaf_rn(x, inv, kRound), kRound), pf, x);
-                            if (two) {
-                                float y = __uint_as_float(w[q]);
-                                y = __fmaf_rn(-__fsub_rn(__fmaf_rn(y, inv, kRound), kRound), pf, y);
-                                x = __fadd_rn(x, y);
-                            }
-                            float r = __fmaf_rn(-floorf(x * inv), pf, x);
+                            float r = __fmaf_rn(-floorf(x[q] * inv), pf, x[q]);
                             if (r < 0.0f) r = __fadd_rn(r, pf);
                             if (r >= pf) r = __fsub_rn(r, pf);
-                            const uint32_t vi = v0 + 32u * j + q;
-                            if (row < M && vi < NV) {
-                                if (whole) epi.store(row, vi, static_cast<uint32_t>(r));
-                                else epi.add(row, vi, static_cast<uint32_t>(r));
+                            v[q] = static_cast<uint32_t>(r);
+                        }
+                        // one loop of stores or one of atomics: a choice per element costs a tile's end 10 us
+                        if (row < M) {
+                            const uint32_t vj = v0 + 32u * j;
+                            if (whole) {
+#pragma unroll
+                                for (int q = 0; q < 32; ++q)
+                                    if (vj + q < NV) epi.store(row, vj + q, v[q]);
+                            } else {
+#pragma unroll
+                                for (int q = 0; q < 32; ++q)
+                                    if (vj + q < NV) epi.add(row, vj + q, v[q]);
                             }
                         }
                     }
@@ -675,26 +688,30 @@ static bool pair_split_schedule(uint64_t tiles, uint64_t n_tiles, uint32_t nchun
     return true;
 }
 
-// Chunk ranges per tile of a Z_p launch: the fewest that bring its tiles (or ranges) within 2% of the
-// best fill of whole waves on `pairs` clusters, when that saves at least 8%.  A tile of such a
-// launch does a quarter of a 4-limb tile's work per byte of D and reads the vector rows (134 MB at
-// 1024 x 65536, more than L2 holds beside D) once per row tile, so all clusters must stay on the same
-// columns: stream-K shares, which spread the clusters over all of K, read them from DRAM for every row
-// tile.  3072 rows, 1024 vectors of 65536 entries, 48 tiles on 76 pairs: whole tiles 290 us, stream-K
-// shares 331, three ranges 250 (and 12 for zeroing and the last mod p).
-static uint32_t field_ksplit(uint64_t tiles, uint32_t nchunks, uint64_t pairs) {
+// Chunk ranges per tile of a Z_p launch, from its time in us: whole waves of ranges on `pairs` clusters, each
+// chunk 2.1 (tensor cores) or, when every cluster reads its own rows of D, up to 2.9 (HBM), and at most 20 for
+// a range's end, when the epilogue combines 256 x 256 residues and the MMAs wait; with more than one range
+// also 12 for two more launches, and the zeroing, adding and last mod p of the output.  Split when that saves
+// 5%.  All clusters work on the same range: a tile does a quarter of a 4-limb tile's work per byte of D and
+// reads the vector rows (134 MB at 1024 x 65536, more than L2 holds beside D) once per row tile, and
+// stream-K shares, which spread the clusters over all of K, read them from DRAM for every row tile.
+// 3072 rows, 1024 vectors of 65536 entries, 48 tiles on 76 pairs: whole tiles 290 us, stream-K shares 331,
+// three ranges 238 (and 12 for zeroing and the last mod p).  32768 x 32768, 256 vectors: whole tiles 421 in all, seven
+// ranges 688; 4000 columns, 600 rows: 36 and 48.
+static uint32_t field_ksplit(uint64_t tiles, uint64_t n_tiles, uint32_t nchunks, uint64_t pairs, uint64_t outputs) {
     if (pairs == 0) return 1;
-    auto fill = [&](uint64_t s) {
-        const uint64_t waves = (tiles * s + pairs - 1) / pairs;
-        return static_cast<double>(tiles * s) / static_cast<double>(waves * pairs);
+    auto time = [&](uint64_t s) {
+        const uint64_t units = tiles * s, waves = (units + pairs - 1) / pairs;
+        const double busy = units < pairs ? static_cast<double>(units) / pairs : 1.0;
+        const double chunk = busy * 2.9 / n_tiles > 2.1 ? busy * 2.9 / n_tiles : 2.1;
+        const double extra = s > 1 ? 12.0 + 12.0 * static_cast<double>(outputs) / 5e6 : 0.0;
+        return static_cast<double>(waves) * (chunk * nchunks / s + 20.0) + extra;
     };
     const uint32_t most = nchunks / 4 < 8 ? nchunks / 4 : 8;   // ranges of at least four chunks
-    double best = fill(1);
-    for (uint32_t s = 2; s <= most; ++s) best = fill(s) > best ? fill(s) : best;
-    if (fill(1) > 0.92 * best) return 1;
+    uint32_t pick = 1;
     for (uint32_t s = 2; s <= most; ++s)
-        if (fill(s) >= 0.98 * best) return s;
-    return 1;
+        if (time(s) < time(pick)) pick = s;
+    return time(pick) < 0.95 * time(1) ? pick : 1;
 }
 
 template <int BN, class Epi, bool PLANED>
@@ -724,7 +741,7 @@ static cudaError_t launch_pair_t(const CUtensorMap &a_map, const PairBMaps &bm, 
         }
     }
     if constexpr (std::is_same<Epi, ModPEpi>::value) {
-        if (epi.ld_m == 1 && epi.ld_b == M) ksplit = field_ksplit(tiles, (KB + ckb - 1) / ckb, pairs);
+        if (epi.ld_m == 1 && epi.ld_b == M) ksplit = field_ksplit(tiles, n_tiles, (KB + ckb - 1) / ckb, pairs, (uint64_t)M * NV);
         if (ksplit > 1) {
             const cudaError_t e = cudaMemsetAsync(epi.out, 0, 4ull * M * NV, stream);
             if (e != cudaSuccess) return e;
