@@ -344,6 +344,8 @@ __global__ void __launch_bounds__(kTThreads, 1)
         const uint32_t taddr = tmem_base + ((quarter * 32u) << 16) + 96u * box;
         const FoldConsts consts;
         griddep_wait();   // the sums and the zeroed output come from the kernel this one overlaps
+        // a row-major output (the hint) is stored 16 bytes at a time: 30000 x 600 digits by 512 columns 214 -> 84 us
+        const bool quads = ld_b == 1 && ld_m % 4 == 0 && (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
         uint32_t item = 0;
         while (!failed && iter.next(pc)) {
             const uint32_t row = pc.m * 2 * kTM + rank * kTM + quarter * 32u + static_cast<uint32_t>(lane);
@@ -393,7 +395,19 @@ __global__ void __launch_bounds__(kTThreads, 1)
             const bool whole = pc.c0 == 0 && pc.c1 == nchunks;   // no other cluster works on this tile
             if (row < M) {
 #pragma unroll
-                for (int h = 0; h < H; ++h)
+                for (int h = 0; h < H; ++h) {
+                    if (quads && whole && v0 + 64u * h + 32u <= NV) {   // 32 neighbouring words of a row
+                        uint4 *dst = reinterpret_cast<uint4 *>(out + (uint64_t)row * ld_m + v0 + 64u * h);
+#pragma unroll
+                        for (int q = 0; q < 32; q += 4) {
+                            const uint32_t *sv = sums + v0 + 64u * h + q;
+                            dst[q / 4] = make_uint4(run[h][q] + kTriCentre * __ldg(sv),
+                                                    run[h][q + 1] + kTriCentre * __ldg(sv + 1),
+                                                    run[h][q + 2] + kTriCentre * __ldg(sv + 2),
+                                                    run[h][q + 3] + kTriCentre * __ldg(sv + 3));
+                        }
+                        continue;
+                    }
 #pragma unroll
                     for (int q = 0; q < 32; ++q) {
                         const uint32_t v = v0 + 64u * h + q;
@@ -405,6 +419,7 @@ __global__ void __launch_bounds__(kTThreads, 1)
                         if (whole) *dst = r;
                         else atomicAdd(dst, r);
                     }
+                }
             }
         }
     }
@@ -676,14 +691,17 @@ static uint32_t tri_ksplit(uint64_t tiles, uint32_t nchunks, uint64_t pairs, dou
 
 // Halves per tile.  Two, so that a row of tiles has no odd narrow one where that can be helped: up to 64 vectors
 // one, and three for three halves (129 to 192 vectors: one tile; 8192 x 32768, 160 vectors: 277 us, tiles of
-// two and one 318) or five (3 + 2).
-static int tri_halves(uint32_t NV) {
+// two and one 318) or five (3 + 2).  One also for so few columns that tiles are not cut into ranges, when even
+// then a tile is left for every cluster (600 x 700 by 512 columns: 18 us, 41 with two halves and word stores).
+static int tri_halves(uint32_t M, uint32_t NV, uint64_t K, int num_sms) {
+    const uint64_t m_tiles = ((uint64_t)M + 2 * kTM - 1) / (2 * kTM);
     const uint32_t nh = (NV - 1) / 64 + 1;
-    return nh == 1 ? 1 : (nh == 3 || nh == 5 ? 3 : 2);
+    if (nh == 1 || (K <= 15 * kTK * kChunkSteps && m_tiles * nh <= (uint64_t)num_sms / 2)) return 1;
+    return nh == 3 || nh == 5 ? 3 : 2;
 }
 
 double limb_gemm_tri_waves(uint32_t M, uint32_t NV, uint64_t K, int num_sms) {
-    const int h = tri_halves(NV);
+    const int h = tri_halves(M, NV, K, num_sms);
     const uint64_t pairs = static_cast<uint64_t>(h == 1 ? tri_resident_pairs<1>(num_sms)
                                                  : (h == 2 ? tri_resident_pairs<2>(num_sms) : tri_resident_pairs<3>(num_sms)));
     if (pairs == 0) return 0.0;
@@ -698,7 +716,7 @@ uint32_t limb_gemm_tri_ranges(uint32_t M, uint32_t NV, uint64_t K, uint64_t ld_m
     if (!((ld_m == 1 && ld_b == M) || (ld_b == 1 && ld_m == NV))) return 1;
     const uint64_t m_tiles = ((uint64_t)M + 2 * kTM - 1) / (2 * kTM);
     const uint32_t nchunks = static_cast<uint32_t>((K + kTK * kChunkSteps - 1) / (kTK * kChunkSteps));
-    const int h = tri_halves(NV);
+    const int h = tri_halves(M, NV, K, num_sms);
     const uint64_t tiles = m_tiles * (((uint64_t)NV + 64 * h - 1) / (64 * h));
     const int pairs = h == 1 ? tri_resident_pairs<1>(num_sms)
                              : (h == 2 ? tri_resident_pairs<2>(num_sms) : tri_resident_pairs<3>(num_sms));
@@ -724,7 +742,7 @@ cudaError_t launch_limb_gemm_tri(const CUtensorMap &a_map, const CUtensorMap &b_
                                  uint32_t ranges, int num_sms, int *status, cudaStream_t stream) {
     if (M == 0 || NV == 0 || K == 0 || ranges == 0 || num_sms < 2) return cudaErrorInvalidValue;
     const uint32_t KB = static_cast<uint32_t>((K + kTK - 1) / kTK);
-    const int h = tri_halves(NV);
+    const int h = tri_halves(M, NV, K, num_sms);
     if (h == 1) return launch_tri_t<1>(a_map, b_map, sums, out, ld_m, ld_b, M, NV, KB, ranges, num_sms, status, stream);
     if (h == 3) return launch_tri_t<3>(a_map, b_map, sums, out, ld_m, ld_b, M, NV, KB, ranges, num_sms, status, stream);
     return launch_tri_t<2>(a_map, b_map, sums, out, ld_m, ld_b, M, NV, KB, ranges, num_sms, status, stream);

@@ -50,7 +50,8 @@ def test_batched_response(R, C, B):
     db.close()
 
 
-@pytest.mark.parametrize("R,C,n", [(200, 300, 33), (300, 1000, 100), (520, 2100, 512), (257, 131, 70), (2000, 700, 130)])
+@pytest.mark.parametrize("R,C,n", [(200, 300, 33), (300, 1000, 100), (520, 2100, 512), (257, 131, 70), (2000, 700, 130),
+                                   (600, 700, 512), (300, 5000, 68), (9000, 200, 96), (700, 4000, 320)])
 def test_hint(R, C, n):
     D = inputs.db_digits(R, C, 256, seed=R + n)
     A = inputs.public_matrix(C, n, seed=C)
