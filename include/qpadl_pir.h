@@ -92,7 +92,9 @@ int qpadl_version(void);
 #define QPADL_OPT_STREAM_RAW 3       /* 1: one or two queries are packed inside the streaming
                                         kernel (one launch, no scratch; two queries share one
                                         pass over D); 0 (default): a separate packing launch
-                                        first */
+                                        first, except that until the option is set a small
+                                        database (at most 4096 columns and 16 Mi digits, 4 Mi
+                                        for two queries) takes one ordinary launch */
 #define QPADL_OPT_U8_MAX_BATCH 4     /* batches of up to this many queries (0..2^30, default 64)
                                         run the tensor-core GEMM on the uint8 digits as stored;
                                         larger ones use the handle's fp16 operand copy, and so
