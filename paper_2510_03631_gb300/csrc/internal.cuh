@@ -13,6 +13,9 @@ namespace qpadl {
 
 // Row pitch (elements) of a limb operand for this database: roundup(C, 8).
 uint64_t db_limb_pitch(const qpadl_db *db);
+// Bytes of limb workspace for B queries: four fp16 limbs, and from three queries on (the smallest batch
+// that needs it) a word each for their sums.
+inline uint64_t limb_workspace_bytes(uint32_t B, uint64_t pitch) { return 8ull * B * pitch + (B > 2 ? 4ull * B : 0); }
 int db_num_sms(const qpadl_db *db);
 int *db_status_word(qpadl_db *db);
 
@@ -31,7 +34,7 @@ int db_fill_u8_group(qpadl_db *db, GroupedGemmArgs &args, int g, const __half *l
 // Whether this handle runs its batched GEMMs on CTA pairs (QPADL_OPT_PAIR_GEMM).
 bool db_pair_gemm(const qpadl_db *db);
 
-// Batched answer on the fp16 copy with the limbs in caller workspace (8 B pitch bytes).
+// Batched answer on the fp16 copy with the limbs in caller workspace (limb_workspace_bytes).
 int db_answer_f16_ws(qpadl_db *db, const uint32_t *Q, uint32_t B, uint32_t *ans, __half *limbs,
                      cudaStream_t stream);
 

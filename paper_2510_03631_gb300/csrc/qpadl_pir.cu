@@ -328,15 +328,12 @@ bool four_limbs(const qpadl_db *db, uint32_t B) {
     return four < three;
 }
 
-// Limb scratch of a batch of B (at most 4096): four limbs and a word per query.
-uint64_t limb_bytes(const qpadl_db *db, uint32_t B) { return 8ull * B * db->pitch + 4ull * B; }
-
 // Answers of B queries (at most 4096) on an fp16 copy that exists, their limbs made at `limbs`
-// (8 B pitch bytes, or limb_bytes where four limbs on pair tiles are allowed).
-int answer_f16(qpadl_db *db, const uint32_t *Q, uint32_t B, uint32_t *ans, __half *limbs, bool tri, bool allow_four,
+// (limb_workspace_bytes).
+int answer_f16(qpadl_db *db, const uint32_t *Q, uint32_t B, uint32_t *ans, __half *limbs, bool tri,
                cudaStream_t stream) {
     const uint64_t C = db->prm.cols, R = db->prm.rows;
-    if (tri && allow_four && four_limbs(db, B)) {
+    if (tri && four_limbs(db, B)) {
         QPADL_CU(launch_vec_limbs_four(Q, C, B, C, limbs, db->pitch, stream));
         PairBMaps bm;
         std::memset(&bm, 0, sizeof(bm));
@@ -511,12 +508,12 @@ int answer_tensor(qpadl_db *db, const uint32_t *Q, uint32_t B, uint32_t *ans, cu
     if (rc != QPADL_OK) return rc;
     // chunks of at most 4096 queries bound the limb scratch (8 bytes per query per column)
     constexpr uint32_t kChunk = 4096;
-    rc = ensure_limbs(db, limb_bytes(db, std::min(B, kChunk)));
+    rc = ensure_limbs(db, limb_workspace_bytes(std::min(B, kChunk), db->pitch));
     if (rc != QPADL_OK) return rc;
     const uint64_t C = db->prm.cols, R = db->prm.rows;
     for (uint32_t b0 = 0; b0 < B; b0 += kChunk) {
         const uint32_t Bc = std::min(B - b0, kChunk);
-        rc = answer_f16(db, Q + (uint64_t)b0 * C, Bc, ans + (uint64_t)b0 * R, db->limbs, use_tri(db), true, stream);
+        rc = answer_f16(db, Q + (uint64_t)b0 * C, Bc, ans + (uint64_t)b0 * R, db->limbs, use_tri(db), stream);
         if (rc != QPADL_OK) return rc;
     }
     return QPADL_OK;
@@ -561,7 +558,7 @@ int db_answer_f16_ws(qpadl_db *db, const uint32_t *Q, uint32_t B, uint32_t *ans,
     // the copy that was prepared, even if the handle's tile option has changed since
     const bool tri = db->d16c && (use_tri(db) || !db->d16);
     if (!tri && !db->d16) return QPADL_EINVAL;
-    return answer_f16(db, Q, B, ans, limbs, tri, false, stream);   // the workspace has no room for the sums of four
+    return answer_f16(db, Q, B, ans, limbs, tri, stream);
 }
 
 int db_answer_one_noscratch(qpadl_db *db, const uint32_t *q, uint32_t *ans, cudaStream_t stream) {
@@ -757,7 +754,7 @@ int qpadl_pir_reserve(qpadl_db *db, uint32_t max_batch, qpadl_stream_t stream) {
             if (rc != QPADL_OK) return rc;
         }
         // the batched paths work in chunks of at most 4096 queries
-        int rc = ensure_limbs(db, limb_bytes(db, std::min<uint32_t>(max_batch, 4096u)));
+        int rc = ensure_limbs(db, limb_workspace_bytes(std::min<uint32_t>(max_batch, 4096u), db->pitch));
         if (rc != QPADL_OK) return rc;
     }
     QPADL_CU(cudaStreamSynchronize(s));

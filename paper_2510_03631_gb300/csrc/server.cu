@@ -252,10 +252,13 @@ namespace {
 constexpr uint64_t align256(uint64_t x) { return (x + 255) & ~255ull; }
 constexpr size_t kMaxGemmLaunches = 2;   // launches in flight at once while a GEMM is among them
 
-// Device workspace of one group of `take` requests: queries, answers and the byte limbs of the
-// queries (any group can join a grouped GEMM).
+// Device workspace of one group of `take` requests: queries, answers and the limbs of the
+// queries (any group can join a grouped GEMM, or run alone on either fp16 GEMM).
+uint64_t limb_part(const DbEntry &e, uint32_t take) {
+    return align256(qpadl::limb_workspace_bytes(take, e.pitch));
+}
 uint64_t group_bytes(const DbEntry &e, uint32_t take) {
-    return align256(4ull * take * e.C) + align256(4ull * take * e.R) + align256(8ull * take * e.pitch);
+    return align256(4ull * take * e.C) + align256(4ull * take * e.R) + limb_part(e, take);
 }
 }  // namespace
 
@@ -294,7 +297,7 @@ bool qpadl_server::form_launch(int si, std::unique_lock<std::mutex> &lk) {
         g.da_off = need;
         need += align256(4ull * take * e.R);
         g.dl_off = need;
-        need += align256(8ull * take * e.pitch);
+        need += limb_part(e, take);
         total += take;
         groups.push_back(g);
     }

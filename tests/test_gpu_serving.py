@@ -143,6 +143,33 @@ def test_group_above_the_uint8_gemm_limit_takes_the_fp16_copy(dbs):
         pir.qpadl_pir_set_option(h1, pir.QPADL_OPT_U8_MAX_BATCH, 64)
 
 
+@pytest.mark.parametrize("d,count", [(0, 150), (1, 192), (2, 129), (0, 3)])
+@pytest.mark.parametrize("pair", [1, 0])
+def test_group_of_an_odd_number_of_64_query_halves(dbs, d, count, pair):
+    # one launch of 129-192 queries on the fp16 copy, where four byte limbs and a sum per query can be the
+    # faster form: the workspace of a group has room for them (the smallest group on the copy too)
+    D, h = dbs[d]
+    pir.qpadl_pir_set_option(h, pir.QPADL_OPT_PAIR_GEMM, pair)
+    pir.qpadl_pir_set_option(h, pir.QPADL_OPT_U8_MAX_BATCH, 2)
+    try:
+        srv = pir.qpadl_server_create(pir.server_config(max_batch=256, num_streams=1, max_inflight=512,
+                                                        host_budget_bytes=64 << 20))
+        db_id = pir.qpadl_server_add_db(srv, h)
+        Q = inputs.uniform_u32(count * SHAPES[d][1], seed=count + d, tag=inputs.TAG_MISC).reshape(count, -1)
+        tickets = [pir.qpadl_server_submit(srv, db_id, q) for q in Q]
+        pir.qpadl_server_start(srv)
+        exp = oracle.answer_batch(D, Q, threads=oracle.max_threads())
+        for b, t in enumerate(tickets):
+            rc, ans, _ = _wait(srv, t, SHAPES[d][0])
+            assert rc == pir.QPADL_OK and np.array_equal(ans, exp[b])
+        st = pir.qpadl_server_stats(srv)
+        assert st["launches"] == 1 and st["gemm_kernels"] == 1
+        srv.close()
+    finally:
+        pir.qpadl_pir_set_option(h, pir.QPADL_OPT_U8_MAX_BATCH, 64)
+        pir.qpadl_pir_set_option(h, pir.QPADL_OPT_PAIR_GEMM, 1)
+
+
 @pytest.mark.parametrize("ratio,grouped", [(0.0, False), (1.5, False), (2.5, True)])
 def test_group_size_ratio(dbs, ratio, grouped):
     # sizes R*C: 0.5M, 2M and 1.24M words; with ratio 2.5 databases 1 and 2 share a launch
