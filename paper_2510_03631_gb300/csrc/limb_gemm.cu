@@ -5,12 +5,15 @@
 // q-bar queries against one database) and for the offline hint
 // H = D * A (X = columns of A; Sec. 5.3 offline precomputation).
 //
+// The matrix holds the digits minus 128 (one fp16 copy serves these tiles and the
+// CTA-pair ones); 128 times a vector's sum, made with its limbs, is added at the end.
+//
 // Exactness.  Each X word is split into four balanced byte limbs
 // x = sum_k 2^{8k} c_k with c_k in [-128, 127] (low byte, minus 256 and a
 // carry when >= 128; the last carry is a multiple of 2^32 and is dropped).
-// Digits d in [0, 255] and limbs are small integers, exactly representable
-// in fp16, and every product d*c is an integer of magnitude <= 32640.  A run
-// of 512 such products sums to less than 2^24 in magnitude, so the fp32
+// Centred digits, field digits (0..255) and limbs are small integers, exactly
+// representable in fp16, and every product is an integer of magnitude <= 32640.  A
+// run of 512 such products sums to less than 2^24 in magnitude, so the fp32
 // tensor-core accumulator holds every partial sum of a 512-deep K-chunk
 // exactly.  After each chunk the epilogue converts the four limb sums to
 // int32 (exact), recombines them as sum_k 2^{8k} s_k in uint32 arithmetic
@@ -454,7 +457,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                     // part of a split tile: exact, since addition mod 2^32 commutes
 #pragma unroll
                     for (int q = 0; q < QPT; ++q)
-                        if (v0 + q < NV) epi.add(row, v0 + q, run[q]);
+                        if (v0 + q < NV)   // the first piece of a tile adds what centred digits leave out
+                            epi.add(row, v0 + q, run[q] + (pc.c0 == 0 ? epi.pre(row, v0 + q) : 0u));
                     continue;
                 }
             }
@@ -815,10 +819,10 @@ static cudaError_t launch_epi(int bn, const CUtensorMap &a_map, const CUtensorMa
     }
 }
 
-cudaError_t launch_limb_gemm(int bn, const CUtensorMap &a_map, const CUtensorMap &b_map, uint32_t *out,
-                             uint64_t ld_m, uint64_t ld_b, uint32_t M, uint32_t NV, uint64_t K, int num_sms,
-                             int *status, cudaStream_t stream) {
-    return launch_epi(bn, a_map, b_map, StoreEpi{out, ld_m, ld_b, nullptr, 0u}, M, NV, K, 0, num_sms, status, stream);
+cudaError_t launch_limb_gemm(int bn, const CUtensorMap &a_map, const CUtensorMap &b_map, const uint32_t *sums,
+                             uint32_t centre, uint32_t *out, uint64_t ld_m, uint64_t ld_b, uint32_t M, uint32_t NV,
+                             uint64_t K, int num_sms, int *status, cudaStream_t stream) {
+    return launch_epi(bn, a_map, b_map, StoreEpi{out, ld_m, ld_b, sums, centre}, M, NV, K, 0, num_sms, status, stream);
 }
 
 cudaError_t launch_limb_gemm_query(int bn, const CUtensorMap &a_map, const CUtensorMap &b_map, const QueryNoiseEpi &epi,

@@ -528,9 +528,10 @@ __global__ void __launch_bounds__(512, 2) vec_limbs_sums_kernel(const uint32_t *
 
 // A (uint32, C x n row-major): block (x, y) turns rows [128 x, 128 x + 128) x columns [32 y, 32 y + 32)
 // through shared memory; 16 threads write one column's 128 limbs, 16 bytes each.
-__global__ void __launch_bounds__(256) mat_col_limbs_tri_kernel(const uint32_t *__restrict__ A, uint64_t C, uint32_t n,
-                                                                __half *__restrict__ L, uint64_t pitch,
-                                                                uint32_t *__restrict__ sums) {
+template <int LIMBS>
+__global__ void __launch_bounds__(256) mat_col_limbs_sums_kernel(const uint32_t *__restrict__ A, uint64_t C, uint32_t n,
+                                                                 __half *__restrict__ L, uint64_t pitch,
+                                                                 uint32_t *__restrict__ sums) {
     griddep_launch_dependents();   // as in vec_limbs_sums_kernel
     __shared__ uint32_t tile[128][33];
     const uint64_t j0 = (uint64_t)blockIdx.x * 128;
@@ -547,14 +548,15 @@ __global__ void __launch_bounds__(256) mat_col_limbs_tri_kernel(const uint32_t *
     const bool aligned = (reinterpret_cast<uintptr_t>(L) & 15u) == 0;
     for (uint32_t kk = threadIdx.x >> 4; kk < 32; kk += 16) {
         const uint32_t k = k0 + kk;
-        int l[3][8];
+        int l[LIMBS][8];
         uint32_t sum = 0;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const uint32_t x = tile[8 * t + i][kk];
-            int u[3];
+            int u[LIMBS];
             balanced(x, u);
-            l[0][i] = u[0], l[1][i] = u[1], l[2][i] = u[2];
+#pragma unroll
+            for (int m = 0; m < LIMBS; ++m) l[m][i] = u[m];
             sum += x;
         }
 #pragma unroll
@@ -562,9 +564,9 @@ __global__ void __launch_bounds__(256) mat_col_limbs_tri_kernel(const uint32_t *
         if (k >= n) continue;
         if (t == 0) atomicAdd(sums + k, sum);
         const uint64_t j = j0 + 8 * t;
-        __half *dst = L + 3ull * k * pitch + j;
+        __half *dst = L + (uint64_t)LIMBS * k * pitch + j;
 #pragma unroll
-        for (int u = 0; u < 3; ++u) {
+        for (int u = 0; u < LIMBS; ++u) {
             if (aligned && j + 8 <= C) {
                 store8(dst + u * pitch, l[u]);
             } else {
@@ -602,21 +604,34 @@ cudaError_t launch_vec_limbs_tri(const uint32_t *X, uint64_t x_ld, uint32_t NV, 
     return launch_vec_limbs_sums<3>(X, x_ld, NV, C, L, pitch, tri_sums(L, NV, pitch), zero, zero_words, stream);
 }
 
+static uint32_t *four_sums(__half *L, uint32_t nv, uint64_t pitch) {
+    return reinterpret_cast<uint32_t *>(reinterpret_cast<uint8_t *>(L) + four_sums_offset(nv, pitch));
+}
+
 cudaError_t launch_vec_limbs_four(const uint32_t *X, uint64_t x_ld, uint32_t NV, uint64_t C, __half *L, uint64_t pitch,
                                   cudaStream_t stream) {
-    uint32_t *sums = reinterpret_cast<uint32_t *>(reinterpret_cast<uint8_t *>(L) + four_sums_offset(NV, pitch));
-    return launch_vec_limbs_sums<4>(X, x_ld, NV, C, L, pitch, sums, nullptr, 0, stream);
+    return launch_vec_limbs_sums<4>(X, x_ld, NV, C, L, pitch, four_sums(L, NV, pitch), nullptr, 0, stream);
+}
+
+template <int LIMBS>
+static cudaError_t launch_mat_col_limbs_sums(const uint32_t *A, uint64_t C, uint32_t n, __half *L, uint64_t pitch,
+                                             uint32_t *sums, cudaStream_t stream) {
+    if (n == 0 || C == 0 || pitch % 8 != 0) return cudaErrorInvalidValue;
+    const cudaError_t e = cudaMemsetAsync(sums, 0, 4ull * n, stream);
+    if (e != cudaSuccess) return e;
+    const dim3 grid(static_cast<unsigned>((C + 127) / 128), (n + 31) / 32);
+    mat_col_limbs_sums_kernel<LIMBS><<<grid, 256, 0, stream>>>(A, C, n, L, pitch, sums);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_mat_col_limbs_tri(const uint32_t *A, uint64_t C, uint32_t n, __half *L, uint64_t pitch,
                                      cudaStream_t stream) {
-    if (n == 0 || C == 0 || pitch % 8 != 0) return cudaErrorInvalidValue;
-    uint32_t *sums = tri_sums(L, n, pitch);
-    const cudaError_t e = cudaMemsetAsync(sums, 0, 4ull * n, stream);
-    if (e != cudaSuccess) return e;
-    const dim3 grid(static_cast<unsigned>((C + 127) / 128), (n + 31) / 32);
-    mat_col_limbs_tri_kernel<<<grid, 256, 0, stream>>>(A, C, n, L, pitch, sums);
-    return cudaGetLastError();
+    return launch_mat_col_limbs_sums<3>(A, C, n, L, pitch, tri_sums(L, n, pitch), stream);
+}
+
+cudaError_t launch_mat_col_limbs_four(const uint32_t *A, uint64_t C, uint32_t n, __half *L, uint64_t pitch,
+                                      cudaStream_t stream) {
+    return launch_mat_col_limbs_sums<4>(A, C, n, L, pitch, four_sums(L, n, pitch), stream);
 }
 
 cudaError_t prepare_limb_gemm_tri_kernels() {

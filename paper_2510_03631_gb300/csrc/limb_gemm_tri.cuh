@@ -16,8 +16,8 @@ constexpr uint32_t kTriGroup = 32;
 // Never more than the 8 NV pitch bytes of the four-limb layout.
 inline uint64_t tri_sums_offset(uint32_t nv, uint64_t pitch) { return 6ull * nv * pitch; }
 
-// The same with four byte limbs (limb k of vector v in row 4 v + k) for limb_gemm_pair.cu; the sums lie
-// 8 NV pitch bytes on.
+// The same with four byte limbs (limb k of vector v in row 4 v + k) for limb_gemm_pair.cu and limb_gemm.cu; the
+// sums lie 8 NV pitch bytes on.
 inline uint64_t four_sums_offset(uint32_t nv, uint64_t pitch) { return 8ull * nv * pitch; }
 
 cudaError_t prepare_limb_gemm_tri_kernels();
@@ -29,9 +29,11 @@ cudaError_t launch_vec_limbs_tri(const uint32_t *X, uint64_t x_ld, uint32_t NV, 
                                  uint32_t *zero, uint64_t zero_words, cudaStream_t stream);
 cudaError_t launch_vec_limbs_four(const uint32_t *X, uint64_t x_ld, uint32_t NV, uint64_t C, __half *L, uint64_t pitch,
                                   cudaStream_t stream);
-// The three limbs of the columns of A (C x n row-major): vector k is column k.
+// The three limbs, or four, of the columns of A (C x n row-major): vector k is column k.
 cudaError_t launch_mat_col_limbs_tri(const uint32_t *A, uint64_t C, uint32_t n, __half *L, uint64_t pitch,
                                      cudaStream_t stream);
+cudaError_t launch_mat_col_limbs_four(const uint32_t *A, uint64_t C, uint32_t n, __half *L, uint64_t pitch,
+                                      cudaStream_t stream);
 
 // The time of the launch below in the time of one half (256 rows x 64 vectors).
 double limb_gemm_tri_waves(uint32_t M, uint32_t NV, uint64_t K, int num_sms);

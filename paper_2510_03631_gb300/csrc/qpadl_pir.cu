@@ -51,8 +51,8 @@ struct qpadl_db {
     uint32_t u8_max_batch = 64;      // QPADL_OPT_U8_MAX_BATCH
     int u8_kstep = 0;                // QPADL_OPT_U8_KSTEP (0 = per tile width default)
     int pair_gemm = 1;               // QPADL_OPT_PAIR_GEMM
-    __half *d16 = nullptr;           // digits as fp16, R x pitch (single-SM tiles, Z_p)
-    __half *d16c = nullptr;          // digits minus 128 as fp16, R x pitch (three-limb pair tiles)
+    __half *d16 = nullptr;           // digits as fp16, R x pitch (Z_p handles)
+    __half *d16c = nullptr;          // digits minus 128 as fp16, R x pitch (lattice handles, either tile form)
     uint64_t pitch = 0;              // roundup(C, 8)
     CUtensorMap a_map, ac_map;       // over d16, d16c
     __half *limbs = nullptr;         // limb scratch
@@ -244,17 +244,17 @@ int build_f16_copy(qpadl_db *db, __half **copy, CUtensorMap *map, int centre, cu
     return QPADL_OK;
 }
 
-int ensure_tensor_copy(qpadl_db *db, cudaStream_t stream) {
+int ensure_field_copy(qpadl_db *db, cudaStream_t stream) {
     return build_f16_copy(db, &db->d16, &db->a_map, 0, stream);
 }
 
 // Whether batches beyond the uint8-digit GEMM run on three-limb pair tiles (else on single SMs).
 bool use_tri(const qpadl_db *db) { return db->pair_gemm && db->num_sms >= 2; }
 
-// The fp16 copy that batches of this handle read.
+// The fp16 copy that batches and hints of a lattice handle read, whatever its tile option says: a change
+// of the option after qpadl_pir_reserve builds nothing.
 int ensure_batch_copy(qpadl_db *db, cudaStream_t stream) {
-    return use_tri(db) ? build_f16_copy(db, &db->d16c, &db->ac_map, kTriCentre, stream)
-                       : ensure_tensor_copy(db, stream);
+    return build_f16_copy(db, &db->d16c, &db->ac_map, kTriCentre, stream);
 }
 
 int ensure_limbs(qpadl_db *db, uint64_t bytes) {
@@ -279,9 +279,8 @@ int set_device(const qpadl_db *db) {
     return QPADL_OK;
 }
 
-// out[i * ld_m + v * ld_b] = D * X[v] for NV vectors given as limbs at `limbs`: three limbs and the
-// vectors' sums (launch_vec_limbs_tri) for pair tiles over d16c, or (run_limb_gemm) four, 4 NV rows of
-// db->pitch elements, for single-SM tiles over d16
+// out[i * ld_m + v * ld_b] = D * X[v] for NV vectors given at `limbs` as three limbs (pair tiles) or, in
+// run_limb_gemm, four (single-SM tiles) and the vectors' sums
 int run_tri_gemm(qpadl_db *db, const __half *limbs, uint32_t NV, uint32_t *out, uint64_t ld_m, uint64_t ld_b,
                  uint32_t ranges, cudaStream_t stream) {
     const uint64_t C = db->prm.cols;
@@ -309,10 +308,15 @@ int run_limb_gemm(qpadl_db *db, const __half *limbs, uint32_t NV, uint32_t *out,
     if (!encode_2d(&b_map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, limbs, db->prm.cols, 4ull * NV, db->pitch * 2,
                    kLimbBoxK, static_cast<uint32_t>(bn), CU_TENSOR_MAP_SWIZZLE_128B))
         return QPADL_ECUDA;
-    QPADL_CU(launch_limb_gemm(bn, db->a_map, b_map, out, ld_m, ld_b, static_cast<uint32_t>(db->prm.rows), NV,
-                              db->prm.cols, db->num_sms, db->d_status, stream));
+    const uint32_t *sums = reinterpret_cast<const uint32_t *>(reinterpret_cast<const uint8_t *>(limbs) +
+                                                              four_sums_offset(NV, db->pitch));
+    QPADL_CU(launch_limb_gemm(bn, db->ac_map, b_map, sums, kTriCentre, out, ld_m, ld_b,
+                              static_cast<uint32_t>(db->prm.rows), NV, db->prm.cols, db->num_sms, db->d_status, stream));
     return QPADL_OK;
 }
+
+// Limb scratch of NV vectors on the handle: four limbs and a word each.
+uint64_t limb_scratch_bytes(const qpadl_db *db, uint32_t NV) { return 8ull * NV * db->pitch + 4ull * NV; }
 
 // Whether a batch on pair tiles takes four byte limbs instead of three: only with an odd number of
 // 64-vector halves, where the three-limb tiles (two halves, or three for 3 and 5) leave a half empty
@@ -328,11 +332,11 @@ bool four_limbs(const qpadl_db *db, uint32_t B) {
     return four < three;
 }
 
-// Answers of B queries (at most 4096) on an fp16 copy that exists, their limbs made at `limbs`
-// (limb_workspace_bytes).
-int answer_f16(qpadl_db *db, const uint32_t *Q, uint32_t B, uint32_t *ans, __half *limbs, bool tri,
-               cudaStream_t stream) {
+// Answers of B queries (at most 4096) on the fp16 copy, which exists, their limbs made at `limbs`
+// (limb_workspace_bytes; single-SM tiles need a word more per query for B <= 2).
+int answer_f16(qpadl_db *db, const uint32_t *Q, uint32_t B, uint32_t *ans, __half *limbs, cudaStream_t stream) {
     const uint64_t C = db->prm.cols, R = db->prm.rows;
+    const bool tri = use_tri(db);
     if (tri && four_limbs(db, B)) {
         QPADL_CU(launch_vec_limbs_four(Q, C, B, C, limbs, db->pitch, stream));
         PairBMaps bm;
@@ -352,7 +356,7 @@ int answer_f16(qpadl_db *db, const uint32_t *Q, uint32_t B, uint32_t *ans, __hal
         QPADL_CU(launch_vec_limbs_tri(Q, C, B, C, limbs, db->pitch, ranges > 1 ? ans : nullptr, (uint64_t)B * R, stream));
         return run_tri_gemm(db, limbs, B, ans, 1, R, ranges, stream);
     }
-    QPADL_CU(launch_vec_limbs(Q, C, B, C, limbs, db->pitch, db->num_sms, stream));
+    QPADL_CU(launch_vec_limbs_four(Q, C, B, C, limbs, db->pitch, stream));
     return run_limb_gemm(db, limbs, B, ans, 1, R, stream);
 }
 
@@ -508,12 +512,12 @@ int answer_tensor(qpadl_db *db, const uint32_t *Q, uint32_t B, uint32_t *ans, cu
     if (rc != QPADL_OK) return rc;
     // chunks of at most 4096 queries bound the limb scratch (8 bytes per query per column)
     constexpr uint32_t kChunk = 4096;
-    rc = ensure_limbs(db, limb_workspace_bytes(std::min(B, kChunk), db->pitch));
+    rc = ensure_limbs(db, limb_scratch_bytes(db, std::min(B, kChunk)));
     if (rc != QPADL_OK) return rc;
     const uint64_t C = db->prm.cols, R = db->prm.rows;
     for (uint32_t b0 = 0; b0 < B; b0 += kChunk) {
         const uint32_t Bc = std::min(B - b0, kChunk);
-        rc = answer_f16(db, Q + (uint64_t)b0 * C, Bc, ans + (uint64_t)b0 * R, db->limbs, use_tri(db), stream);
+        rc = answer_f16(db, Q + (uint64_t)b0 * C, Bc, ans + (uint64_t)b0 * R, db->limbs, stream);
         if (rc != QPADL_OK) return rc;
     }
     return QPADL_OK;
@@ -555,10 +559,12 @@ int db_fill_u8_group(qpadl_db *db, GroupedGemmArgs &args, int g, const __half *l
 
 int db_answer_f16_ws(qpadl_db *db, const uint32_t *Q, uint32_t B, uint32_t *ans, __half *limbs,
                      cudaStream_t stream) {
-    // the copy that was prepared, even if the handle's tile option has changed since
-    const bool tri = db->d16c && (use_tri(db) || !db->d16);
-    if (!tri && !db->d16) return QPADL_EINVAL;
-    return answer_f16(db, Q, B, ans, limbs, tri, stream);
+    if (!db->d16c) return QPADL_EINVAL;
+    if (B <= 2 && !use_tri(db)) {   // no room for sums: the streaming kernel, which needs no workspace
+        const uint64_t C = db->prm.cols, R = db->prm.rows;
+        return B == 1 ? db_answer_one_noscratch(db, Q, ans, stream) : db_answer_two_noscratch(db, Q, C, ans, R, stream);
+    }
+    return answer_f16(db, Q, B, ans, limbs, stream);
 }
 
 int db_answer_one_noscratch(qpadl_db *db, const uint32_t *q, uint32_t *ans, cudaStream_t stream) {
@@ -754,7 +760,7 @@ int qpadl_pir_reserve(qpadl_db *db, uint32_t max_batch, qpadl_stream_t stream) {
             if (rc != QPADL_OK) return rc;
         }
         // the batched paths work in chunks of at most 4096 queries
-        int rc = ensure_limbs(db, limb_workspace_bytes(std::min<uint32_t>(max_batch, 4096u), db->pitch));
+        int rc = ensure_limbs(db, limb_scratch_bytes(db, std::min<uint32_t>(max_batch, 4096u)));
         if (rc != QPADL_OK) return rc;
     }
     QPADL_CU(cudaStreamSynchronize(s));
@@ -780,7 +786,7 @@ int qpadl_pir_hint(qpadl_db *db, const uint32_t *A_dev, uint32_t *H_dev, qpadl_s
     const bool u8 = db->u8_ok && n <= db->u8_max_batch;   // the lean layout keeps no fp16 copy
     int rc = u8 ? ensure_blocked(db, s) : ensure_batch_copy(db, s);
     if (rc != QPADL_OK) return rc;
-    rc = ensure_limbs(db, 8ull * n * db->pitch);
+    rc = ensure_limbs(db, limb_scratch_bytes(db, n));
     if (rc != QPADL_OK) return rc;
     if (!u8 && use_tri(db)) {
         const uint64_t R = db->prm.rows;
@@ -789,8 +795,12 @@ int qpadl_pir_hint(qpadl_db *db, const uint32_t *A_dev, uint32_t *H_dev, qpadl_s
         QPADL_CU(launch_mat_col_limbs_tri(A_dev, db->prm.cols, n, db->limbs, db->pitch, s));
         return run_tri_gemm(db, db->limbs, n, H_dev, n, 1, ranges, s);
     }
+    if (!u8) {
+        QPADL_CU(launch_mat_col_limbs_four(A_dev, db->prm.cols, n, db->limbs, db->pitch, s));
+        return run_limb_gemm(db, db->limbs, n, H_dev, n, 1, s);
+    }
     QPADL_CU(launch_mat_col_limbs(A_dev, db->prm.cols, n, db->limbs, db->pitch, s));
-    return u8 ? run_u8_gemm(db, n, H_dev, n, 1, s) : run_limb_gemm(db, db->limbs, n, H_dev, n, 1, s);
+    return run_u8_gemm(db, n, H_dev, n, 1, s);
 }
 
 int qpadl_pir_query(const qpadl_params *prm, const uint32_t *A_dev, const uint32_t *s_dev, const int32_t *e_dev,
@@ -1521,7 +1531,7 @@ int qpadl_goldberg_answer_batch(qpadl_goldberg *h, const uint32_t *Q_dev, uint32
         QPADL_CU(launch_mod_p_signed(out_dev, (uint64_t)B * R, h->p, db->num_sms, s));
         return QPADL_OK;
     }
-    int rc = ensure_tensor_copy(db, s);
+    int rc = ensure_field_copy(db, s);
     if (rc != QPADL_OK) return rc;
     // one centred fp16 row per query, in chunks that the limb scratch holds
     constexpr uint32_t kChunk = 1024;
