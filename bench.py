@@ -479,7 +479,8 @@ def chor_measure(torch, pir, inputs, seed=31):
         alg = rows * W * 4 + B * ((rows + 31) // 32) * 4 + B * W * 4
         ent = {"ms": round(ms, 4), "queries_per_s": round(qps, 1),
                "db_scan_gbs": round(B * rows * W * 4 / (ms * 1e-3) / 1e9, 1),
-               "kernel": "tensor cores (mxf4)" if B >= 9 else "masked-XOR scan"}
+               "kernel": "tensor cores (mxf4)" if B >= pir.qpadl_chor_get_option(h, pir.QPADL_CHOR_OPT_M4RM_MIN_BATCH)
+               else "masked-XOR scan"}
         if one_qps:
             ent["x_vs_one_at_a_time"] = round(qps / one_qps, 2)
         if B == 1:

@@ -120,6 +120,11 @@ constexpr uint64_t kRawCells = 16ull << 20, kRawCells2 = 4ull << 20, kRawCols = 
 // words (60,000 rows) 41 / 26 us at one query; 768 words (2^18 rows) 148 / 187 us at one, 159 / 189
 // at 2, 195 / 189 at 3; 8192 words (32,768 rows) 241 / 251 at 8 and 356 / 251 at 9.
 uint32_t chor_large_batch(uint32_t W) { return W < 512 ? 1u : (W < 1024 ? 3u : 9u); }
+// Whether the caller's threshold applies (choosing a scan form asks for the scan below it), and the one in force.
+bool chor_min_batch_set(const qpadl_chor *h) { return h->large_set || h->scan_form >= 0; }
+uint32_t chor_min_batch(const qpadl_chor *h) {
+    return chor_min_batch_set(h) ? h->large_min_batch : chor_large_batch(h->words);
+}
 uint32_t chor_units(uint64_t rows) { return static_cast<uint32_t>((rows + kChorGemmUnitRows - 1) / kChorGemmUnitRows); }
 // Goldberg sums stay exact (|centred sum| < 2^31, unsigned sum < 2^32) below this many columns
 constexpr uint64_t kGoldbergMaxCols = 65792;
@@ -1366,11 +1371,17 @@ int qpadl_chor_answer_batch(qpadl_chor *h, const uint32_t *Q_dev, uint32_t B, ui
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const uint64_t W = h->words;
     QPADL_CU(cudaMemsetAsync(out_dev, 0, 4ull * W * B, s));
-    const uint32_t large = h->large_set || h->scan_form >= 0 ? h->large_min_batch : chor_large_batch(h->words);
-    for (uint32_t b0 = 0, Bc; b0 < B; b0 += Bc) {
-        Bc = std::min(B - b0, kChorMaxBatch);
-        if (Bc >= large) {
-            Bc = std::min(Bc, kChorGemmMaxBatch);
+    const uint32_t large = chor_min_batch(h);
+    for (uint32_t b0 = 0, Bc, left = 0; b0 < B; b0 += Bc) {
+        // a threshold set by the caller decides for a chunk of 256 as a whole (`left`: what remains of one that the
+        // tensor cores take); the library's own also for what is left of it after the first 128
+        if (left == 0 || !chor_min_batch_set(h)) {
+            Bc = std::min(B - b0, kChorMaxBatch);
+            left = Bc >= large ? Bc : 0;
+        }
+        if (left) {
+            Bc = std::min(left, kChorGemmMaxBatch);
+            left -= Bc;
             int rc = chor_answer_gemm(h, Q_dev + (uint64_t)b0 * h->qw, Bc, out_dev + (uint64_t)b0 * W, s);
             if (rc != QPADL_OK) return rc;
             continue;
@@ -1412,7 +1423,7 @@ int qpadl_chor_set_option(qpadl_chor *h, int option, int64_t value) {
 int qpadl_chor_get_option(qpadl_chor *h, int option, int64_t *value) {
     if (!h || !value) return QPADL_EINVAL;
     switch (option) {
-        case QPADL_CHOR_OPT_M4RM_MIN_BATCH: *value = h->large_min_batch; return QPADL_OK;
+        case QPADL_CHOR_OPT_M4RM_MIN_BATCH: *value = chor_min_batch(h); return QPADL_OK;
         case QPADL_CHOR_OPT_SCAN_FORM: *value = h->scan_form; return QPADL_OK;
         default: return QPADL_EINVAL;
     }

@@ -52,3 +52,22 @@ def test_largest_counts(rows, B):
 def test_default_choice(bits, B):
     rows = 300
     _check(rows, bits, B, inputs.chor_db(rows, bits, seed=bits), inputs.chor_queries(B, rows, seed=B), None)
+
+
+@pytest.mark.parametrize("min_batch,B", [(129, 128), (200, 199), (200, 256), (200, 330), (256, 256), (3, 258)])
+def test_threshold_decides_for_chunks_of_256(min_batch, B):
+    rows, bits = 700, 2048
+    _check(rows, bits, B, inputs.chor_db(rows, bits, seed=B), inputs.chor_queries(B, rows, seed=min_batch), min_batch)
+
+
+def test_option_reads_as_the_threshold_in_force():
+    for bits, own in ((128, 1), (511 * 32 // 128 * 128, 1), (512 * 32, 3), (1023 * 32 // 128 * 128, 3), (1024 * 32, 9)):
+        h = pir.qpadl_chor_setup(64, bits, _dev(np.zeros((64, bits // 32))))
+        opt = lambda: pir.qpadl_chor_get_option(h, pir.QPADL_CHOR_OPT_M4RM_MIN_BATCH)
+        assert opt() == own
+        pir.qpadl_chor_set_option(h, pir.QPADL_CHOR_OPT_SCAN_FORM, 1)
+        assert opt() == 48
+        pir.qpadl_chor_set_option(h, pir.QPADL_CHOR_OPT_SCAN_FORM, -1)
+        pir.qpadl_chor_set_option(h, pir.QPADL_CHOR_OPT_M4RM_MIN_BATCH, 200)
+        assert opt() == 200
+        h.close()
