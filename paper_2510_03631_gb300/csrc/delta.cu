@@ -18,7 +18,8 @@
 //                        load over the entries in order, a CTA max, one atomic max
 //   delta_encode_kernel  a CTA per 128 blocks x 128 positions: four entries of four
 //                        blocks per thread, packed into row words in registers and
-//                        turned through shared memory into 128-byte row segments
+//                        turned through shared memory into 128-byte row segments;
+//                        blocks of up to 80 entries are staged whole instead
 //   delta_decode_kernel  one CTA per recovered block: eight entries per thread,
 //                        a CTA-wide scan of their sums, 16-byte stores
 #include <cstdint>
@@ -193,6 +194,59 @@ __global__ void __launch_bounds__(kEncThreads) delta_encode_kernel(const uint32_
     }
 }
 
+// The same for blocks of up to 80 entries, of which the tile above would be mostly positions past the block's
+// end: a CTA stages its 128 blocks whole (one contiguous run of 128 E entries) and writes their rows.  Bound by
+// the row stores.  2^24 entries, one byte, blocks of 2 / 5 / 16 / 33 / 64 / 80 entries: 84 / 47 / 31 / 41 / 27 /
+// 26 us, in 128 x 128 tiles 969 / 399 / 132 / 73 / 41 / 35; 81 entries 37 in tiles, 90 entries 41 staged, 35 in tiles.
+constexpr uint32_t kShortEntries = 80;
+__global__ void __launch_bounds__(kEncThreads) delta_encode_short_kernel(const uint32_t *__restrict__ x, uint64_t n,
+                                                                         uint32_t E, uint32_t w, uint64_t C,
+                                                                         uint8_t *__restrict__ db) {
+    extern __shared__ uint32_t ent[];   // [kEncCols][ld]; an odd stride puts neighbouring columns in distinct banks
+    const uint32_t ld = E | 1u;
+    const uint64_t j0 = (uint64_t)blockIdx.x * kEncCols;
+    const uint32_t ncols = static_cast<uint32_t>(C - j0 < (uint64_t)kEncCols ? C - j0 : (uint64_t)kEncCols);
+    const uint64_t k0 = j0 * E;
+    if (k0 + (uint64_t)ncols * E <= n) {   // one check: the loads do not wait for one another
+#pragma unroll 4
+        for (uint32_t f = threadIdx.x; f < ncols * E; f += kEncThreads) {
+            const uint32_t c = f / E;
+            ent[c * ld + f - c * E] = x[k0 + f];
+        }
+    } else {
+        for (uint32_t f = threadIdx.x; f < ncols * E; f += kEncThreads) {
+            const uint32_t c = f / E;
+            ent[c * ld + f - c * E] = entry_at(x, n, k0 + f);
+        }
+    }
+    __syncthreads();
+    // row r < 4: byte r of the first entries; row 4 + (i - 1) w + b: byte b of the differences at position i
+    const uint32_t rows = (E - 1) * w;
+    uint8_t *diffs = db + 4 * C + j0;
+    db += j0;
+    if (C % 4 == 0 && (reinterpret_cast<uintptr_t>(db) & 3u) == 0) {   // four columns in one store
+        constexpr uint32_t kQuads = kEncCols / 4;
+        for (uint32_t t = threadIdx.x; t < rows * kQuads; t += kEncThreads) {
+            const uint32_t r = t / kQuads, c = 4 * (t % kQuads);
+            if (c >= ncols) continue;   // C % 4 == 0: whole quads
+            const uint32_t i = r / w, sh = 8u * (r - i * w);
+            uint32_t v = 0;
+#pragma unroll
+            for (uint32_t k = 0; k < 4; ++k) v |= (((ent[(c + k) * ld + i + 1] - ent[(c + k) * ld + i]) >> sh) & 255u) << (8u * k);
+            *reinterpret_cast<uint32_t *>(diffs + r * C + c) = v;
+        }
+    } else {
+        for (uint32_t t = threadIdx.x; t < rows * kEncCols; t += kEncThreads) {
+            const uint32_t r = t / kEncCols, c = t % kEncCols, i = r / w;
+            if (c < ncols) diffs[r * C + c] = static_cast<uint8_t>((ent[c * ld + i + 1] - ent[c * ld + i]) >> (8u * (r - i * w)));
+        }
+    }
+    for (uint32_t t = threadIdx.x; t < 4 * kEncCols; t += kEncThreads) {   // the first entry of each block in full
+        const uint32_t r = t / kEncCols, c = t % kEncCols;
+        if (c < ncols) db[r * C + c] = static_cast<uint8_t>(ent[c * ld] >> (8u * r));
+    }
+}
+
 // Block b: digits b * Rp .. (4-byte first entry, then E - 1 differences of W bytes) -> out b * E ..
 // Thread t takes positions 8 t .. 8 t + 7 of a run of 8192 (its digits are independent loads of
 // adjacent bytes), a two-level shuffle scan gives the sum before them, and the runs of a longer
@@ -317,6 +371,11 @@ int qpadl_pir_delta_encode(const uint32_t *entries_dev, uint64_t n, uint32_t E, 
     if (!entries_dev || !db_dev || !delta_shape_ok(n, E, w)) return QPADL_EINVAL;
     const uint64_t C = (n + E - 1) / E;
     if (E > kMaxEncodeEntries) return QPADL_EINVAL;
+    if (E <= kShortEntries) {
+        delta_encode_short_kernel<<<static_cast<unsigned>((C + kEncCols - 1) / kEncCols), kEncThreads, kEncCols * (E | 1u) * 4,
+                                    reinterpret_cast<cudaStream_t>(stream)>>>(entries_dev, n, E, w, C, db_dev);
+        return cudaGetLastError() == cudaSuccess ? QPADL_OK : QPADL_ECUDA;
+    }
     const int vec = (E % 4 == 0) && (reinterpret_cast<uintptr_t>(entries_dev) & 15u) == 0;
     const dim3 grid(static_cast<unsigned>((C + kEncCols - 1) / kEncCols),
                     static_cast<unsigned>((E + kEncPos - 1) / kEncPos));

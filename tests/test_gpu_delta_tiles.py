@@ -50,3 +50,24 @@ def test_width_sees_one_large_difference(at):
     x = np.arange(4096, dtype=np.uint32)
     x[at:] += 70000
     assert pir.qpadl_pir_delta_width(torch.from_numpy(x.view(np.int32)).cuda(), 512) == oracle.delta_width(x, 512)
+
+
+# blocks staged whole (up to 80 entries) and the first tiled length; 1, 127 to 132 and many columns; the ragged last
+# block; rows of whole words and not
+@pytest.mark.parametrize("E", [1, 2, 3, 5, 16, 64, 79, 80, 81])
+@pytest.mark.parametrize("C,short", [(1, 0), (3, 1), (127, 0), (128, 1), (132, 2), (2000, 0)])
+@pytest.mark.parametrize("w", [1, 2, 3, 4])
+def test_encode_of_short_blocks(E, C, short, w):
+    n = max(1, C * E - short)
+    C = -(-n // E)
+    x = inputs.uniform_u32(n, seed=n + w, tag=inputs.TAG_MISC)   # the encoder keeps w bytes of any difference
+    for at in (0, 1):   # the database on and off a 4-byte boundary
+        buf = torch.full((pir.delta_rows(E, w) * C + at,), 0xAB, dtype=torch.uint8, device="cuda")
+        pir.qpadl_pir_delta_encode(torch.from_numpy(x.view(np.int32)).cuda(), E, w, buf[at:])
+        got = buf[at:].cpu().numpy().reshape(-1, C)
+        v = np.concatenate([x, np.full(C * E - n, x[-1], dtype=np.uint32)]).reshape(C, E)
+        d = v[:, 1:] - v[:, :-1]
+        exp = [(v[:, 0] >> np.uint32(8 * k)) & 255 for k in range(4)]
+        exp += [(d[:, i] >> np.uint32(8 * k)) & 255 for i in range(E - 1) for k in range(w)]
+        assert np.array_equal(got, np.array(exp, dtype=np.uint8))
+        assert at == 0 or int(buf[0]) == 0xAB
