@@ -248,14 +248,15 @@ __global__ void __launch_bounds__(kEncThreads) delta_encode_short_kernel(const u
 }
 
 // Block b: digits b * Rp .. (4-byte first entry, then E - 1 differences of W bytes) -> out b * E ..
-// Thread t takes positions 8 t .. 8 t + 7 of a run of 8192 (its digits are independent loads of
+// Thread t takes positions 8 t .. 8 t + 7 of a run of 8 blockDim.x (its digits are independent loads of
 // adjacent bytes), a two-level shuffle scan gives the sum before them, and the runs of a longer
 // block follow one another with the last sum carried.  64 blocks of 8192: 4.2 us, 12.1 with each thread
-// adding up a run of 32 bytes of its own.
-constexpr int kDecodeThreads = 1024;
+// adding up a run of 32 bytes of its own.  A CTA has as many warps as its block of entries needs, at most 32:
+// 4096 blocks of 2048 / 4096 entries 12 / 25 us, 32 / 39 with 32 warps for each; 2^18 blocks of 16 135, 1644.
+constexpr int kDecodeThreads = 1024;   // at most
 constexpr int kDecodeRun = 8;
 
-template <int W>
+template <int W, bool FULL>   // FULL: 32 warps
 __global__ void __launch_bounds__(kDecodeThreads) delta_decode_kernel(const uint8_t *__restrict__ digits, uint64_t E,
                                                                       uint64_t Rp, int vec,
                                                                       uint32_t *__restrict__ out) {
@@ -263,9 +264,10 @@ __global__ void __launch_bounds__(kDecodeThreads) delta_decode_kernel(const uint
     const uint8_t *dg = digits + (uint64_t)blockIdx.x * Rp;
     uint32_t *o = out + (uint64_t)blockIdx.x * E;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t threads = FULL ? kDecodeThreads : blockDim.x;
     uint32_t carry = 0;
     int turn = 0;
-    for (uint64_t e0 = 0; e0 < E; e0 += kDecodeThreads * kDecodeRun, turn ^= 1) {
+    for (uint64_t e0 = 0; e0 < E; e0 += threads * kDecodeRun, turn ^= 1) {
         const uint64_t t0 = e0 + (uint64_t)threadIdx.x * kDecodeRun;
         uint32_t v[kDecodeRun];
 #pragma unroll
@@ -293,7 +295,7 @@ __global__ void __launch_bounds__(kDecodeThreads) delta_decode_kernel(const uint
         }
         if (lane == 31) part[turn][warp] = sum;
         __syncthreads();   // the other buffer's readers are done before this one is written again
-        uint32_t ps = part[turn][lane];
+        uint32_t ps = FULL || lane < static_cast<int>(threads >> 5) ? part[turn][lane] : 0u;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
             const uint32_t a = __shfl_up_sync(0xffffffffu, ps, off);
@@ -389,9 +391,18 @@ int qpadl_pir_delta_decode(const uint8_t *digits_dev, uint32_t B, uint32_t E, ui
     if (!digits_dev || !entries_dev || B == 0 || !delta_shape_ok(E, E, w)) return QPADL_EINVAL;
     const uint64_t Rp = 4 + (uint64_t)w * (E - 1);
     const int vec = (E % 4 == 0) && (reinterpret_cast<uintptr_t>(entries_dev) & 15u) == 0;
-    const auto kernel = w == 1 ? delta_decode_kernel<1>
-                               : (w == 2 ? delta_decode_kernel<2> : (w == 3 ? delta_decode_kernel<3> : delta_decode_kernel<4>));
-    kernel<<<B, kDecodeThreads, 0, reinterpret_cast<cudaStream_t>(stream)>>>(digits_dev, E, Rp, vec, entries_dev);
+    const uint64_t want = ((uint64_t)E + 32 * kDecodeRun - 1) / (32 * kDecodeRun) * 32;   // whole warps for one run
+    const unsigned threads = static_cast<unsigned>(want < kDecodeThreads ? want : kDecodeThreads);
+    auto launch = [&](auto full, auto part) {
+        const auto kernel = threads == kDecodeThreads ? full : part;
+        kernel<<<B, threads, 0, reinterpret_cast<cudaStream_t>(stream)>>>(digits_dev, E, Rp, vec, entries_dev);
+    };
+    switch (w) {
+        case 1: launch(delta_decode_kernel<1, true>, delta_decode_kernel<1, false>); break;
+        case 2: launch(delta_decode_kernel<2, true>, delta_decode_kernel<2, false>); break;
+        case 3: launch(delta_decode_kernel<3, true>, delta_decode_kernel<3, false>); break;
+        default: launch(delta_decode_kernel<4, true>, delta_decode_kernel<4, false>); break;
+    }
     return cudaGetLastError() == cudaSuccess ? QPADL_OK : QPADL_ECUDA;
 }
 

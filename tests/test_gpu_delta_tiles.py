@@ -71,3 +71,18 @@ def test_encode_of_short_blocks(E, C, short, w):
         exp += [(d[:, i] >> np.uint32(8 * k)) & 255 for i in range(E - 1) for k in range(w)]
         assert np.array_equal(got, np.array(exp, dtype=np.uint8))
         assert at == 0 or int(buf[0]) == 0xAB
+
+
+# CTAs of one warp, of two, of 31 and of 32, one run and two; many blocks
+@pytest.mark.parametrize("E", [1, 2, 255, 256, 257, 512, 513, 7936, 7937, 8192, 8193])
+@pytest.mark.parametrize("w,B", [(1, 1), (2, 70), (4, 5)])
+def test_decode_warps_per_block(E, w, B):
+    Rp = pir.delta_rows(E, w)
+    digits = np.ascontiguousarray(inputs.uniform_u32((B * Rp + 3) // 4, seed=E + w, tag=inputs.TAG_MISC)
+                                  .view(np.uint8)[:B * Rp]).reshape(B, Rp)
+    out = torch.full((B * E + 8,), -1, dtype=torch.int32, device="cuda")
+    pir.qpadl_pir_delta_decode(torch.from_numpy(digits).cuda(), B, E, w, out[:B * E])
+    got = pir.as_u32(out)
+    exp = np.stack([oracle.delta_decode(digits[b], E, w) for b in range(B)])
+    assert np.array_equal(got[:B * E].reshape(B, E), exp)
+    assert (got[B * E:] == 0xFFFFFFFF).all()
