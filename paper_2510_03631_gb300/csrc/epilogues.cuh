@@ -14,25 +14,26 @@ __device__ __forceinline__ void prefetch_l2(const void *p) {
 #pragma once
 #include <cstdint>
 
+#include "vec_sums.cuh"
+
 namespace qpadl {
 
 // kLimbs: limb rows per vector in the GEMM's vector operand (4 byte limbs
 // recombined as sum_k 2^{8k} s_k; 1 = each row is its own vector).
 
-// Plain store: out[i * ld_m + b * ld_b] = dot, or dot + centre * sums[b] when the matrix holds digits
-// minus `centre` and sums[b] is the sum of vector b.
+// Plain store: out[i * ld_m + b * ld_b] = dot, plus what centring the matrix took from vector b (which the
+// kernels add to their running sums).
 struct StoreEpi {
     static constexpr int kLimbs = 4;
     uint32_t *out;
     uint64_t ld_m, ld_b;
-    const uint32_t *sums;
-    uint32_t centre;
+    VecSums sums;
     __device__ __forceinline__ void prefetch(uint64_t, uint32_t, uint32_t) const {}
-    __device__ __forceinline__ uint32_t pre(uint64_t, uint32_t b) const { return sums ? centre * __ldg(sums + b) : 0u; }
-    __device__ __forceinline__ void put(uint64_t i, uint32_t b, uint32_t dot, uint32_t pre_v) const {
-        out[i * ld_m + (uint64_t)b * ld_b] = dot + pre_v;
+    __device__ __forceinline__ uint32_t pre(uint64_t, uint32_t) const { return 0u; }
+    __device__ __forceinline__ void put(uint64_t i, uint32_t b, uint32_t dot, uint32_t) const {
+        out[i * ld_m + (uint64_t)b * ld_b] = dot;
     }
-    __device__ __forceinline__ void operator()(uint64_t i, uint32_t b, uint32_t dot) const { put(i, b, dot, pre(i, b)); }
+    __device__ __forceinline__ void operator()(uint64_t i, uint32_t b, uint32_t dot) const { put(i, b, dot, 0u); }
     // one CTA's part of the element (split tiles; the output starts at zero)
     __device__ __forceinline__ void add(uint64_t i, uint32_t b, uint32_t part) const {
         atomicAdd(out + i * ld_m + (uint64_t)b * ld_b, part);

@@ -8,6 +8,7 @@
 
 #include "limb_gemm_u8.cuh"
 #include "qpadl_pir.h"
+#include "vec_sums.cuh"
 
 namespace qpadl {
 
@@ -15,7 +16,9 @@ namespace qpadl {
 uint64_t db_limb_pitch(const qpadl_db *db);
 // Bytes of limb workspace for B queries: four fp16 limbs, and from three queries on (the smallest batch
 // that needs it) a word each for their sums.
-inline uint64_t limb_workspace_bytes(uint32_t B, uint64_t pitch) { return 8ull * B * pitch + (B > 2 ? 4ull * B : 0); }
+inline uint64_t limb_workspace_bytes(uint32_t B, uint64_t pitch) {
+    return 8ull * B * pitch + (B > 2 ? 4ull * B : 0);
+}
 int db_num_sms(const qpadl_db *db);
 int *db_status_word(qpadl_db *db);
 

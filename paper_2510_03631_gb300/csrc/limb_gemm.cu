@@ -300,6 +300,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             uint32_t run[RUN];
 #pragma unroll
             for (int q = 0; q < RUN; ++q) run[q] = 0u;
+            // what the first piece of a tile adds for the centring: lane l holds vectors l, 32 + l, ...
+            constexpr bool kCentred = std::is_same<Epi, StoreEpi>::value;
+            uint32_t held[(QPT + 31) / 32];
+            if constexpr (kCentred) {
+#pragma unroll
+                for (int q = 0; q < QPT; q += 32) {
+                    const uint32_t o = q + static_cast<uint32_t>(lane);
+                    held[q / 32] = pc.c0 == 0 && o < (uint32_t)QPT && v0 + o < NV ? epi.sums.centred(v0 + o) : 0u;
+                }
+            }
             // planed (client) tiles are short in K: their epilogue inputs (Query noise, Recover
             // answers) are loaded when the tile starts, so the loads overlap its MMAs
             constexpr int EARLY = PLANED ? QPT : 1;
@@ -311,7 +321,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             }
             for (uint32_t c = pc.c0; c < pc.c1; ++c, ++ci) {
                 const uint32_t buf = ci & 1u;
-                if (!mbar_wait(&acc_full[buf], (ci >> 1) & 1u, abort)) {
+                const bool ok = mbar_wait(&acc_full[buf], (ci >> 1) & 1u, abort);
+                if (__any_sync(0xffffffffu, !ok)) {   // the TMEM loads and shuffles below are warp-collective
                     failed = true;
                     break;
                 }
@@ -452,13 +463,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             if (failed) break;
             if constexpr (TMEMSUM) continue;   // the last chunk already wrote the tile
             const uint32_t row = m0 + quarter * 32u + static_cast<uint32_t>(lane);
+            if constexpr (kCentred) {
+#pragma unroll
+                for (int q = 0; q < QPT; ++q) run[q] += __shfl_sync(0xffffffffu, held[q / 32], q % 32);
+            }
             if constexpr (kSplit) {
                 if (row < M && !(pc.c0 == 0 && pc.c1 == nchunks)) {
                     // part of a split tile: exact, since addition mod 2^32 commutes
 #pragma unroll
                     for (int q = 0; q < QPT; ++q)
-                        if (v0 + q < NV)   // the first piece of a tile adds what centred digits leave out
-                            epi.add(row, v0 + q, run[q] + (pc.c0 == 0 ? epi.pre(row, v0 + q) : 0u));
+                        if (v0 + q < NV) epi.add(row, v0 + q, run[q]);
                     continue;
                 }
             }
@@ -819,10 +833,10 @@ static cudaError_t launch_epi(int bn, const CUtensorMap &a_map, const CUtensorMa
     }
 }
 
-cudaError_t launch_limb_gemm(int bn, const CUtensorMap &a_map, const CUtensorMap &b_map, const uint32_t *sums,
-                             uint32_t centre, uint32_t *out, uint64_t ld_m, uint64_t ld_b, uint32_t M, uint32_t NV,
+cudaError_t launch_limb_gemm(int bn, const CUtensorMap &a_map, const CUtensorMap &b_map, const VecSums &sums,
+                             uint32_t *out, uint64_t ld_m, uint64_t ld_b, uint32_t M, uint32_t NV,
                              uint64_t K, int num_sms, int *status, cudaStream_t stream) {
-    return launch_epi(bn, a_map, b_map, StoreEpi{out, ld_m, ld_b, sums, centre}, M, NV, K, 0, num_sms, status, stream);
+    return launch_epi(bn, a_map, b_map, StoreEpi{out, ld_m, ld_b, sums}, M, NV, K, 0, num_sms, status, stream);
 }
 
 cudaError_t launch_limb_gemm_query(int bn, const CUtensorMap &a_map, const CUtensorMap &b_map, const QueryNoiseEpi &epi,

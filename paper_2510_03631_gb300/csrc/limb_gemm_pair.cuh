@@ -4,6 +4,8 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include "vec_sums.cuh"
+
 #include "epilogues.cuh"
 
 namespace qpadl {
@@ -25,10 +27,10 @@ __host__ __device__ inline uint32_t pair_b_box_rows(int bn, bool planed, int u) 
 int limb_gemm_pair_bn_for(uint32_t nv);
 
 // out[i * ld_m + v * ld_b] = sum_j D[i][j] X[v][j] mod 2^32 (i < M, v < NV, j < K) on CTA
-// pairs: a_map covers D - centre as fp16 (box 64 x 128), bm.m[0] four byte limbs per vector (box
+// pairs: a_map covers D - 128 as fp16 (box 64 x 128), bm.m[0] four byte limbs per vector (box
 // 64 x 128), sums the vectors' sums.
-cudaError_t launch_limb_gemm_pair(const CUtensorMap &a_map, const PairBMaps &bm, const uint32_t *sums, uint32_t centre,
-                                  uint32_t *out, uint64_t ld_m, uint64_t ld_b, uint32_t M, uint32_t NV, uint64_t K,
+cudaError_t launch_limb_gemm_pair(const CUtensorMap &a_map, const PairBMaps &bm, const VecSums &sums, uint32_t *out,
+                                  uint64_t ld_m, uint64_t ld_b, uint32_t M, uint32_t NV, uint64_t K,
                                   int num_sms, int *status, cudaStream_t stream);
 // The time of that launch in tile times (256 rows x 64 vectors).
 double limb_gemm_pair_waves(uint32_t M, uint32_t NV, uint64_t K, int num_sms);

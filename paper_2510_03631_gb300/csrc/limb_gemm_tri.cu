@@ -161,7 +161,7 @@ __device__ __forceinline__ void high_limbs(const FoldConsts &k, uint64_t l1, uin
 template <int H>
 __global__ void __launch_bounds__(kTThreads, 1)
     limb_gemm_tri_kernel(const __grid_constant__ CUtensorMap a_map, const __grid_constant__ CUtensorMap b_map,
-                         const uint32_t *__restrict__ sums, uint32_t *__restrict__ out, uint64_t ld_m, uint64_t ld_b,
+                         VecSums sums, uint32_t *__restrict__ out, uint64_t ld_m, uint64_t ld_b,
                          uint32_t M, uint32_t NV, uint32_t KB, uint32_t ksplit, int *__restrict__ status) {
     using Cfg = TriCfg<H>;
     constexpr int ST = Cfg::kStages;
@@ -351,10 +351,14 @@ __global__ void __launch_bounds__(kTThreads, 1)
             const uint32_t row = pc.m * 2 * kTM + rank * kTM + quarter * 32u + static_cast<uint32_t>(lane);
             const uint32_t v0 = pc.n * VPT + box * kTriGroup;
             uint32_t run[H][32];
+            uint32_t held[H];   // lane q: what the first range of a tile adds to vector q, whose digits were centred
 #pragma unroll
-            for (int h = 0; h < H; ++h)
+            for (int h = 0; h < H; ++h) {
+                const uint32_t v = v0 + 64u * h + static_cast<uint32_t>(lane);
+                held[h] = pc.c0 == 0 && v < NV ? sums.centred(v) : 0u;
 #pragma unroll
                 for (int q = 0; q < 32; ++q) run[h][q] = 0u;
+            }
             for (uint32_t c = pc.c0; c < pc.c1 && !failed; ++c) {
 #pragma unroll
                 for (int h = 0; h < H; ++h) {
@@ -393,31 +397,27 @@ __global__ void __launch_bounds__(kTThreads, 1)
             }
             if (failed) break;
             const bool whole = pc.c0 == 0 && pc.c1 == nchunks;   // no other cluster works on this tile
+#pragma unroll
+            for (int h = 0; h < H; ++h)
+#pragma unroll
+                for (int q = 0; q < 32; ++q) run[h][q] += __shfl_sync(0xffffffffu, held[h], q);
             if (row < M) {
 #pragma unroll
                 for (int h = 0; h < H; ++h) {
                     if (quads && whole && v0 + 64u * h + 32u <= NV) {   // 32 neighbouring words of a row
                         uint4 *dst = reinterpret_cast<uint4 *>(out + (uint64_t)row * ld_m + v0 + 64u * h);
 #pragma unroll
-                        for (int q = 0; q < 32; q += 4) {
-                            const uint32_t *sv = sums + v0 + 64u * h + q;
-                            dst[q / 4] = make_uint4(run[h][q] + kTriCentre * __ldg(sv),
-                                                    run[h][q + 1] + kTriCentre * __ldg(sv + 1),
-                                                    run[h][q + 2] + kTriCentre * __ldg(sv + 2),
-                                                    run[h][q + 3] + kTriCentre * __ldg(sv + 3));
-                        }
+                        for (int q = 0; q < 32; q += 4)
+                            dst[q / 4] = make_uint4(run[h][q], run[h][q + 1], run[h][q + 2], run[h][q + 3]);
                         continue;
                     }
 #pragma unroll
                     for (int q = 0; q < 32; ++q) {
                         const uint32_t v = v0 + 64u * h + q;
                         if (v >= NV) continue;
-                        uint32_t r = run[h][q];
-                        // the digits were centred; the first range of a tile puts the vector's part back
-                        if (pc.c0 == 0) r += static_cast<uint32_t>(kTriCentre) * __ldg(sums + v);
                         uint32_t *dst = out + (uint64_t)row * ld_m + (uint64_t)v * ld_b;
-                        if (whole) *dst = r;
-                        else atomicAdd(dst, r);
+                        if (whole) *dst = run[h][q];
+                        else atomicAdd(dst, run[h][q]);
                     }
                 }
             }
@@ -579,44 +579,39 @@ __global__ void __launch_bounds__(256) mat_col_limbs_sums_kernel(const uint32_t 
 }
 
 // ------------------------------------------------------------------ host side
-static uint32_t *tri_sums(__half *L, uint32_t nv, uint64_t pitch) {
-    return reinterpret_cast<uint32_t *>(reinterpret_cast<uint8_t *>(L) + tri_sums_offset(nv, pitch));
-}
-
 template <int LIMBS>
 static cudaError_t launch_vec_limbs_sums(const uint32_t *X, uint64_t x_ld, uint32_t NV, uint64_t C, __half *L,
-                                         uint64_t pitch, uint32_t *sums, uint32_t *zero, uint64_t zero_words,
+                                         uint64_t pitch, const VecSums &sums, uint32_t *zero, uint64_t zero_words,
                                          cudaStream_t stream) {
     if (NV == 0 || C == 0 || NV > 65535 || pitch % 8 != 0) return cudaErrorInvalidValue;
+    uint32_t *words = const_cast<uint32_t *>(sums.words);
     const uint64_t nx = (C + kSumCols - 1) / kSumCols;
     if (nx > 1) {
-        const cudaError_t e = cudaMemsetAsync(sums, 0, 4ull * NV, stream);
+        const cudaError_t e = cudaMemsetAsync(words, 0, 4ull * NV, stream);
         if (e != cudaSuccess) return e;
     }
     const uint64_t want = ((C + 7) / 8 + 31) / 32 * 32;   // threads for one pass
     vec_limbs_sums_kernel<LIMBS><<<dim3(static_cast<unsigned>(nx), NV), static_cast<unsigned>(want < 512 ? want : 512),
-                                   0, stream>>>(X, x_ld, C, L, pitch, sums, zero, zero ? zero_words : 0);
+                                   0, stream>>>(X, x_ld, C, L, pitch, words, zero, zero ? zero_words : 0);
     return cudaGetLastError();
 }
 
 cudaError_t launch_vec_limbs_tri(const uint32_t *X, uint64_t x_ld, uint32_t NV, uint64_t C, __half *L, uint64_t pitch,
                                  uint32_t *zero, uint64_t zero_words, cudaStream_t stream) {
-    return launch_vec_limbs_sums<3>(X, x_ld, NV, C, L, pitch, tri_sums(L, NV, pitch), zero, zero_words, stream);
-}
-
-static uint32_t *four_sums(__half *L, uint32_t nv, uint64_t pitch) {
-    return reinterpret_cast<uint32_t *>(reinterpret_cast<uint8_t *>(L) + four_sums_offset(nv, pitch));
+    return launch_vec_limbs_sums<3>(X, x_ld, NV, C, L, pitch, tri_sums(L, NV, pitch, 1), zero, zero_words,
+                                    stream);
 }
 
 cudaError_t launch_vec_limbs_four(const uint32_t *X, uint64_t x_ld, uint32_t NV, uint64_t C, __half *L, uint64_t pitch,
                                   cudaStream_t stream) {
-    return launch_vec_limbs_sums<4>(X, x_ld, NV, C, L, pitch, four_sums(L, NV, pitch), nullptr, 0, stream);
+    return launch_vec_limbs_sums<4>(X, x_ld, NV, C, L, pitch, four_sums(L, NV, pitch, 1), nullptr, 0, stream);
 }
 
 template <int LIMBS>
 static cudaError_t launch_mat_col_limbs_sums(const uint32_t *A, uint64_t C, uint32_t n, __half *L, uint64_t pitch,
-                                             uint32_t *sums, cudaStream_t stream) {
+                                             const VecSums &vs, cudaStream_t stream) {
     if (n == 0 || C == 0 || pitch % 8 != 0) return cudaErrorInvalidValue;
+    uint32_t *sums = const_cast<uint32_t *>(vs.words);
     const cudaError_t e = cudaMemsetAsync(sums, 0, 4ull * n, stream);
     if (e != cudaSuccess) return e;
     const dim3 grid(static_cast<unsigned>((C + 127) / 128), (n + 31) / 32);
@@ -626,12 +621,12 @@ static cudaError_t launch_mat_col_limbs_sums(const uint32_t *A, uint64_t C, uint
 
 cudaError_t launch_mat_col_limbs_tri(const uint32_t *A, uint64_t C, uint32_t n, __half *L, uint64_t pitch,
                                      cudaStream_t stream) {
-    return launch_mat_col_limbs_sums<3>(A, C, n, L, pitch, tri_sums(L, n, pitch), stream);
+    return launch_mat_col_limbs_sums<3>(A, C, n, L, pitch, tri_sums(L, n, pitch, 1), stream);
 }
 
 cudaError_t launch_mat_col_limbs_four(const uint32_t *A, uint64_t C, uint32_t n, __half *L, uint64_t pitch,
                                       cudaStream_t stream) {
-    return launch_mat_col_limbs_sums<4>(A, C, n, L, pitch, four_sums(L, n, pitch), stream);
+    return launch_mat_col_limbs_sums<4>(A, C, n, L, pitch, four_sums(L, n, pitch, 1), stream);
 }
 
 cudaError_t prepare_limb_gemm_tri_kernels() {
@@ -739,7 +734,7 @@ uint32_t limb_gemm_tri_ranges(uint32_t M, uint32_t NV, uint64_t K, uint64_t ld_m
 }
 
 template <int H>
-static cudaError_t launch_tri_t(const CUtensorMap &a_map, const CUtensorMap &b_map, const uint32_t *sums, uint32_t *out,
+static cudaError_t launch_tri_t(const CUtensorMap &a_map, const CUtensorMap &b_map, const VecSums &sums, uint32_t *out,
                                 uint64_t ld_m, uint64_t ld_b, uint32_t M, uint32_t NV, uint32_t KB, uint32_t ranges,
                                 int num_sms, int *status, cudaStream_t stream) {
     const uint64_t tiles = ((uint64_t)M + 2 * kTM - 1) / (2 * kTM) * (((uint64_t)NV + 64 * H - 1) / (64 * H));
@@ -752,7 +747,7 @@ static cudaError_t launch_tri_t(const CUtensorMap &a_map, const CUtensorMap &b_m
                               status);
 }
 
-cudaError_t launch_limb_gemm_tri(const CUtensorMap &a_map, const CUtensorMap &b_map, const uint32_t *sums,
+cudaError_t launch_limb_gemm_tri(const CUtensorMap &a_map, const CUtensorMap &b_map, const VecSums &sums,
                                  uint32_t *out, uint64_t ld_m, uint64_t ld_b, uint32_t M, uint32_t NV, uint64_t K,
                                  uint32_t ranges, int num_sms, int *status, cudaStream_t stream) {
     if (M == 0 || NV == 0 || K == 0 || ranges == 0 || num_sms < 2) return cudaErrorInvalidValue;

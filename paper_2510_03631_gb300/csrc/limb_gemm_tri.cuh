@@ -5,31 +5,32 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include "vec_sums.cuh"
+
 namespace qpadl {
 
-// Digits are stored centred, as d - 128.
-constexpr int kTriCentre = 128;
 // Limb rows per box of the vector operand: 32 vectors x 3 limbs.
 constexpr uint32_t kTriGroup = 32;
 
-// Bytes of limb scratch for NV vectors: three fp16 rows of `pitch` each, then one word per vector.
-// Never more than the 8 NV pitch bytes of the four-limb layout.
-inline uint64_t tri_sums_offset(uint32_t nv, uint64_t pitch) { return 6ull * nv * pitch; }
-
-// The same with four byte limbs (limb k of vector v in row 4 v + k) for limb_gemm_pair.cu and limb_gemm.cu; the
-// sums lie 8 NV pitch bytes on.
-inline uint64_t four_sums_offset(uint32_t nv, uint64_t pitch) { return 8ull * nv * pitch; }
+// Where the sums of NV vectors lie behind their limbs: three fp16 rows of `pitch` each (then the sums end within
+// 8 NV pitch bytes), or four byte limbs for limb_gemm_pair.cu and limb_gemm.cu (limb k of vector v in row 4 v + k).
+inline VecSums tri_sums(const __half *L, uint32_t nv, uint64_t pitch, uint32_t parts) {
+    return VecSums{reinterpret_cast<const uint32_t *>(L + 3ull * nv * pitch), nv, parts};
+}
+inline VecSums four_sums(const __half *L, uint32_t nv, uint64_t pitch, uint32_t parts) {
+    return VecSums{reinterpret_cast<const uint32_t *>(L + 4ull * nv * pitch), nv, parts};
+}
 
 cudaError_t prepare_limb_gemm_tri_kernels();
 
 // Limbs (11, 11 and 10 bits, balanced) of NV vectors (vector v at X + v * x_ld) into L, limb k of
-// vector v in row 3 v + k, and the vectors' sums mod 2^32 into the words behind them.  When `zero` is
+// vector v in row 3 v + k, and the vectors' sums behind them (one word each).  When `zero` is
 // given, the same launch zeroes zero_words words there.
 cudaError_t launch_vec_limbs_tri(const uint32_t *X, uint64_t x_ld, uint32_t NV, uint64_t C, __half *L, uint64_t pitch,
                                  uint32_t *zero, uint64_t zero_words, cudaStream_t stream);
 cudaError_t launch_vec_limbs_four(const uint32_t *X, uint64_t x_ld, uint32_t NV, uint64_t C, __half *L, uint64_t pitch,
                                   cudaStream_t stream);
-// The three limbs, or four, of the columns of A (C x n row-major): vector k is column k.
+// The three limbs, or four, of the columns of A (C x n row-major), and one sum each: vector k is column k.
 cudaError_t launch_mat_col_limbs_tri(const uint32_t *A, uint64_t C, uint32_t n, __half *L, uint64_t pitch,
                                      cudaStream_t stream);
 cudaError_t launch_mat_col_limbs_four(const uint32_t *A, uint64_t C, uint32_t n, __half *L, uint64_t pitch,
@@ -43,10 +44,10 @@ double limb_gemm_tri_waves(uint32_t M, uint32_t NV, uint64_t K, int num_sms);
 uint32_t limb_gemm_tri_ranges(uint32_t M, uint32_t NV, uint64_t K, uint64_t ld_m, uint64_t ld_b, int num_sms);
 
 // out[i * ld_m + v * ld_b] = sum_j D[i][j] X[v][j] mod 2^32 (i < M, v < NV, j < K): a_map covers the
-// centred digits (box 64 x 128), b_map the limbs as (K, NV, 3) (box 64 x 32 x 3), sums the vectors' sums.
+// centred digits (box 64 x 128), b_map the limbs as (K, NV, 3) (box 64 x 32 x 3).
 // Launched as the programmatic dependent of the kernel before it in the stream, which makes the limbs (and
 // zeroes the output); everything earlier must have completed when that one starts.
-cudaError_t launch_limb_gemm_tri(const CUtensorMap &a_map, const CUtensorMap &b_map, const uint32_t *sums,
+cudaError_t launch_limb_gemm_tri(const CUtensorMap &a_map, const CUtensorMap &b_map, const VecSums &sums,
                                  uint32_t *out, uint64_t ld_m, uint64_t ld_b, uint32_t M, uint32_t NV, uint64_t K,
                                  uint32_t ranges, int num_sms, int *status, cudaStream_t stream);
 

@@ -259,7 +259,7 @@ bool use_tri(const qpadl_db *db) { return db->pair_gemm && db->num_sms >= 2; }
 // The fp16 copy that batches and hints of a lattice handle read, whatever its tile option says: a change
 // of the option after qpadl_pir_reserve builds nothing.
 int ensure_batch_copy(qpadl_db *db, cudaStream_t stream) {
-    return build_f16_copy(db, &db->d16c, &db->ac_map, kTriCentre, stream);
+    return build_f16_copy(db, &db->d16c, &db->ac_map, kCentre, stream);
 }
 
 int ensure_limbs(qpadl_db *db, uint64_t bytes) {
@@ -286,8 +286,8 @@ int set_device(const qpadl_db *db) {
 
 // out[i * ld_m + v * ld_b] = D * X[v] for NV vectors given at `limbs` as three limbs (pair tiles) or, in
 // run_limb_gemm, four (single-SM tiles) and the vectors' sums
-int run_tri_gemm(qpadl_db *db, const __half *limbs, uint32_t NV, uint32_t *out, uint64_t ld_m, uint64_t ld_b,
-                 uint32_t ranges, cudaStream_t stream) {
+int run_tri_gemm(qpadl_db *db, const __half *limbs, uint32_t NV, uint32_t parts, uint32_t *out, uint64_t ld_m,
+                 uint64_t ld_b, uint32_t ranges, cudaStream_t stream) {
     const uint64_t C = db->prm.cols;
     CUtensorMap b_map;   // (column, vector, limb): a box is one CTA's 32 vectors x 3 limbs
     auto fn = encode_fn();
@@ -299,29 +299,27 @@ int run_tri_gemm(qpadl_db *db, const __half *limbs, uint32_t NV, uint32_t *out, 
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return QPADL_ECUDA;
-    const uint32_t *sums = reinterpret_cast<const uint32_t *>(reinterpret_cast<const uint8_t *>(limbs) +
-                                                              tri_sums_offset(NV, db->pitch));
-    QPADL_CU(launch_limb_gemm_tri(db->ac_map, b_map, sums, out, ld_m, ld_b, static_cast<uint32_t>(db->prm.rows), NV, C,
-                                  ranges, db->num_sms, db->d_status, stream));
+    QPADL_CU(launch_limb_gemm_tri(db->ac_map, b_map, tri_sums(limbs, NV, db->pitch, parts), out, ld_m, ld_b,
+                                  static_cast<uint32_t>(db->prm.rows), NV, C, ranges, db->num_sms, db->d_status, stream));
     return QPADL_OK;
 }
 
-int run_limb_gemm(qpadl_db *db, const __half *limbs, uint32_t NV, uint32_t *out, uint64_t ld_m, uint64_t ld_b,
-                  cudaStream_t stream) {
+int run_limb_gemm(qpadl_db *db, const __half *limbs, uint32_t NV, uint32_t parts, uint32_t *out, uint64_t ld_m,
+                  uint64_t ld_b, cudaStream_t stream) {
     const int bn = limb_gemm_bn_for(NV);
     CUtensorMap b_map;
     if (!encode_2d(&b_map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, limbs, db->prm.cols, 4ull * NV, db->pitch * 2,
                    kLimbBoxK, static_cast<uint32_t>(bn), CU_TENSOR_MAP_SWIZZLE_128B))
         return QPADL_ECUDA;
-    const uint32_t *sums = reinterpret_cast<const uint32_t *>(reinterpret_cast<const uint8_t *>(limbs) +
-                                                              four_sums_offset(NV, db->pitch));
-    QPADL_CU(launch_limb_gemm(bn, db->ac_map, b_map, sums, kTriCentre, out, ld_m, ld_b,
+    QPADL_CU(launch_limb_gemm(bn, db->ac_map, b_map, four_sums(limbs, NV, db->pitch, parts), out, ld_m, ld_b,
                               static_cast<uint32_t>(db->prm.rows), NV, db->prm.cols, db->num_sms, db->d_status, stream));
     return QPADL_OK;
 }
 
-// Limb scratch of NV vectors on the handle: four limbs and a word each.
-uint64_t limb_scratch_bytes(const qpadl_db *db, uint32_t NV) { return 8ull * NV * db->pitch + 4ull * NV; }
+// Limb scratch of NV vectors on the handle: four limbs and the sums.
+uint64_t limb_scratch_bytes(const qpadl_db *db, uint32_t NV) {
+    return 8ull * NV * db->pitch + 4ull * NV;
+}
 
 // Whether a batch on pair tiles takes four byte limbs instead of three: only with an odd number of
 // 64-vector halves, where the three-limb tiles (two halves, or three for 3 and 5) leave a half empty
@@ -338,9 +336,10 @@ bool four_limbs(const qpadl_db *db, uint32_t B) {
 }
 
 // Answers of B queries (at most 4096) on the fp16 copy, which exists, their limbs made at `limbs`
-// (limb_workspace_bytes; single-SM tiles need a word more per query for B <= 2).
+// (limb_workspace_bytes; single-SM tiles need room for the sums for B <= 2 as well).
 int answer_f16(qpadl_db *db, const uint32_t *Q, uint32_t B, uint32_t *ans, __half *limbs, cudaStream_t stream) {
     const uint64_t C = db->prm.cols, R = db->prm.rows;
+    const uint32_t parts = 1;
     const bool tri = use_tri(db);
     if (tri && four_limbs(db, B)) {
         QPADL_CU(launch_vec_limbs_four(Q, C, B, C, limbs, db->pitch, stream));
@@ -349,20 +348,18 @@ int answer_f16(qpadl_db *db, const uint32_t *Q, uint32_t B, uint32_t *ans, __hal
         if (!encode_2d(&bm.m[0], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, limbs, C, 4ull * B, db->pitch * 2, kLimbBoxK,
                        pair_b_box_rows(256, false, 0), CU_TENSOR_MAP_SWIZZLE_128B))
             return QPADL_ECUDA;
-        const uint32_t *sums = reinterpret_cast<const uint32_t *>(reinterpret_cast<const uint8_t *>(limbs) +
-                                                                  four_sums_offset(B, db->pitch));
-        QPADL_CU(launch_limb_gemm_pair(db->ac_map, bm, sums, kTriCentre, ans, 1, R, static_cast<uint32_t>(R), B, C,
-                                       db->num_sms, db->d_status, stream));
+        QPADL_CU(launch_limb_gemm_pair(db->ac_map, bm, four_sums(limbs, B, db->pitch, parts), ans, 1, R,
+                                       static_cast<uint32_t>(R), B, C, db->num_sms, db->d_status, stream));
         return QPADL_OK;
     }
     if (tri) {
         const uint32_t ranges = limb_gemm_tri_ranges(static_cast<uint32_t>(R), B, C, 1, R, db->num_sms);
         // one launch makes the limbs and zeroes the answers that ranges add to
         QPADL_CU(launch_vec_limbs_tri(Q, C, B, C, limbs, db->pitch, ranges > 1 ? ans : nullptr, (uint64_t)B * R, stream));
-        return run_tri_gemm(db, limbs, B, ans, 1, R, ranges, stream);
+        return run_tri_gemm(db, limbs, B, parts, ans, 1, R, ranges, stream);
     }
     QPADL_CU(launch_vec_limbs_four(Q, C, B, C, limbs, db->pitch, stream));
-    return run_limb_gemm(db, limbs, B, ans, 1, R, stream);
+    return run_limb_gemm(db, limbs, B, parts, ans, 1, R, stream);
 }
 
 int answer_stream_group(qpadl_db *db, const uint32_t *Q, uint32_t nq, uint32_t *ans, cudaStream_t stream) {
@@ -798,11 +795,11 @@ int qpadl_pir_hint(qpadl_db *db, const uint32_t *A_dev, uint32_t *H_dev, qpadl_s
         const uint32_t ranges = limb_gemm_tri_ranges(static_cast<uint32_t>(R), n, db->prm.cols, n, 1, db->num_sms);
         if (ranges > 1) QPADL_CU(cudaMemsetAsync(H_dev, 0, 4ull * n * R, s));
         QPADL_CU(launch_mat_col_limbs_tri(A_dev, db->prm.cols, n, db->limbs, db->pitch, s));
-        return run_tri_gemm(db, db->limbs, n, H_dev, n, 1, ranges, s);
+        return run_tri_gemm(db, db->limbs, n, 1, H_dev, n, 1, ranges, s);
     }
     if (!u8) {
         QPADL_CU(launch_mat_col_limbs_four(A_dev, db->prm.cols, n, db->limbs, db->pitch, s));
-        return run_limb_gemm(db, db->limbs, n, H_dev, n, 1, s);
+        return run_limb_gemm(db, db->limbs, n, 1, H_dev, n, 1, s);
     }
     QPADL_CU(launch_mat_col_limbs(A_dev, db->prm.cols, n, db->limbs, db->pitch, s));
     return run_u8_gemm(db, n, H_dev, n, 1, s);
