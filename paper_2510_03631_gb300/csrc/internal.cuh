@@ -15,9 +15,9 @@ namespace qpadl {
 // Row pitch (elements) of a limb operand for this database: roundup(C, 8).
 uint64_t db_limb_pitch(const qpadl_db *db);
 // Bytes of limb workspace for B queries: four fp16 limbs, and from three queries on (the smallest batch
-// that needs it) a word each for their sums.
+// that needs it) their sums.
 inline uint64_t limb_workspace_bytes(uint32_t B, uint64_t pitch) {
-    return 8ull * B * pitch + (B > 2 ? 4ull * B : 0);
+    return 8ull * B * pitch + (B > 2 ? 4ull * B * limb_sum_parts(pitch) : 0);
 }
 int db_num_sms(const qpadl_db *db);
 int *db_status_word(qpadl_db *db);

@@ -469,15 +469,16 @@ __device__ __forceinline__ void store8(__half *dst, const int (&l)[8]) {
     *reinterpret_cast<uint4 *>(dst) = *reinterpret_cast<const uint4 *>(h);
 }
 
-// Blocks (x, y) make the limbs of vector y, 8 consecutive columns per thread and pass.  Up to kSumCols
-// columns are one block's, which then stores the vector's sum; of a longer vector each block adds its part to a
-// zeroed one.  z: words to zero (the output of a GEMM whose ranges add up).
-constexpr uint64_t kSumCols = 65536;
+// Block (x, y) makes the limbs of columns [2048 x, 2048 x + 2048) of vector y, 8 consecutive columns per thread, and
+// the sum of those words; the GEMM adds a vector's sums up.  One block per vector and whole row left SMs idle and
+// made every thread walk: 130 vectors of 30000 columns 10.5 us, 7.5 this way; 256 of 32768 (three limbs) 20 and
+// 16; a cluster of blocks per vector that adds up in shared memory 11.1 and 20.  z: words to zero (the output of a
+// GEMM whose pieces add up).
 template <int LIMBS>
-__global__ void __launch_bounds__(512, 2) vec_limbs_sums_kernel(const uint32_t *__restrict__ X, uint64_t x_ld, uint64_t C,
-                                                              __half *__restrict__ L, uint64_t pitch,
-                                                              uint32_t *__restrict__ sums, uint32_t *__restrict__ Z,
-                                                              uint64_t z_words) {
+__global__ void __launch_bounds__(kSumCols / 8) vec_limbs_sums_kernel(const uint32_t *__restrict__ X, uint64_t x_ld, uint64_t C,
+                                                                     __half *__restrict__ L, uint64_t pitch,
+                                                                     uint32_t *__restrict__ sums, uint32_t *__restrict__ Z,
+                                                                     uint64_t z_words) {
     griddep_launch_dependents();   // the GEMM's start overlaps this kernel; it waits before it reads the limbs
     for (uint64_t i = ((uint64_t)blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x; i < z_words;
          i += (uint64_t)gridDim.x * gridDim.y * blockDim.x)
@@ -486,31 +487,28 @@ __global__ void __launch_bounds__(512, 2) vec_limbs_sums_kernel(const uint32_t *
     __half *dst = L + (uint64_t)LIMBS * blockIdx.y * pitch;
     const bool vec = ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15u) == 0;
     uint32_t sum = 0;
-#pragma unroll 2
-    for (uint64_t j0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) * 8; j0 < C;
-         j0 += 8ull * gridDim.x * blockDim.x) {
-        if (vec && j0 + 8 <= C) {
-            const uint4 a = *reinterpret_cast<const uint4 *>(src + j0);
-            const uint4 b = *reinterpret_cast<const uint4 *>(src + j0 + 4);
-            const uint32_t x[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-            int l[LIMBS][8];
+    const uint64_t j0 = (uint64_t)blockIdx.x * kSumCols + threadIdx.x * 8;
+    if (vec && j0 + 8 <= C) {
+        const uint4 a = *reinterpret_cast<const uint4 *>(src + j0);
+        const uint4 b = *reinterpret_cast<const uint4 *>(src + j0 + 4);
+        const uint32_t x[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+        int l[LIMBS][8];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                int t[LIMBS];
-                balanced(x[i], t);
+        for (int i = 0; i < 8; ++i) {
+            int t[LIMBS];
+            balanced(x[i], t);
 #pragma unroll
-                for (int k = 0; k < LIMBS; ++k) l[k][i] = t[k];
-                sum += x[i];
-            }
+            for (int k = 0; k < LIMBS; ++k) l[k][i] = t[k];
+            sum += x[i];
+        }
 #pragma unroll
-            for (int k = 0; k < LIMBS; ++k) store8(dst + k * pitch + j0, l[k]);   // pitch % 8 == 0
-        } else {
-            for (uint64_t j = j0; j < C && j < j0 + 8; ++j) {
-                int t[LIMBS];
-                balanced(src[j], t);
-                for (int k = 0; k < LIMBS; ++k) dst[k * pitch + j] = __int2half_rn(t[k]);
-                sum += src[j];
-            }
+        for (int k = 0; k < LIMBS; ++k) store8(dst + k * pitch + j0, l[k]);   // pitch % 8 == 0
+    } else {
+        for (uint64_t j = j0; j < C && j < j0 + 8; ++j) {
+            int t[LIMBS];
+            balanced(src[j], t);
+            for (int k = 0; k < LIMBS; ++k) dst[k * pitch + j] = __int2half_rn(t[k]);
+            sum += src[j];
         }
     }
     __shared__ uint32_t part[32];
@@ -519,10 +517,8 @@ __global__ void __launch_bounds__(512, 2) vec_limbs_sums_kernel(const uint32_t *
     if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = sum;
     __syncthreads();
     if (threadIdx.x == 0) {
-        sum = 0;
-        for (uint32_t w = 0; w < blockDim.x / 32; ++w) sum += part[w];
-        if (gridDim.x == 1) sums[blockIdx.y] = sum;
-        else atomicAdd(sums + blockIdx.y, sum);
+        for (uint32_t w = 1; w < blockDim.x / 32; ++w) sum += part[w];
+        sums[(uint64_t)blockIdx.x * gridDim.y + blockIdx.y] = sum;
     }
 }
 
@@ -584,27 +580,22 @@ static cudaError_t launch_vec_limbs_sums(const uint32_t *X, uint64_t x_ld, uint3
                                          uint64_t pitch, const VecSums &sums, uint32_t *zero, uint64_t zero_words,
                                          cudaStream_t stream) {
     if (NV == 0 || C == 0 || NV > 65535 || pitch % 8 != 0) return cudaErrorInvalidValue;
-    uint32_t *words = const_cast<uint32_t *>(sums.words);
-    const uint64_t nx = (C + kSumCols - 1) / kSumCols;
-    if (nx > 1) {
-        const cudaError_t e = cudaMemsetAsync(words, 0, 4ull * NV, stream);
-        if (e != cudaSuccess) return e;
-    }
-    const uint64_t want = ((C + 7) / 8 + 31) / 32 * 32;   // threads for one pass
-    vec_limbs_sums_kernel<LIMBS><<<dim3(static_cast<unsigned>(nx), NV), static_cast<unsigned>(want < 512 ? want : 512),
-                                   0, stream>>>(X, x_ld, C, L, pitch, words, zero, zero ? zero_words : 0);
+    const uint64_t want = ((C + 7) / 8 + 31) / 32 * 32;   // threads for all columns
+    vec_limbs_sums_kernel<LIMBS>
+        <<<dim3(sums.parts, NV), static_cast<unsigned>(want < kSumCols / 8 ? want : kSumCols / 8), 0, stream>>>(
+            X, x_ld, C, L, pitch, const_cast<uint32_t *>(sums.words), zero, zero ? zero_words : 0);
     return cudaGetLastError();
 }
 
 cudaError_t launch_vec_limbs_tri(const uint32_t *X, uint64_t x_ld, uint32_t NV, uint64_t C, __half *L, uint64_t pitch,
                                  uint32_t *zero, uint64_t zero_words, cudaStream_t stream) {
-    return launch_vec_limbs_sums<3>(X, x_ld, NV, C, L, pitch, tri_sums(L, NV, pitch, 1), zero, zero_words,
+    return launch_vec_limbs_sums<3>(X, x_ld, NV, C, L, pitch, tri_sums(L, NV, pitch, limb_sum_parts(C)), zero, zero_words,
                                     stream);
 }
 
 cudaError_t launch_vec_limbs_four(const uint32_t *X, uint64_t x_ld, uint32_t NV, uint64_t C, __half *L, uint64_t pitch,
                                   cudaStream_t stream) {
-    return launch_vec_limbs_sums<4>(X, x_ld, NV, C, L, pitch, four_sums(L, NV, pitch, 1), nullptr, 0, stream);
+    return launch_vec_limbs_sums<4>(X, x_ld, NV, C, L, pitch, four_sums(L, NV, pitch, limb_sum_parts(C)), nullptr, 0, stream);
 }
 
 template <int LIMBS>

@@ -24,7 +24,7 @@ inline VecSums four_sums(const __half *L, uint32_t nv, uint64_t pitch, uint32_t 
 cudaError_t prepare_limb_gemm_tri_kernels();
 
 // Limbs (11, 11 and 10 bits, balanced) of NV vectors (vector v at X + v * x_ld) into L, limb k of
-// vector v in row 3 v + k, and the vectors' sums behind them (one word each).  When `zero` is
+// vector v in row 3 v + k, and the vectors' sums behind them (limb_sum_parts(C) words each).  When `zero` is
 // given, the same launch zeroes zero_words words there.
 cudaError_t launch_vec_limbs_tri(const uint32_t *X, uint64_t x_ld, uint32_t NV, uint64_t C, __half *L, uint64_t pitch,
                                  uint32_t *zero, uint64_t zero_words, cudaStream_t stream);

@@ -318,7 +318,7 @@ int run_limb_gemm(qpadl_db *db, const __half *limbs, uint32_t NV, uint32_t parts
 
 // Limb scratch of NV vectors on the handle: four limbs and the sums.
 uint64_t limb_scratch_bytes(const qpadl_db *db, uint32_t NV) {
-    return 8ull * NV * db->pitch + 4ull * NV;
+    return 8ull * NV * db->pitch + 4ull * NV * limb_sum_parts(db->prm.cols);
 }
 
 // Whether a batch on pair tiles takes four byte limbs instead of three: only with an odd number of
@@ -339,7 +339,7 @@ bool four_limbs(const qpadl_db *db, uint32_t B) {
 // (limb_workspace_bytes; single-SM tiles need room for the sums for B <= 2 as well).
 int answer_f16(qpadl_db *db, const uint32_t *Q, uint32_t B, uint32_t *ans, __half *limbs, cudaStream_t stream) {
     const uint64_t C = db->prm.cols, R = db->prm.rows;
-    const uint32_t parts = 1;
+    const uint32_t parts = limb_sum_parts(C);
     const bool tri = use_tri(db);
     if (tri && four_limbs(db, B)) {
         QPADL_CU(launch_vec_limbs_four(Q, C, B, C, limbs, db->pitch, stream));

@@ -6,6 +6,11 @@ namespace qpadl {
 
 // Digits are stored centred, as d - 128.
 constexpr uint32_t kCentre = 128;
+// Columns per partial sum of a vector.
+constexpr uint32_t kSumCols = 2048;
+__host__ __device__ constexpr uint32_t limb_sum_parts(uint64_t cols) {
+    return static_cast<uint32_t>((cols + kSumCols - 1) / kSumCols);
+}
 // The sum mod 2^32 of vector v is that of words[x * nv + v] over x < parts.
 struct VecSums {
     const uint32_t *words;
