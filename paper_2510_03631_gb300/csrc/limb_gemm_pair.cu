@@ -242,6 +242,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
 #pragma unroll
                 for (int u = 0; u < (PLANED ? 4 : 1); ++u) tma_prefetch_desc(&bm.m[u]);
             }
+            if (!mat) griddep_wait();   // the plain store's limbs come from the kernel it overlaps
             const uint32_t kpp = PLANED ? ckb * plane_chunks : KB;   // k-steps per limb plane
             uint32_t it = 0, st = 0, ph = 0;
             PairPieceIter pit(tiles, dp_tiles, n_tiles, nchunks, tparts, ks, cluster, nclusters);
@@ -357,6 +358,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
         // ---------------- epilogue (warps 2..5 of both CTAs; TMEM lane quarter = warp % 4)
         const uint32_t quarter = static_cast<uint32_t>(warp & 3);
         const uint32_t lane_addr = (quarter * 32u) << 16;
+        griddep_wait();   // so do its sums and its zeroed output
         uint32_t ci = 0;
         PairPieceIter pit(tiles, dp_tiles, n_tiles, nchunks, tparts, ks, cluster, nclusters);
         PairPiece pc;
@@ -623,9 +625,11 @@ int limb_gemm_pair_bn_for(uint32_t nv) {
     return 256;
 }
 
-// Launch configuration of a pair kernel: clusters of 2 CTAs, one CTA per SM.
+// Launch configuration of a pair kernel: clusters of 2 CTAs, one CTA per SM; a dependent one overlaps the kernel
+// before it in the stream.
 template <int BN>
-static cudaLaunchConfig_t pair_config(unsigned clusters, cudaStream_t stream, cudaLaunchAttribute *attr) {
+static cudaLaunchConfig_t pair_config(unsigned clusters, cudaStream_t stream, cudaLaunchAttribute (&attr)[2],
+                                      bool dependent = false) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * clusters);
     cfg.blockDim = dim3(kPThreads);
@@ -635,8 +639,10 @@ static cudaLaunchConfig_t pair_config(unsigned clusters, cudaStream_t stream, cu
     attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = dependent ? 2 : 1;
     return cfg;
 }
 
@@ -648,7 +654,7 @@ static int resident_pairs(int num_sms) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return num_sms / 2;
     if (cache[dev] > 0) return cache[dev];
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg = pair_config<BN>(static_cast<unsigned>(num_sms / 2), nullptr, attr);
     int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, limb_gemm_pair_kernel<BN, Epi, PLANED>, &cfg) != cudaSuccess || n <= 0) {
@@ -739,20 +745,8 @@ static cudaError_t launch_pair_t(const CUtensorMap &a_map, const PairBMaps &bm, 
     uint64_t clusters = tiles < pairs ? tiles : pairs;
     uint32_t dp = 0xffffffffu, tail_parts = 0;
     uint32_t ksplit = 1;
-    // split tiles add into the output, so it is zeroed first; only a dense output (every
-    // element of the M x NV block, in either order) can be zeroed in one piece
-    if constexpr (std::is_same<Epi, StoreEpi>::value) {
-        const bool dense = (epi.ld_m == 1 && epi.ld_b == M) || (epi.ld_b == 1 && epi.ld_m == NV);
-        uint64_t c2 = clusters;
-        uint32_t dp2 = 0, tp2 = 0;
-        if (dense && pair_split_schedule(tiles, n_tiles, (KB + ckb - 1) / ckb, pairs, &c2, &dp2, &tp2)) {
-            const cudaError_t e = cudaMemsetAsync(epi.out, 0, 4ull * M * NV, stream);
-            if (e != cudaSuccess) return e;
-            clusters = c2;
-            dp = dp2;
-            tail_parts = tp2;
-        }
-    }
+    if constexpr (std::is_same<Epi, StoreEpi>::value)   // split tiles add into the output, which is zero then
+        pair_split_schedule(tiles, n_tiles, (KB + ckb - 1) / ckb, pairs, &clusters, &dp, &tail_parts);
     if constexpr (std::is_same<Epi, ModPEpi>::value) {
         if (epi.ld_m == 1 && epi.ld_b == M) ksplit = field_ksplit(tiles, n_tiles, (KB + ckb - 1) / ckb, pairs, (uint64_t)M * NV);
         if (ksplit > 1) {
@@ -762,8 +756,9 @@ static cudaError_t launch_pair_t(const CUtensorMap &a_map, const PairBMaps &bm, 
         }
     }
     if (clusters == 0) return cudaSuccess;
-    cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = pair_config<BN>(static_cast<unsigned>(clusters), stream, attr);
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t cfg =
+        pair_config<BN>(static_cast<unsigned>(clusters), stream, attr, std::is_same<Epi, StoreEpi>::value);
     const cudaError_t e = cudaLaunchKernelEx(&cfg, limb_gemm_pair_kernel<BN, Epi, PLANED>, a_map, bm, epi, M, NV, KB,
                                              ckb, plane_chunks, dp, tail_parts, ksplit, status);
     if constexpr (std::is_same<Epi, ModPEpi>::value) {
@@ -821,21 +816,35 @@ static cudaError_t launch_pair_epi(int bn, const CUtensorMap &a_map, const PairB
 }
 
 cudaError_t launch_limb_gemm_pair(const CUtensorMap &a_map, const PairBMaps &bm, const VecSums &sums, uint32_t *out,
-                                  uint64_t ld_m, uint64_t ld_b, uint32_t M, uint32_t NV, uint64_t K,
-                                  int num_sms, int *status, cudaStream_t stream) {
-    return launch_pair_epi(256, a_map, bm, StoreEpi{out, ld_m, ld_b, sums}, M, NV, K, 0, num_sms, status, stream);
+                                  uint32_t M, uint32_t NV, uint64_t K, int num_sms, int *status,
+                                  cudaStream_t stream) {
+    return launch_pair_epi(256, a_map, bm, StoreEpi{out, 1, M, sums}, M, NV, K, 0, num_sms, status, stream);
 }
 
-double limb_gemm_pair_waves(uint32_t M, uint32_t NV, uint64_t K, int num_sms) {
+// The schedule of that launch: whole waves in *waves, or its split.
+static bool store_schedule(uint32_t M, uint32_t NV, uint64_t K, int num_sms, double *waves) {
     const uint64_t n_tiles = ((uint64_t)NV + 63) / 64, tiles = ((uint64_t)M + 2 * kPM - 1) / (2 * kPM) * n_tiles;
     const uint32_t KB = static_cast<uint32_t>((K + kPK - 1) / kPK), ckb = store_chunk_kb(KB);
     const uint64_t pairs = static_cast<uint64_t>(resident_pairs<256, StoreEpi, false>(num_sms));
     uint64_t clusters = 0;
     uint32_t dp = 0, tail = 0;
-    if (pairs == 0) return 0.0;
-    if (pair_split_schedule(tiles, n_tiles, (KB + ckb - 1) / ckb, pairs, &clusters, &dp, &tail))
-        return static_cast<double>(dp) / pairs + static_cast<double>(tiles - dp) / (tail * n_tiles);
-    return static_cast<double>((tiles + pairs - 1) / pairs);
+    *waves = 0.0;
+    if (pairs == 0) return false;
+    const bool split = pair_split_schedule(tiles, n_tiles, (KB + ckb - 1) / ckb, pairs, &clusters, &dp, &tail);
+    *waves = split ? static_cast<double>(dp) / pairs + static_cast<double>(tiles - dp) / (tail * n_tiles)
+                   : static_cast<double>((tiles + pairs - 1) / pairs);
+    return split;
+}
+
+bool limb_gemm_pair_splits(uint32_t M, uint32_t NV, uint64_t K, int num_sms) {
+    double waves;
+    return store_schedule(M, NV, K, num_sms, &waves);
+}
+
+double limb_gemm_pair_waves(uint32_t M, uint32_t NV, uint64_t K, int num_sms) {
+    double waves;
+    store_schedule(M, NV, K, num_sms, &waves);
+    return waves;
 }
 
 cudaError_t launch_limb_gemm_pair_query(int bn, const CUtensorMap &a_map, const PairBMaps &bm,

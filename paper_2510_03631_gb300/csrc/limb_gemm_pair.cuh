@@ -26,13 +26,15 @@ __host__ __device__ inline uint32_t pair_b_box_rows(int bn, bool planed, int u) 
 // Tile width (vector-operand rows per pair tile, 128 or 256) for nv vectors of 4 limbs.
 int limb_gemm_pair_bn_for(uint32_t nv);
 
-// out[i * ld_m + v * ld_b] = sum_j D[i][j] X[v][j] mod 2^32 (i < M, v < NV, j < K) on CTA
-// pairs: a_map covers D - 128 as fp16 (box 64 x 128), bm.m[0] four byte limbs per vector (box
-// 64 x 128), sums the vectors' sums.
+// out[v * M + i] = sum_j D[i][j] X[v][j] mod 2^32 (i < M, v < NV, j < K) on CTA pairs: a_map covers
+// D - 128 as fp16 (box 64 x 128), bm.m[0] four byte limbs per vector (box 64 x 128), sums the vectors' sums.
+// Launched as the programmatic dependent of the kernel before it in the stream, which makes the limbs and, when
+// limb_gemm_pair_splits, zeroes out; everything earlier must have completed when that one starts.
 cudaError_t launch_limb_gemm_pair(const CUtensorMap &a_map, const PairBMaps &bm, const VecSums &sums, uint32_t *out,
-                                  uint64_t ld_m, uint64_t ld_b, uint32_t M, uint32_t NV, uint64_t K,
-                                  int num_sms, int *status, cudaStream_t stream);
-// The time of that launch in tile times (256 rows x 64 vectors).
+                                  uint32_t M, uint32_t NV, uint64_t K, int num_sms, int *status,
+                                  cudaStream_t stream);
+// Whether that launch splits tiles, whose pieces add into out, and its time in tile times (256 rows x 64 vectors).
+bool limb_gemm_pair_splits(uint32_t M, uint32_t NV, uint64_t K, int num_sms);
 double limb_gemm_pair_waves(uint32_t M, uint32_t NV, uint64_t K, int num_sms);
 
 // Client Query / Recover batches on CTA pairs.  plane_chunks = n / 512 selects

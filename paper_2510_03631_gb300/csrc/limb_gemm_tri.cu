@@ -594,8 +594,9 @@ cudaError_t launch_vec_limbs_tri(const uint32_t *X, uint64_t x_ld, uint32_t NV, 
 }
 
 cudaError_t launch_vec_limbs_four(const uint32_t *X, uint64_t x_ld, uint32_t NV, uint64_t C, __half *L, uint64_t pitch,
-                                  cudaStream_t stream) {
-    return launch_vec_limbs_sums<4>(X, x_ld, NV, C, L, pitch, four_sums(L, NV, pitch, limb_sum_parts(C)), nullptr, 0, stream);
+                                  uint32_t *zero, uint64_t zero_words, cudaStream_t stream) {
+    return launch_vec_limbs_sums<4>(X, x_ld, NV, C, L, pitch, four_sums(L, NV, pitch, limb_sum_parts(C)), zero,
+                                    zero_words, stream);
 }
 
 template <int LIMBS>

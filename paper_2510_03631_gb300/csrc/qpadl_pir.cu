@@ -342,13 +342,15 @@ int answer_f16(qpadl_db *db, const uint32_t *Q, uint32_t B, uint32_t *ans, __hal
     const uint32_t parts = limb_sum_parts(C);
     const bool tri = use_tri(db);
     if (tri && four_limbs(db, B)) {
-        QPADL_CU(launch_vec_limbs_four(Q, C, B, C, limbs, db->pitch, stream));
+        // as below, one launch makes the limbs and zeroes the answers that split tiles add to
+        const bool split = limb_gemm_pair_splits(static_cast<uint32_t>(R), B, C, db->num_sms);
+        QPADL_CU(launch_vec_limbs_four(Q, C, B, C, limbs, db->pitch, split ? ans : nullptr, (uint64_t)B * R, stream));
         PairBMaps bm;
         std::memset(&bm, 0, sizeof(bm));
         if (!encode_2d(&bm.m[0], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, limbs, C, 4ull * B, db->pitch * 2, kLimbBoxK,
                        pair_b_box_rows(256, false, 0), CU_TENSOR_MAP_SWIZZLE_128B))
             return QPADL_ECUDA;
-        QPADL_CU(launch_limb_gemm_pair(db->ac_map, bm, four_sums(limbs, B, db->pitch, parts), ans, 1, R,
+        QPADL_CU(launch_limb_gemm_pair(db->ac_map, bm, four_sums(limbs, B, db->pitch, parts), ans,
                                        static_cast<uint32_t>(R), B, C, db->num_sms, db->d_status, stream));
         return QPADL_OK;
     }
@@ -358,7 +360,7 @@ int answer_f16(qpadl_db *db, const uint32_t *Q, uint32_t B, uint32_t *ans, __hal
         QPADL_CU(launch_vec_limbs_tri(Q, C, B, C, limbs, db->pitch, ranges > 1 ? ans : nullptr, (uint64_t)B * R, stream));
         return run_tri_gemm(db, limbs, B, parts, ans, 1, R, ranges, stream);
     }
-    QPADL_CU(launch_vec_limbs_four(Q, C, B, C, limbs, db->pitch, stream));
+    QPADL_CU(launch_vec_limbs_four(Q, C, B, C, limbs, db->pitch, nullptr, 0, stream));
     return run_limb_gemm(db, limbs, B, parts, ans, 1, R, stream);
 }
 
