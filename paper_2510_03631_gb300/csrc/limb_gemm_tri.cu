@@ -54,6 +54,13 @@ constexpr int kTN = 192;           // limb columns per accumulator
 constexpr int kChunkSteps = 2;     // k-steps per exact chunk: 128 columns of D
 constexpr int kTThreads = 384;     // warps: 0 matrix producer, 1 MMA, 2 vector producer, 4..11 epilogue
 
+// How the output is stored: a word per lane and vector (the lanes' rows are neighbours in column-major answers), or, for
+// the hint's rows, 16 bytes a lane where they allow it (30000 x 600 digits by 512 columns: 214 us with word stores,
+// 84), else 32 rows x 32 vectors turned, so that a warp writes a row's 128 bytes at a time (4864 x 1088 by 630 columns: word
+// stores 46.9 us, turned 35.9; 7104 x 2471 by 1024 in all: 16-byte stores 91.5, turned 99.3).
+// out[row + v * ld], or the others' out[row * ld + v].
+enum { kWords, kQuads, kTurned };
+
 template <int H>
 struct TriCfg {
     static constexpr uint32_t kABytes = kTM * kTK * 2;              // 16 KB
@@ -172,10 +179,10 @@ __device__ __forceinline__ void high_limbs(const FoldConsts &k, uint64_t l1, uin
 
 }  // namespace
 
-template <int H>
+template <int H, int OUT>
 __global__ void __launch_bounds__(kTThreads, 1)
     limb_gemm_tri_kernel(const __grid_constant__ CUtensorMap a_map, const __grid_constant__ CUtensorMap b_map,
-                         VecSums sums, uint32_t *__restrict__ out, uint64_t ld_m, uint64_t ld_b,
+                         VecSums sums, uint32_t *__restrict__ out, uint64_t ld,
                          uint32_t M, uint32_t NV, uint32_t KB, uint32_t ksplit, int *__restrict__ status) {
     using Cfg = TriCfg<H>;
     constexpr int ST = Cfg::kStages;
@@ -358,11 +365,6 @@ __global__ void __launch_bounds__(kTThreads, 1)
         const uint32_t taddr = tmem_base + ((quarter * 32u) << 16) + 96u * box;
         const FoldConsts consts;
         griddep_wait();   // the sums and the zeroed output come from the kernel this one overlaps
-        // A row-major output (the hint) is stored 16 bytes a lane where its rows allow it (30000 x 600 digits by 512
-        // columns: 214 us with word stores, 84); else 32 rows x 32 vectors are turned, so that a warp writes a row's
-        // 128 bytes at a time (4864 x 1088 by 630 columns: word stores 46.9 us, turned 35.9; 7104 x 2471 by 1024
-        // in all: 16-byte stores 91.5, turned 99.3).
-        const bool quads = ld_b == 1 && ld_m % 4 == 0 && (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
         uint32_t item = 0;
         while (!failed && iter.next(pc)) {
             const uint32_t row = pc.m * 2 * kTM + rank * kTM + quarter * 32u + static_cast<uint32_t>(lane);
@@ -418,21 +420,14 @@ __global__ void __launch_bounds__(kTThreads, 1)
             for (int h = 0; h < H; ++h)
 #pragma unroll
                 for (int q = 0; q < 32; ++q) run[h][q] += __shfl_sync(0xffffffffu, held[h], q);
-            if (ld_b == 1) {
+            if constexpr (OUT == kTurned) {
 #pragma unroll
                 for (int h = 0; h < H; ++h) {
-                    if (quads && whole && v0 + 64u * h + 32u <= NV) {   // 32 neighbouring words of a row
-                        uint4 *dst = reinterpret_cast<uint4 *>(out + (uint64_t)row * ld_m + v0 + 64u * h);
-#pragma unroll
-                        for (int q = 0; q < 32; q += 4)
-                            if (row < M) dst[q / 4] = make_uint4(run[h][q], run[h][q + 1], run[h][q + 2], run[h][q + 3]);
-                        continue;
-                    }
                     turn32(run[h], lane);
                     const uint32_t v = v0 + 64u * h + static_cast<uint32_t>(lane), i0 = row - static_cast<uint32_t>(lane);
-                    uint32_t *dst = out + (uint64_t)i0 * ld_m + v;
+                    uint32_t *dst = out + (uint64_t)i0 * ld + v;
 #pragma unroll
-                    for (int q = 0; q < 32; ++q, dst += ld_m) {
+                    for (int q = 0; q < 32; ++q, dst += ld) {
                         if (v >= NV || i0 + q >= M) continue;
                         if (whole) *dst = run[h][q];
                         else atomicAdd(dst, run[h][q]);
@@ -440,15 +435,23 @@ __global__ void __launch_bounds__(kTThreads, 1)
                 }
             } else if (row < M) {
 #pragma unroll
-                for (int h = 0; h < H; ++h)
+                for (int h = 0; h < H; ++h) {
+                    if (OUT == kQuads && v0 + 64u * h + 32u <= NV) {   // 32 neighbouring words of a row
+                        uint4 *dst = reinterpret_cast<uint4 *>(out + (uint64_t)row * ld + v0 + 64u * h);
 #pragma unroll
-                    for (int q = 0; q < 32; ++q) {
-                        const uint32_t v = v0 + 64u * h + q;
-                        if (v >= NV) continue;
-                        uint32_t *dst = out + (uint64_t)row * ld_m + (uint64_t)v * ld_b;
-                        if (whole) *dst = run[h][q];
+                        for (int q = 0; q < 32; q += 4)
+                            dst[q / 4] = make_uint4(run[h][q], run[h][q + 1], run[h][q + 2], run[h][q + 3]);
+                        continue;
+                    }
+                    const uint32_t v = v0 + 64u * h, n = NV > v ? NV - v : 0u;
+                    uint32_t *dst = out + (OUT == kWords ? row + (uint64_t)v * ld : (uint64_t)row * ld + v);
+#pragma unroll
+                    for (uint32_t q = 0; q < 32; ++q, dst += OUT == kWords ? ld : 1) {
+                        if (q >= n) continue;
+                        if (OUT == kQuads || whole) *dst = run[h][q];
                         else atomicAdd(dst, run[h][q]);
                     }
+                }
             }
         }
     }
@@ -650,15 +653,19 @@ cudaError_t launch_mat_col_limbs_four(const uint32_t *A, uint64_t C, uint32_t n,
     return launch_mat_col_limbs_sums<4>(A, C, n, L, pitch, four_sums(L, n, pitch, 1), stream);
 }
 
+template <int H>
+static cudaError_t set_tri_attrs() {
+    const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaError_t e = cudaFuncSetAttribute(limb_gemm_tri_kernel<H, kWords>, attr, TriCfg<H>::kSmemBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(limb_gemm_tri_kernel<H, kQuads>, attr, TriCfg<H>::kSmemBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(limb_gemm_tri_kernel<H, kTurned>, attr, TriCfg<H>::kSmemBytes);
+    return e;
+}
+
 cudaError_t prepare_limb_gemm_tri_kernels() {
-    cudaError_t e = cudaFuncSetAttribute(limb_gemm_tri_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         TriCfg<1>::kSmemBytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(limb_gemm_tri_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 TriCfg<2>::kSmemBytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(limb_gemm_tri_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 TriCfg<3>::kSmemBytes);
+    cudaError_t e = set_tri_attrs<1>();
+    if (e == cudaSuccess) e = set_tri_attrs<2>();
+    if (e == cudaSuccess) e = set_tri_attrs<3>();
     return e;
 }
 
@@ -692,7 +699,7 @@ static int tri_resident_pairs(int num_sms) {
     cudaLaunchConfig_t cfg = tri_config<H>(static_cast<unsigned>(num_sms / 2), nullptr, attr);
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, limb_gemm_tri_kernel<H>, &cfg) != cudaSuccess || n <= 0) {
+    if (cudaOccupancyMaxActiveClusters(&n, limb_gemm_tri_kernel<H, kWords>, &cfg) != cudaSuccess || n <= 0) {
         cudaGetLastError();
         return num_sms / 2;
     }
@@ -764,8 +771,12 @@ static cudaError_t launch_tri_t(const CUtensorMap &a_map, const CUtensorMap &b_m
     const uint64_t units = tiles * ranges;
     cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg = tri_config<H>(static_cast<unsigned>(units < pairs ? units : pairs), stream, attr);
-    return cudaLaunchKernelEx(&cfg, limb_gemm_tri_kernel<H>, a_map, b_map, sums, out, ld_m, ld_b, M, NV, KB, ranges,
-                              status);
+    const bool rows = ld_m != 1, quads = ld_m % 4 == 0 && (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
+    if (rows && ld_b != 1) return cudaErrorInvalidValue;
+    // 16-byte stores are for whole tiles: ranges add a word at a time
+    const auto kernel = !rows ? limb_gemm_tri_kernel<H, kWords>
+                              : (quads && ranges == 1 ? limb_gemm_tri_kernel<H, kQuads> : limb_gemm_tri_kernel<H, kTurned>);
+    return cudaLaunchKernelEx(&cfg, kernel, a_map, b_map, sums, out, rows ? ld_m : ld_b, M, NV, KB, ranges, status);
 }
 
 cudaError_t launch_limb_gemm_tri(const CUtensorMap &a_map, const CUtensorMap &b_map, const VecSums &sums,

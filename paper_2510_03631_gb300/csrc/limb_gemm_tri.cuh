@@ -43,7 +43,7 @@ double limb_gemm_tri_waves(uint32_t M, uint32_t NV, uint64_t K, int num_sms);
 // when the GEMM starts adding to it.
 uint32_t limb_gemm_tri_ranges(uint32_t M, uint32_t NV, uint64_t K, uint64_t ld_m, uint64_t ld_b, int num_sms);
 
-// out[i * ld_m + v * ld_b] = sum_j D[i][j] X[v][j] mod 2^32 (i < M, v < NV, j < K): a_map covers the
+// out[i * ld_m + v * ld_b] = sum_j D[i][j] X[v][j] mod 2^32 (i < M, v < NV, j < K; one of the strides is 1): a_map covers the
 // centred digits (box 64 x 128), b_map the limbs as (K, NV, 3) (box 64 x 32 x 3).
 // Launched as the programmatic dependent of the kernel before it in the stream, which makes the limbs (and
 // zeroes the output); everything earlier must have completed when that one starts.
