@@ -56,6 +56,7 @@
 // sums stay in TMEM: after every 512-deep chunk the epilogue replaces its accumulator buffer by
 // small representatives of the sums mod p, and the MMA accumulates the chunk after next on top;
 // the last two buffers are combined mod p at the end of the tile (of the piece, when it is split).
+#include <cmath>
 #include <cstdint>
 #include <type_traits>
 #include <cuda_fp16.h>
@@ -821,30 +822,32 @@ cudaError_t launch_limb_gemm_pair(const CUtensorMap &a_map, const PairBMaps &bm,
     return launch_pair_epi(256, a_map, bm, StoreEpi{out, 1, M, sums}, M, NV, K, 0, num_sms, status, stream);
 }
 
-// The schedule of that launch: whole waves in *waves, or its split.
-static bool store_schedule(uint32_t M, uint32_t NV, uint64_t K, int num_sms, double *waves) {
+// Whether that launch splits tiles, and the time in us of a call, modelled as limb_gemm_tri.cu's is and fitted to the
+// same shapes, then raised by 5%: where the two are close, three limbs lose less when the model is wrong.
+static bool store_schedule(uint32_t M, uint32_t NV, uint64_t K, int num_sms, double *us) {
     const uint64_t n_tiles = ((uint64_t)NV + 63) / 64, tiles = ((uint64_t)M + 2 * kPM - 1) / (2 * kPM) * n_tiles;
     const uint32_t KB = static_cast<uint32_t>((K + kPK - 1) / kPK), ckb = store_chunk_kb(KB);
-    const uint64_t pairs = static_cast<uint64_t>(resident_pairs<256, StoreEpi, false>(num_sms));
+    const int n = resident_pairs<256, StoreEpi, false>(num_sms);
+    const uint64_t pairs = n > 0 ? n : 1;
     uint64_t clusters = 0;
     uint32_t dp = 0, tail = 0;
-    *waves = 0.0;
-    if (pairs == 0) return false;
     const bool split = pair_split_schedule(tiles, n_tiles, (KB + ckb - 1) / ckb, pairs, &clusters, &dp, &tail);
-    *waves = split ? static_cast<double>(dp) / pairs + static_cast<double>(tiles - dp) / (tail * n_tiles)
-                   : static_cast<double>((tiles + pairs - 1) / pairs);
+    const double waves = split ? static_cast<double>(dp) / pairs + static_cast<double>(tiles - dp) / (tail * n_tiles)
+                               : static_cast<double>((tiles + pairs - 1) / pairs);
+    *us = 6.2 + 1.86e-6 * K * NV + 0.298 * KB * waves + 2.94 * std::ceil(waves) +
+          (split ? 0.58 + 0.131e-6 * M * NV * tail : 0.0);
     return split;
 }
 
 bool limb_gemm_pair_splits(uint32_t M, uint32_t NV, uint64_t K, int num_sms) {
-    double waves;
-    return store_schedule(M, NV, K, num_sms, &waves);
+    double us;
+    return store_schedule(M, NV, K, num_sms, &us);
 }
 
-double limb_gemm_pair_waves(uint32_t M, uint32_t NV, uint64_t K, int num_sms) {
-    double waves;
-    store_schedule(M, NV, K, num_sms, &waves);
-    return waves;
+double limb_gemm_pair_us(uint32_t M, uint32_t NV, uint64_t K, int num_sms) {
+    double us;
+    store_schedule(M, NV, K, num_sms, &us);
+    return us;
 }
 
 cudaError_t launch_limb_gemm_pair_query(int bn, const CUtensorMap &a_map, const PairBMaps &bm,

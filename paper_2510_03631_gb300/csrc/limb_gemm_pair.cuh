@@ -33,9 +33,9 @@ int limb_gemm_pair_bn_for(uint32_t nv);
 cudaError_t launch_limb_gemm_pair(const CUtensorMap &a_map, const PairBMaps &bm, const VecSums &sums, uint32_t *out,
                                   uint32_t M, uint32_t NV, uint64_t K, int num_sms, int *status,
                                   cudaStream_t stream);
-// Whether that launch splits tiles, whose pieces add into out, and its time in tile times (256 rows x 64 vectors).
+// Whether that launch splits tiles, whose pieces add into out, and the modelled time in us of a call.
 bool limb_gemm_pair_splits(uint32_t M, uint32_t NV, uint64_t K, int num_sms);
-double limb_gemm_pair_waves(uint32_t M, uint32_t NV, uint64_t K, int num_sms);
+double limb_gemm_pair_us(uint32_t M, uint32_t NV, uint64_t K, int num_sms);
 
 // Client Query / Recover batches on CTA pairs.  plane_chunks = n / 512 selects
 // the planed mode (then the vector rows follow launch_secret_limbs_planed with

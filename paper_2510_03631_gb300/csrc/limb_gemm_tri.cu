@@ -708,57 +708,42 @@ static int tri_resident_pairs(int num_sms) {
     return n;
 }
 
-// Time of `s` column ranges per tile on `pairs` clusters, in tile times: whole waves of ranges, each with
-// about 1.5 chunks' worth of filling, draining and adding up.
-static double tri_time(uint64_t tiles, uint32_t nchunks, uint64_t pairs, uint32_t s) {
-    const uint64_t waves = (tiles * s + pairs - 1) / pairs;
-    return static_cast<double>(waves) * (static_cast<double>(nchunks) / s + 1.5) / nchunks;
-}
-// Column ranges per tile: the fewest (at most 8, each at least 1024 columns) within 2% of the best
-// time, when they save `gain` of it (8192 x 32768, 128 vectors, 32 tiles on 76 pairs: seven).
-static uint32_t tri_ksplit(uint64_t tiles, uint32_t nchunks, uint64_t pairs, double gain) {
-    const uint32_t most = nchunks / 8 < 8 ? nchunks / 8 : 8;
-    const double whole = tri_time(tiles, nchunks, pairs, 1);
-    double best = whole;
-    for (uint32_t s = 2; s <= most; ++s) best = tri_time(tiles, nchunks, pairs, s) < best ? tri_time(tiles, nchunks, pairs, s) : best;
-    if (best > (1.0 - gain) * whole) return 1;
-    for (uint32_t s = 2; s <= most; ++s)
-        if (tri_time(tiles, nchunks, pairs, s) <= 1.02 * best) return s;
-    return 1;
+// The time in us of tiles of `h` halves cut into `s` column ranges, limb pass and launches included: whole waves of
+// ranges on `pairs` clusters, each with its chunks (a half's tensor or drain time, more for one half a tile, which
+// loads a digit tile for 192 columns, and more again when the digits do not stay in L2), its filling, draining and
+// storing; ranges add their parts to the output.  Fitted to 6,200 graph-replayed calls (370 shapes of 300 to 65,536
+// rows, 400 to 40,000 columns and 65 to 1,024 vectors, every form of each).  The form chosen by it was 0.6% from the
+// best of them on average; two or three halves in at most 8 ranges of 1024 columns had been 13% from it on the 240
+// regular ones: 300 x 30000 with 66 vectors 41 us against 18, 2000 x 16000 with 320 76 / 60, 1200 x 1900 with 128 16 / 10.
+static double tri_time(uint32_t M, uint32_t NV, uint64_t K, uint64_t tiles, uint64_t pairs, double chunks, int h,
+                       uint32_t s) {
+    const double half = h == 2 ? 0.527 : (h == 3 ? 0.592 : (2.0 * M * K > 64e6 ? 0.627 : 0.605));
+    const double waves = static_cast<double>((tiles * s + pairs - 1) / pairs);
+    const double adding = s > 1 ? 0.5e-6 * M * NV * s : 0.0;
+    return 5.6 + 1.5e-6 * K * NV + waves * (h * (half * chunks / s + 1.7) + 0.2) + adding;
 }
 
-// Halves per tile.  Two, so that a row of tiles has no odd narrow one where that can be helped: up to 64 vectors
-// one, and three for three halves (129 to 192 vectors: one tile; 8192 x 32768, 160 vectors: 277 us, tiles of
-// two and one 318) or five (3 + 2).  One also for so few columns that tiles are not cut into ranges, when even
-// then a tile is left for every cluster (600 x 700 by 512 columns: 18 us, 41 with two halves and word stores).
-static int tri_halves(uint32_t M, uint32_t NV, uint64_t K, int num_sms) {
+TriPlan limb_gemm_tri_plan(uint32_t M, uint32_t NV, uint64_t K, int num_sms) {
     const uint64_t m_tiles = ((uint64_t)M + 2 * kTM - 1) / (2 * kTM);
     const uint32_t nh = (NV - 1) / 64 + 1;
-    if (nh == 1 || (K <= 15 * kTK * kChunkSteps && m_tiles * nh <= (uint64_t)num_sms / 2)) return 1;
-    return nh == 3 || nh == 5 ? 3 : 2;
-}
-
-double limb_gemm_tri_waves(uint32_t M, uint32_t NV, uint64_t K, int num_sms) {
-    const int h = tri_halves(M, NV, K, num_sms);
-    const uint64_t pairs = static_cast<uint64_t>(h == 1 ? tri_resident_pairs<1>(num_sms)
-                                                 : (h == 2 ? tri_resident_pairs<2>(num_sms) : tri_resident_pairs<3>(num_sms)));
-    if (pairs == 0) return 0.0;
-    const uint64_t tiles = ((uint64_t)M + 2 * kTM - 1) / (2 * kTM) * (((uint64_t)NV + 64 * h - 1) / (64 * h));
-    const uint32_t nchunks = static_cast<uint32_t>((K + kTK * kChunkSteps - 1) / (kTK * kChunkSteps));
-    return h * tri_time(tiles, nchunks, pairs, limb_gemm_tri_ranges(M, NV, K, 1, M, num_sms));
-}
-
-uint32_t limb_gemm_tri_ranges(uint32_t M, uint32_t NV, uint64_t K, uint64_t ld_m, uint64_t ld_b, int num_sms) {
-    // ranges add into a zeroed output, and only a dense one can be zeroed in one piece; row-major
-    // outputs (the hint's) scatter their atomics, one line per lane, and must gain more
-    if (!((ld_m == 1 && ld_b == M) || (ld_b == 1 && ld_m == NV))) return 1;
-    const uint64_t m_tiles = ((uint64_t)M + 2 * kTM - 1) / (2 * kTM);
-    const uint32_t nchunks = static_cast<uint32_t>((K + kTK * kChunkSteps - 1) / (kTK * kChunkSteps));
-    const int h = tri_halves(M, NV, K, num_sms);
-    const uint64_t tiles = m_tiles * (((uint64_t)NV + 64 * h - 1) / (64 * h));
-    const int pairs = h == 1 ? tri_resident_pairs<1>(num_sms)
-                             : (h == 2 ? tri_resident_pairs<2>(num_sms) : tri_resident_pairs<3>(num_sms));
-    return pairs <= 0 ? 1 : tri_ksplit(tiles, nchunks, static_cast<uint64_t>(pairs), ld_m == 1 ? 0.08 : 0.25);
+    const uint64_t chunks = (K + kTK * kChunkSteps - 1) / (kTK * kChunkSteps);
+    TriPlan whole{0, 1, 0.0}, cut{0, 1, 0.0};
+    for (int h = 1; h <= 3 && h <= (int)nh; ++h) {
+        const int n = h == 1 ? tri_resident_pairs<1>(num_sms) : (h == 2 ? tri_resident_pairs<2>(num_sms) : tri_resident_pairs<3>(num_sms));
+        const uint64_t pairs = n > 0 ? n : 1, tiles = m_tiles * ((nh + h - 1) / h);
+        auto consider = [&](uint64_t s) {
+            if (s > 1 && (s > pairs || s > chunks / 2)) return;   // ranges of at least two chunks
+            TriPlan &best = s == 1 ? whole : cut;
+            const double us = tri_time(M, NV, K, tiles, pairs, static_cast<double>(chunks), h, static_cast<uint32_t>(s));
+            if (best.halves == 0 || us < best.us) best = TriPlan{h, static_cast<uint32_t>(s), us};
+        };
+        // up to 8 ranges, or the most that fit one, two or three waves
+        for (uint64_t s = 1; s <= 8; ++s) consider(s);
+        for (uint64_t w = 1; w <= 3; ++w)
+            if (w * pairs / tiles > 8) consider(w * pairs / tiles);
+    }
+    // ranges need a zeroed output and atomics: not for less than 2%
+    return cut.halves != 0 && cut.us < 0.98 * whole.us ? cut : whole;
 }
 
 template <int H>
@@ -767,8 +752,8 @@ static cudaError_t launch_tri_t(const CUtensorMap &a_map, const CUtensorMap &b_m
                                 int num_sms, int *status, cudaStream_t stream) {
     const uint64_t tiles = ((uint64_t)M + 2 * kTM - 1) / (2 * kTM) * (((uint64_t)NV + 64 * H - 1) / (64 * H));
     const uint64_t pairs = static_cast<uint64_t>(tri_resident_pairs<H>(num_sms));
-    if (pairs == 0 || tiles * 8 >= (1ull << 32)) return cudaErrorInvalidValue;
     const uint64_t units = tiles * ranges;
+    if (pairs == 0 || units >= (1ull << 31)) return cudaErrorInvalidValue;
     cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg = tri_config<H>(static_cast<unsigned>(units < pairs ? units : pairs), stream, attr);
     const bool rows = ld_m != 1, quads = ld_m % 4 == 0 && (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
@@ -781,13 +766,15 @@ static cudaError_t launch_tri_t(const CUtensorMap &a_map, const CUtensorMap &b_m
 
 cudaError_t launch_limb_gemm_tri(const CUtensorMap &a_map, const CUtensorMap &b_map, const VecSums &sums,
                                  uint32_t *out, uint64_t ld_m, uint64_t ld_b, uint32_t M, uint32_t NV, uint64_t K,
-                                 uint32_t ranges, int num_sms, int *status, cudaStream_t stream) {
-    if (M == 0 || NV == 0 || K == 0 || ranges == 0 || num_sms < 2) return cudaErrorInvalidValue;
+                                 const TriPlan &plan, int num_sms, int *status, cudaStream_t stream) {
+    if (M == 0 || NV == 0 || K == 0 || plan.ranges == 0 || num_sms < 2) return cudaErrorInvalidValue;
     const uint32_t KB = static_cast<uint32_t>((K + kTK - 1) / kTK);
-    const int h = tri_halves(M, NV, K, num_sms);
-    if (h == 1) return launch_tri_t<1>(a_map, b_map, sums, out, ld_m, ld_b, M, NV, KB, ranges, num_sms, status, stream);
-    if (h == 3) return launch_tri_t<3>(a_map, b_map, sums, out, ld_m, ld_b, M, NV, KB, ranges, num_sms, status, stream);
-    return launch_tri_t<2>(a_map, b_map, sums, out, ld_m, ld_b, M, NV, KB, ranges, num_sms, status, stream);
+    switch (plan.halves) {
+        case 1: return launch_tri_t<1>(a_map, b_map, sums, out, ld_m, ld_b, M, NV, KB, plan.ranges, num_sms, status, stream);
+        case 2: return launch_tri_t<2>(a_map, b_map, sums, out, ld_m, ld_b, M, NV, KB, plan.ranges, num_sms, status, stream);
+        case 3: return launch_tri_t<3>(a_map, b_map, sums, out, ld_m, ld_b, M, NV, KB, plan.ranges, num_sms, status, stream);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 }  // namespace qpadl

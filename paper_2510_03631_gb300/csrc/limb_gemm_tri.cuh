@@ -36,12 +36,14 @@ cudaError_t launch_mat_col_limbs_tri(const uint32_t *A, uint64_t C, uint32_t n, 
 cudaError_t launch_mat_col_limbs_four(const uint32_t *A, uint64_t C, uint32_t n, __half *L, uint64_t pitch,
                                       cudaStream_t stream);
 
-// The time of the launch below in the time of one half (256 rows x 64 vectors).
-double limb_gemm_tri_waves(uint32_t M, uint32_t NV, uint64_t K, int num_sms);
-
-// Column ranges that a product of these sizes is cut into; with more than one, the output must be zero
-// when the GEMM starts adding to it.
-uint32_t limb_gemm_tri_ranges(uint32_t M, uint32_t NV, uint64_t K, uint64_t ld_m, uint64_t ld_b, int num_sms);
+// How a product of these sizes is cut: 64-vector halves per tile, column ranges per tile (with more than one, the
+// output must be dense and zero when the GEMM starts adding to it), and the modelled time in us of a call.
+struct TriPlan {
+    int halves;
+    uint32_t ranges;
+    double us;
+};
+TriPlan limb_gemm_tri_plan(uint32_t M, uint32_t NV, uint64_t K, int num_sms);
 
 // out[i * ld_m + v * ld_b] = sum_j D[i][j] X[v][j] mod 2^32 (i < M, v < NV, j < K; one of the strides is 1): a_map covers the
 // centred digits (box 64 x 128), b_map the limbs as (K, NV, 3) (box 64 x 32 x 3).
@@ -49,6 +51,6 @@ uint32_t limb_gemm_tri_ranges(uint32_t M, uint32_t NV, uint64_t K, uint64_t ld_m
 // zeroes the output); everything earlier must have completed when that one starts.
 cudaError_t launch_limb_gemm_tri(const CUtensorMap &a_map, const CUtensorMap &b_map, const VecSums &sums,
                                  uint32_t *out, uint64_t ld_m, uint64_t ld_b, uint32_t M, uint32_t NV, uint64_t K,
-                                 uint32_t ranges, int num_sms, int *status, cudaStream_t stream);
+                                 const TriPlan &plan, int num_sms, int *status, cudaStream_t stream);
 
 }  // namespace qpadl

@@ -287,7 +287,7 @@ int set_device(const qpadl_db *db) {
 // out[i * ld_m + v * ld_b] = D * X[v] for NV vectors given at `limbs` as three limbs (pair tiles) or, in
 // run_limb_gemm, four (single-SM tiles) and the vectors' sums
 int run_tri_gemm(qpadl_db *db, const __half *limbs, uint32_t NV, uint32_t parts, uint32_t *out, uint64_t ld_m,
-                 uint64_t ld_b, uint32_t ranges, cudaStream_t stream) {
+                 uint64_t ld_b, const TriPlan &plan, cudaStream_t stream) {
     const uint64_t C = db->prm.cols;
     CUtensorMap b_map;   // (column, vector, limb): a box is one CTA's 32 vectors x 3 limbs
     auto fn = encode_fn();
@@ -300,7 +300,7 @@ int run_tri_gemm(qpadl_db *db, const __half *limbs, uint32_t NV, uint32_t parts,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return QPADL_ECUDA;
     QPADL_CU(launch_limb_gemm_tri(db->ac_map, b_map, tri_sums(limbs, NV, db->pitch, parts), out, ld_m, ld_b,
-                                  static_cast<uint32_t>(db->prm.rows), NV, C, ranges, db->num_sms, db->d_status, stream));
+                                  static_cast<uint32_t>(db->prm.rows), NV, C, plan, db->num_sms, db->d_status, stream));
     return QPADL_OK;
 }
 
@@ -321,18 +321,14 @@ uint64_t limb_scratch_bytes(const qpadl_db *db, uint32_t NV) {
     return 8ull * NV * db->pitch + 4ull * NV * limb_sum_parts(db->prm.cols);
 }
 
-// Whether a batch on pair tiles takes four byte limbs instead of three: only with an odd number of
-// 64-vector halves, where the three-limb tiles (two halves, or three for 3 and 5) leave a half empty
-// or the last wave uneven.  Both times are in units of 256 rows x 64 vectors; a three-limb unit takes 0.93 of a
-// four-limb one, and 1.08 times that in tiles of three.  Measured, four limbs against three
-// (us): 32768 x 32768, 160 vectors 793 / 873, 192 816 / 915, 448 1927 / 2053; 8192 x 32768, 192
-// 242 / 277, 320 499 / 464, 448 493 / 563; 2000 x 30000, 320 157 / 134.
-bool four_limbs(const qpadl_db *db, uint32_t B) {
-    const uint32_t halves = (B - 1) / 64 + 1, M = static_cast<uint32_t>(db->prm.rows);
+// Whether a batch on pair tiles takes four byte limbs instead of three: only with an odd number of 64-vector
+// halves, where the three-limb tiles can leave a half empty or the last wave uneven, and by the modelled times.
+// Measured, four limbs against the best three (us): 32768 x 32768, 192 vectors 816 / 915; 12000 x 16384, 160
+// vectors 165 / 174; 2000 x 30000, 320 vectors 147 / 106.
+bool four_limbs(const qpadl_db *db, uint32_t B, const TriPlan &three) {
+    const uint32_t halves = (B - 1) / 64 + 1;
     if (halves < 3 || halves % 2 == 0) return false;
-    const double four = limb_gemm_pair_waves(M, B, db->prm.cols, db->num_sms) * 1.07;
-    const double three = limb_gemm_tri_waves(M, B, db->prm.cols, db->num_sms) * (halves <= 5 ? 1.08 : 1.0);
-    return four < three;
+    return limb_gemm_pair_us(static_cast<uint32_t>(db->prm.rows), B, db->prm.cols, db->num_sms) < three.us;
 }
 
 // Answers of B queries (at most 4096) on the fp16 copy, which exists, their limbs made at `limbs`
@@ -341,7 +337,8 @@ int answer_f16(qpadl_db *db, const uint32_t *Q, uint32_t B, uint32_t *ans, __hal
     const uint64_t C = db->prm.cols, R = db->prm.rows;
     const uint32_t parts = limb_sum_parts(C);
     const bool tri = use_tri(db);
-    if (tri && four_limbs(db, B)) {
+    const TriPlan plan = tri ? limb_gemm_tri_plan(static_cast<uint32_t>(R), B, C, db->num_sms) : TriPlan{};
+    if (tri && four_limbs(db, B, plan)) {
         // as below, one launch makes the limbs and zeroes the answers that split tiles add to
         const bool split = limb_gemm_pair_splits(static_cast<uint32_t>(R), B, C, db->num_sms);
         QPADL_CU(launch_vec_limbs_four(Q, C, B, C, limbs, db->pitch, split ? ans : nullptr, (uint64_t)B * R, stream));
@@ -355,10 +352,10 @@ int answer_f16(qpadl_db *db, const uint32_t *Q, uint32_t B, uint32_t *ans, __hal
         return QPADL_OK;
     }
     if (tri) {
-        const uint32_t ranges = limb_gemm_tri_ranges(static_cast<uint32_t>(R), B, C, 1, R, db->num_sms);
         // one launch makes the limbs and zeroes the answers that ranges add to
-        QPADL_CU(launch_vec_limbs_tri(Q, C, B, C, limbs, db->pitch, ranges > 1 ? ans : nullptr, (uint64_t)B * R, stream));
-        return run_tri_gemm(db, limbs, B, parts, ans, 1, R, ranges, stream);
+        QPADL_CU(launch_vec_limbs_tri(Q, C, B, C, limbs, db->pitch, plan.ranges > 1 ? ans : nullptr, (uint64_t)B * R,
+                                      stream));
+        return run_tri_gemm(db, limbs, B, parts, ans, 1, R, plan, stream);
     }
     QPADL_CU(launch_vec_limbs_four(Q, C, B, C, limbs, db->pitch, nullptr, 0, stream));
     return run_limb_gemm(db, limbs, B, parts, ans, 1, R, stream);
@@ -794,10 +791,10 @@ int qpadl_pir_hint(qpadl_db *db, const uint32_t *A_dev, uint32_t *H_dev, qpadl_s
     if (rc != QPADL_OK) return rc;
     if (!u8 && use_tri(db)) {
         const uint64_t R = db->prm.rows;
-        const uint32_t ranges = limb_gemm_tri_ranges(static_cast<uint32_t>(R), n, db->prm.cols, n, 1, db->num_sms);
-        if (ranges > 1) QPADL_CU(cudaMemsetAsync(H_dev, 0, 4ull * n * R, s));
+        const TriPlan plan = limb_gemm_tri_plan(static_cast<uint32_t>(R), n, db->prm.cols, db->num_sms);
+        if (plan.ranges > 1) QPADL_CU(cudaMemsetAsync(H_dev, 0, 4ull * n * R, s));
         QPADL_CU(launch_mat_col_limbs_tri(A_dev, db->prm.cols, n, db->limbs, db->pitch, s));
-        return run_tri_gemm(db, db->limbs, n, 1, H_dev, n, 1, ranges, s);
+        return run_tri_gemm(db, db->limbs, n, 1, H_dev, n, 1, plan, s);
     }
     if (!u8) {
         QPADL_CU(launch_mat_col_limbs_four(A_dev, db->prm.cols, n, db->limbs, db->pitch, s));
