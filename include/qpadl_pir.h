@@ -490,14 +490,16 @@ typedef struct qpadl_chor qpadl_chor;
 
 /* Binds a resident database (db_dev: rows x bits/32 uint32 words, caller-
  * owned, 16-byte aligned, kept until destroy) on the current device and
- * allocates the handle's scratch (32 bytes per row; 64 up to 2^18 rows).  QPADL_EINVAL if rows
+ * allocates the handle's scratch (32 bytes per row; for up to 2^18 rows at least 512, at most 16 MiB).
+ * QPADL_EINVAL if rows
  * is 0 or >= 2^31, bits is not a positive multiple of 128, or db_dev is
  * NULL or misaligned. */
 int qpadl_chor_setup(uint64_t rows, uint64_t bits, const uint32_t *db_dev, qpadl_stream_t stream,
                      qpadl_chor **out);
 
 /* Answers B queries (Q_dev: B x ceil(rows/32) words, query b in row b) in
- * one pass over the database per 128 (tensor cores) or 256 (scan) queries; out_dev: B x bits/32 words
+ * one pass over the database per 128 to 1024 (tensor cores, as the scratch allows) or 256 (scan)
+ * queries; out_dev: B x bits/32 words
  * (answer b in row b), overwritten.  Calls on one handle share its scratch:
  * issue them on one stream (or order them). */
 int qpadl_chor_answer_batch(qpadl_chor *h, const uint32_t *Q_dev, uint32_t B, uint32_t *out_dev,
@@ -509,8 +511,9 @@ int qpadl_chor_answer_batch(qpadl_chor *h, const uint32_t *Q_dev, uint32_t B, ui
  *   of 4-bit products); smaller ones the masked-XOR scan.  257 disables the
  *   tensor cores.  Until it or QPADL_CHOR_OPT_SCAN_FORM is set, the library
  *   chooses by record length (1 below 512 words, 3 below 1024, else 9), also
- *   for what a chunk leaves after its first 128 queries, and the option reads
- *   as that number. */
+ *   for what a larger batch leaves after its tiles of 128 queries (which a
+ *   database of up to 64 MiB takes along), and the option reads as that
+ *   number. */
 #define QPADL_CHOR_OPT_M4RM_MIN_BATCH 1
 /* QPADL_CHOR_OPT_SCAN_FORM (-1..3, default -1): inner loop of the masked-XOR
  * scan.  Bit 1: each thread covers 8 database words per row (at most 16

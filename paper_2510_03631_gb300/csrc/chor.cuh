@@ -25,14 +25,21 @@ cudaError_t launch_chor_answer(const CUtensorMap &db_map, const CUtensorMap &qt_
                                uint32_t B, uint32_t qtw, uint32_t *out, int num_sms, int *status,
                                cudaStream_t stream, int form);
 
-// Tensor-core path (chor_gemm.cu): units of 256 rows x 16 words, up to 128 queries per pass.
+// Tensor-core path (chor_gemm.cu): units of 256 rows x 16 words, tiles of up to 128 queries.
 constexpr uint32_t kChorGemmUnitRows = 256;
 constexpr uint32_t kChorGemmUnitWords = 16;
-constexpr uint32_t kChorGemmMaxBatch = 128;
-// Rows per launch: bounds the expanded queries (64 bytes per row) and, far below 2^22, the counts.
+constexpr uint32_t kChorGemmTile = 128;
+// Rows per launch: bounds the expanded queries and, far below 2^22, the counts.
 constexpr uint64_t kChorGemmRows = 1ull << 18;
-// Bytes of expanded queries for B queries of `units` units.
-constexpr uint64_t chor_gemm_query_bytes(uint32_t B, uint32_t units) { return 128ull * B * units; }
+// Queries per launch over `units` units: tiles whose expanded bits (128 bytes per query and unit) stay within
+// 16 MiB, one at 2^18 rows, at most 1024 queries.
+constexpr uint32_t chor_gemm_group(uint32_t units) {
+    return units <= 128 ? 1024u : (16u << 20) / (128u * kChorGemmTile * units) * kChorGemmTile;
+}
+constexpr uint64_t chor_gemm_scratch(uint32_t units) { return 128ull * chor_gemm_group(units) * units; }
+// Up to this many units x column tiles, what a batch leaves for its last tile shares the launch of the others even when
+// it is narrow: a launch of its own costs about 9 us, 128 instead of 64 columns of MMAs 2.2 ns per unit and tile.
+constexpr uint64_t kChorGemmSmall = 4096;
 
 cudaError_t prepare_chor_gemm_kernels();
 // Query rows of a tile (32, 64 or 128) for B queries: the box height of q_map.
@@ -43,7 +50,7 @@ uint32_t chor_gemm_n(uint32_t B);
 cudaError_t launch_chor_nibbles(const uint32_t *Q, uint64_t qw, uint32_t B, uint64_t row0, uint32_t units, uint32_t *QF,
                                 cudaStream_t stream);
 
-// out (B x W words, zeroed by the caller) ^= the responses of B <= 128 queries over the rows
+// out (B x W words, zeroed by the caller) ^= the responses of B queries over the rows
 // [row0, row0 + 256 units); db_map covers the database {W, r} words with box {16, 256} and 64-byte swizzle, q_map QF
 // {128 units, B} bytes with box {128, chor_gemm_n(B)} and 128-byte swizzle.
 cudaError_t launch_chor_gemm(const CUtensorMap &db_map, const CUtensorMap &q_map, uint64_t row0, uint32_t units,

@@ -24,8 +24,9 @@
 // A unit is 16 database words (64 bytes per row) x 256 rows.  Up to 64 queries a CTA runs all four
 // planes (accumulators 4 x 64 TMEM columns); up to 128 queries two CTAs take two planes each
 // (2 x 128 columns), both reading and transposing the same words, the second from L2: the tensor
-// work of 128 queries outweighs it.  Larger batches take several passes (a tile of 256 queries would
-// leave room for one plane, so each unit would be transposed four times).
+// work of 128 queries outweighs it.  Larger batches are several tiles of 128 queries (a tile of 256 queries would
+// leave room for one plane, so each unit would be transposed four times), in one launch as far as the scratch
+// holds their expanded bits.
 //
 // Measured (2^18 records of 3 KB, 805 MB): 64 queries 195 us, 128 queries 303 us; the kernels it
 // replaced took 1,085 and 1,130 us there (four-Russians tables in shared memory) and 606 us at 32
@@ -120,17 +121,19 @@ __device__ __forceinline__ void ldmatrix_bytes(uint32_t addr, uint32_t &a0, uint
 // parity (step 1's stores), so neither meets bank conflicts.
 __device__ __forceinline__ uint32_t x_perm(uint32_t L) { return (L ^ ((L & 7u) >> 1) ^ (L >> 3)) & 7u; }
 
-// A CTA's pieces: p = blockIdx.x, blockIdx.x + gridDim.x, ...
+// A CTA's pieces: p = blockIdx.x, blockIdx.x + gridDim.x, ...; the query tiles of one column tile and band are
+// neighbours, so the database is read from HBM once for all of them.
 struct GPiece {
-    uint32_t tile, u0, u1;   // column tile, units [u0, u1) along the rows
+    uint32_t tile, q, u0, u1;   // column tile, query tile, units [u0, u1) along the rows
 };
 struct GPieceIter {
     uint32_t p;
     __device__ __forceinline__ GPieceIter() : p(blockIdx.x) {}
-    __device__ __forceinline__ bool next(GPiece &pc, uint32_t tiles, uint32_t bands, uint32_t units) {
-        if (p >= tiles * bands) return false;
-        const uint32_t band = p / tiles;
-        pc.tile = p - band * tiles;
+    __device__ __forceinline__ bool next(GPiece &pc, uint32_t tiles, uint32_t qtiles, uint32_t bands, uint32_t units) {
+        if (p >= tiles * qtiles * bands) return false;
+        const uint32_t t = p / qtiles, band = t / tiles;
+        pc.q = p - t * qtiles;
+        pc.tile = t - band * tiles;
         pc.u0 = static_cast<uint32_t>((uint64_t)band * units / bands);
         pc.u1 = static_cast<uint32_t>((uint64_t)(band + 1) * units / bands);
         p += gridDim.x;
@@ -143,10 +146,11 @@ struct GPieceIter {
 template <int N, int MT>
 __global__ void __launch_bounds__(kGThreads, 1)
     chor_gemm_kernel(const __grid_constant__ CUtensorMap db_map, const __grid_constant__ CUtensorMap q_map, uint32_t row0,
-                     uint32_t units, uint32_t tiles, uint32_t bands, uint32_t W, uint32_t B, uint32_t *__restrict__ out,
-                     int *__restrict__ status) {
+                     uint32_t units, uint32_t tiles, uint32_t qtiles, uint32_t bands, uint32_t W, uint32_t B,
+                     uint32_t *__restrict__ out, int *__restrict__ status) {
     using Cfg = GCfg<N, MT>;
     constexpr int SQ = Cfg::kQSlots, SETS = Cfg::kSets;
+    if constexpr (MT == 4) qtiles = 1;   // narrow tiles take one batch each
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t *raw = smem, *xt = smem + kRawSlots * kRawBytes, *qt = smem + Cfg::kQBase;
@@ -228,7 +232,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
             const uint32_t slots = db ? kRawSlots : SQ;
             uint32_t it = 0, sl = 0, ph = 0;
             tma_prefetch_desc(map);
-            while (!failed && pit.next(pc, tiles, bands, units)) {
+            while (!failed && pit.next(pc, tiles, qtiles, bands, units)) {
                 const int32_t x = static_cast<int32_t>((MT == 4 ? pc.tile : pc.tile >> 1) * kUnitWords);
                 for (uint32_t u = pc.u0; u < pc.u1; ++u, ++it) {
                     if (!mbar_wait(&free_[sl], ph ^ 1u, abort)) {
@@ -240,7 +244,8 @@ __global__ void __launch_bounds__(kGThreads, 1)
                         tma_load_2d(raw + sl * kRawBytes, map, &full[sl], x, static_cast<int32_t>(row0 + u * kUnitRows));
                     } else {
                         mbar_arrive_expect_tx(&full[sl], Cfg::kQBytes);
-                        tma_load_2d(qt + sl * Cfg::kQBytes, map, &full[sl], static_cast<int32_t>(u * 128u), 0);
+                        tma_load_2d(qt + sl * Cfg::kQBytes, map, &full[sl], static_cast<int32_t>(u * 128u),
+                                    static_cast<int32_t>(pc.q * N));
                     }
                     if (++sl == slots) {
                         sl = 0;
@@ -261,7 +266,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
         constexpr int PW = MT / kIssuers;                // planes per issuer
         const uint32_t s0 = warp == 1 ? 0u : PW;
         uint32_t it = 0, is = 0, np = 0;                 // units, sets, pieces
-        while (!failed && pit.next(pc, tiles, bands, units)) {
+        while (!failed && pit.next(pc, tiles, qtiles, bands, units)) {
             bool ok = mbar_wait(acc_free, (np & 1u) ^ 1u, abort);
             for (uint32_t u = pc.u0; u < pc.u1; ++u, ++it) {
                 const uint32_t q = it % SQ;
@@ -307,7 +312,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
         // ---------------- epilogue
         const uint32_t lane_addr = (quarter * 32u) << 16;
         uint32_t np = 0;
-        while (!failed && pit.next(pc, tiles, bands, units)) {
+        while (!failed && pit.next(pc, tiles, qtiles, bands, units)) {
             const bool ok = mbar_wait(acc_full, np & 1u, abort);
             if (__any_sync(0xffffffffu, !ok)) {
                 fail_here();
@@ -340,7 +345,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
                     __syncwarp();
                     if (lane == 0) mbar_arrive(acc_free);
                 }
-                const uint32_t b = n0 + static_cast<uint32_t>(lane);
+                const uint32_t b = pc.q * N + n0 + static_cast<uint32_t>(lane);
                 if (b < B) {
 #pragma unroll
                     for (uint32_t wl = 0; wl < 4; ++wl) {
@@ -366,7 +371,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
         const uint32_t laddr = lrow * 64u + ((v ^ ((lrow >> 1) & 3u)) << 4);
         const uint32_t c = ul >> 2, gi = ul & 3u;
         uint32_t it = 0;
-        while (!failed && pit.next(pc, tiles, bands, units)) {
+        while (!failed && pit.next(pc, tiles, qtiles, bands, units)) {
             for (uint32_t u = pc.u0; u < pc.u1; ++u, ++it) {
                 if ((it & 1u) != group) continue;
                 const uint32_t r = it % kRawSlots, x = it % kXSlots;
@@ -410,7 +415,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
         const uint32_t perm = x_perm(L);
         const uint32_t lane_addr = (quarter * 32u) << 16;
         uint32_t it = 0;
-        while (!failed && pit.next(pc, tiles, bands, units)) {
+        while (!failed && pit.next(pc, tiles, qtiles, bands, units)) {
             const bool upper = MT == 2 && (pc.tile & 1u);   // planes 2 and 3
             for (uint32_t u = pc.u0; u < pc.u1; ++u, ++it) {
                 if ((it & 1u) != group) continue;
@@ -557,12 +562,13 @@ static uint32_t chor_bands(uint32_t tiles, uint32_t units, uint32_t sms) {
 template <int N, int MT>
 static cudaError_t launch_gemm_t(const CUtensorMap &db_map, const CUtensorMap &q_map, uint32_t row0, uint32_t units,
                                  uint32_t W, uint32_t B, uint32_t *out, int num_sms, int *status, cudaStream_t stream) {
-    const uint32_t tiles = (W + kUnitWords - 1) / kUnitWords * (4 / MT);
-    const uint32_t bands = chor_bands(tiles, units, static_cast<uint32_t>(num_sms));
-    const uint64_t pieces = (uint64_t)tiles * bands;
+    const uint32_t tiles = (W + kUnitWords - 1) / kUnitWords * (4 / MT), qtiles = (B + N - 1) / N;
+    const uint32_t bands = chor_bands(tiles * qtiles, units, static_cast<uint32_t>(num_sms));
+    const uint64_t pieces = (uint64_t)tiles * qtiles * bands;
+    if (pieces >= (1ull << 31)) return cudaErrorInvalidValue;
     const unsigned grid = static_cast<unsigned>(pieces < (uint64_t)num_sms ? pieces : (uint64_t)num_sms);
-    chor_gemm_kernel<N, MT><<<grid, kGThreads, GCfg<N, MT>::kSmemBytes, stream>>>(db_map, q_map, row0, units, tiles, bands,
-                                                                                 W, B, out, status);
+    chor_gemm_kernel<N, MT><<<grid, kGThreads, GCfg<N, MT>::kSmemBytes, stream>>>(db_map, q_map, row0, units, tiles, qtiles,
+                                                                                 bands, W, B, out, status);
     return cudaGetLastError();
 }
 

@@ -1315,10 +1315,11 @@ int qpadl_chor_setup(uint64_t rows, uint64_t bits, const uint32_t *db_dev, qpadl
         return fail(QPADL_ECUDA);
     int rc = prepare_device(h->device);
     if (rc != QPADL_OK) return fail(rc);
-    // selector bits of the scans, or one launch's expanded queries of the tensor-core path
-    const uint64_t block_rows = std::min<uint64_t>(rows, kChorGemmRows);
-    const uint64_t qt_bytes =
-        std::max<uint64_t>(32 * rows, chor_gemm_query_bytes(kChorGemmMaxBatch, chor_units(block_rows)));
+    // selector bits of the scans, or one launch's expanded queries of the tensor-core path (the last block of rows may be
+    // shorter and then takes more queries)
+    uint64_t qt_bytes = std::max<uint64_t>(32 * rows, chor_gemm_scratch(chor_units(std::min(rows, kChorGemmRows))));
+    if (rows > kChorGemmRows && rows % kChorGemmRows)
+        qt_bytes = std::max(qt_bytes, chor_gemm_scratch(chor_units(rows % kChorGemmRows)));
     if (cudaMalloc(reinterpret_cast<void **>(&h->qt), qt_bytes) != cudaSuccess ||
         cudaMalloc(reinterpret_cast<void **>(&h->d_status), 16) != cudaSuccess) {
         cudaGetLastError();
@@ -1335,7 +1336,11 @@ int qpadl_chor_setup(uint64_t rows, uint64_t bits, const uint32_t *db_dev, qpadl
 
 namespace {
 
-// Up to 128 queries on the tensor cores, kChorGemmRows rows at a time (the scratch holds one such
+bool chor_small(const qpadl_chor *h, uint32_t units) {
+    return (uint64_t)units * ((h->words + kChorGemmUnitWords - 1) / kChorGemmUnitWords) <= kChorGemmSmall;
+}
+
+// B queries on the tensor cores, kChorGemmRows rows and chor_gemm_group queries at a time (the scratch holds one such
 // block's expanded queries; the launches of a stream follow one another).
 int chor_answer_gemm(qpadl_chor *h, const uint32_t *Q, uint32_t B, uint32_t *out, cudaStream_t s) {
     const uint32_t W = h->words;
@@ -1344,14 +1349,35 @@ int chor_answer_gemm(qpadl_chor *h, const uint32_t *Q, uint32_t B, uint32_t *out
                    kChorGemmUnitRows, CU_TENSOR_MAP_SWIZZLE_64B))
         return QPADL_ECUDA;
     for (uint64_t r0 = 0; r0 < h->rows; r0 += kChorGemmRows) {
-        const uint32_t units = chor_units(std::min(h->rows - r0, kChorGemmRows));
-        QPADL_CU(launch_chor_nibbles(Q, h->qw, B, r0, units, h->qt, s));
-        if (!encode_2d(&q_map, CU_TENSOR_MAP_DATA_TYPE_UINT8, h->qt, 128ull * units, B, 128ull * units, 128,
-                       chor_gemm_n(B), CU_TENSOR_MAP_SWIZZLE_128B))
-            return QPADL_ECUDA;
-        QPADL_CU(launch_chor_gemm(db_map, q_map, r0, units, W, B, out, h->num_sms, h->d_status, s));
+        const uint32_t units = chor_units(std::min(h->rows - r0, kChorGemmRows)), group = chor_gemm_group(units);
+        const bool small = chor_small(h, units);
+        for (uint32_t g0 = 0; g0 < B; g0 += group) {
+            const uint32_t Bg = std::min(B - g0, group), rest = Bg % kChorGemmTile;
+            QPADL_CU(launch_chor_nibbles(Q + (uint64_t)g0 * h->qw, h->qw, Bg, r0, units, h->qt, s));
+            // whole tiles and the rest apart when the rest fits a narrower tile and the work is worth a launch
+            const bool apart = Bg > kChorGemmTile && rest != 0 && rest <= kChorGemmTile / 2 && !small;
+            for (uint32_t b0 = 0, Bc; b0 < Bg; b0 += Bc) {
+                Bc = apart && b0 == 0 ? Bg - rest : Bg - b0;
+                if (!encode_2d(&q_map, CU_TENSOR_MAP_DATA_TYPE_UINT8, h->qt + 32ull * units * b0, 128ull * units, Bc,
+                               128ull * units, 128, chor_gemm_n(Bc), CU_TENSOR_MAP_SWIZZLE_128B))
+                    return QPADL_ECUDA;
+                QPADL_CU(launch_chor_gemm(db_map, q_map, r0, units, W, Bc, out + (uint64_t)(g0 + b0) * W, h->num_sms,
+                                          h->d_status, s));
+            }
+        }
     }
     return QPADL_OK;
+}
+
+// How many of a batch's queries, the first ones, take the tensor cores: a threshold set by the caller decides for every
+// chunk of 256 as a whole, the library's own for all tiles and for what is left after them, unless that shares
+// their launch (1024 rows of 512 words, 129 queries: 12 us so, 19 with a scan for the last).
+uint32_t chor_tensor_queries(const qpadl_chor *h, uint32_t B) {
+    const uint32_t large = chor_min_batch(h);
+    const uint32_t chunk = chor_min_batch_set(h) ? kChorMaxBatch : kChorGemmTile;
+    if (large > chunk) return 0;
+    if (!chor_min_batch_set(h) && B > chunk && chor_small(h, chor_units(std::min(h->rows, kChorGemmRows)))) return B;
+    return B - (B % chunk < large ? B % chunk : 0);
 }
 
 }  // namespace
@@ -1367,21 +1393,13 @@ int qpadl_chor_answer_batch(qpadl_chor *h, const uint32_t *Q_dev, uint32_t B, ui
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const uint64_t W = h->words;
     QPADL_CU(cudaMemsetAsync(out_dev, 0, 4ull * W * B, s));
-    const uint32_t large = chor_min_batch(h);
-    for (uint32_t b0 = 0, Bc, left = 0; b0 < B; b0 += Bc) {
-        // a threshold set by the caller decides for a chunk of 256 as a whole (`left`: what remains of one that the
-        // tensor cores take); the library's own also for what is left of it after the first 128
-        if (left == 0 || !chor_min_batch_set(h)) {
-            Bc = std::min(B - b0, kChorMaxBatch);
-            left = Bc >= large ? Bc : 0;
-        }
-        if (left) {
-            Bc = std::min(left, kChorGemmMaxBatch);
-            left -= Bc;
-            int rc = chor_answer_gemm(h, Q_dev + (uint64_t)b0 * h->qw, Bc, out_dev + (uint64_t)b0 * W, s);
-            if (rc != QPADL_OK) return rc;
-            continue;
-        }
+    const uint32_t tensor = chor_tensor_queries(h, B);
+    if (tensor) {
+        const int rc = chor_answer_gemm(h, Q_dev, tensor, out_dev, s);
+        if (rc != QPADL_OK) return rc;
+    }
+    for (uint32_t b0 = tensor, Bc; b0 < B; b0 += Bc) {
+        Bc = std::min(B - b0, kChorMaxBatch);
         uint32_t tw = 0, rb = 0, boxw = 0, qtw = 0;
         // by batch size (measured on the 1 GiB database): the mask form up to 8 queries, the
         // predicated XOR with 4 words per thread up to 16, with 8 words per thread above
