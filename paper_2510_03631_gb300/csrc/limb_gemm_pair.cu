@@ -401,6 +401,9 @@ __global__ void __launch_bounds__(kPThreads, 1)
                 if constexpr (TMEMSUM) {
                     const float pf = static_cast<float>(epi.p), inv = 1.0f / pf;
                     const bool two = pc.c1 - pc.c0 >= 2;   // the piece used both buffers
+                    // groups of 32 columns with vectors: the others' sums are zero and stored nowhere (600 x 4000,
+                    // 130 vectors: 29 us a call, 32 over all 256 columns)
+                    const int groups = v0 + BN <= NV ? BN / 32 : static_cast<int>((NV - v0 + 31) / 32);
                     if (c + 1 < pc.c1) {
                         // replace this buffer's running sums by small representatives of their
                         // residues mod p: q = x / p rounded to an integer through the 1.5 * 2^23
@@ -409,7 +412,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
                         // wait; the next MMAs into this buffer accumulate on top.
                         constexpr float kRound = 12582912.0f;
 #pragma unroll 1
-                        for (int j0 = 0; j0 < BN / 32; j0 += 4) {
+                        for (int j0 = 0; j0 < groups; j0 += 4) {
                             uint32_t v[4][32];
 #pragma unroll
                             for (int g = 0; g < 4; ++g) tmem_ld32(acc + 32u * (j0 + g), v[g]);
@@ -441,7 +444,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
                     const uint32_t oth = tmem_base + lane_addr + (buf ^ 1u) * BN;
                     constexpr float kRound = 12582912.0f;
 #pragma unroll 1
-                    for (int j = 0; j < BN / 32; ++j) {
+                    for (int j = 0; j < groups; ++j) {
                         uint32_t v[32], w[32];
                         tmem_ld32(acc + 32u * j, v);
                         if (two) tmem_ld32(oth + 32u * j, w);
