@@ -670,11 +670,8 @@ static int resident_pairs(int num_sms) {
     return n;
 }
 
-// k-steps (64 deep) per exact chunk: 8 for digits times centred field elements, 16 for limbs or centred
-// digits times limbs.  A split launch deals chunks, so the plain store takes 16 only from 32768 columns
-// up (32768 x 32768, 192 vectors: 875 -> 816 us); with fewer its shares would be too coarse (4096 x 4096,
-// 160 vectors: 32 us with 8, 36 with 16).
-static uint32_t store_chunk_kb(uint32_t KB) { return KB >= 512 ? 16u : 8u; }
+// k-steps (64 deep) per exact chunk: 8 for digits times centred field elements, 16 for limbs times limbs; the plain
+// store's depth is store_plan's.
 template <class Epi>
 constexpr uint32_t pair_chunk_kb() {
     return std::is_same<Epi, ModPEpi>::value ? 8u : 16u;
@@ -709,6 +706,52 @@ static bool pair_split_schedule(uint64_t tiles, uint64_t n_tiles, uint32_t nchun
     *dp_tiles = static_cast<uint32_t>(dp);
     *tail_parts = static_cast<uint32_t>(P);
     return true;
+}
+
+// How a plain-store launch runs: k-steps per exact chunk, clusters, split (dp whole tiles, tail_parts; 0 parts: none)
+// and the modelled time in us of the call.
+struct StorePlan {
+    uint32_t ckb, dp, tail_parts;
+    uint64_t clusters;
+    double us;
+};
+
+// Chunks of 16 k-steps have half the drains of 8 (8192 x 8192, 192 vectors: 65 -> 61 us; 20000 x 20000, 150: 317 -> 304),
+// but a split deals whole chunks, and coarser ones can leave a cluster a longer share (2304 x 12000, 150 vectors: 31 us
+// with 8, 33 with 16).  So 16 from 8192 columns on, where the longest share does not grow by more than 5%.
+// The time is modelled as limb_gemm_tri.cu's is, fitted to 520 calls (rms 6%), then raised by 6%: where the two are
+// close, three limbs lose less when the model is wrong.
+static StorePlan store_plan(uint32_t M, uint32_t NV, uint32_t KB, int num_sms) {
+    const uint64_t n_tiles = ((uint64_t)NV + 63) / 64, tiles = ((uint64_t)M + 2 * kPM - 1) / (2 * kPM) * n_tiles;
+    const int n = resident_pairs<256, StoreEpi, false>(num_sms);
+    const uint64_t pairs = n > 0 ? n : 1;
+    StorePlan best{};
+    double best_steps = 0.0;
+    for (uint32_t ckb = 8; ckb <= (KB >= 128 ? 16u : 8u); ckb += 8) {
+        const uint32_t nchunks = (KB + ckb - 1) / ckb;
+        StorePlan p{ckb, 0xffffffffu, 0, tiles < pairs ? tiles : pairs, 0.0};
+        double waves = static_cast<double>((tiles + pairs - 1) / pairs), steps = waves * KB;   // k-steps of the busiest cluster
+        if (pair_split_schedule(tiles, n_tiles, nchunks, pairs, &p.clusters, &p.dp, &p.tail_parts)) {
+            const uint64_t units = (tiles - p.dp) / n_tiles * nchunks;
+            waves = static_cast<double>(p.dp) / pairs + static_cast<double>(tiles - p.dp) / (p.tail_parts * n_tiles);
+            steps = static_cast<double>((p.dp + pairs - 1) / pairs * KB + (units + p.tail_parts - 1) / p.tail_parts * ckb);
+        }
+        p.us = 1.06 * (5.75 + 1.55e-6 * NV * KB * kPK + (ckb == 8 ? 0.289 : 0.279) * steps + 2.77 * std::ceil(waves) +
+                       (p.tail_parts ? 0.18 + 0.079e-6 * M * NV * p.tail_parts : 0.0));
+        if (ckb == 8 || 0.95 * steps <= best_steps) {
+            best = p;
+            best_steps = steps;
+        }
+    }
+    return best;
+}
+
+bool limb_gemm_pair_splits(uint32_t M, uint32_t NV, uint64_t K, int num_sms) {
+    return store_plan(M, NV, static_cast<uint32_t>((K + kPK - 1) / kPK), num_sms).tail_parts != 0;
+}
+
+double limb_gemm_pair_us(uint32_t M, uint32_t NV, uint64_t K, int num_sms) {
+    return store_plan(M, NV, static_cast<uint32_t>((K + kPK - 1) / kPK), num_sms).us;
 }
 
 // Chunk ranges per tile of a Z_p launch, from its time in us: whole waves of ranges on `pairs` clusters, each
@@ -749,8 +792,13 @@ static cudaError_t launch_pair_t(const CUtensorMap &a_map, const PairBMaps &bm, 
     uint64_t clusters = tiles < pairs ? tiles : pairs;
     uint32_t dp = 0xffffffffu, tail_parts = 0;
     uint32_t ksplit = 1;
-    if constexpr (std::is_same<Epi, StoreEpi>::value)   // split tiles add into the output, which is zero then
-        pair_split_schedule(tiles, n_tiles, (KB + ckb - 1) / ckb, pairs, &clusters, &dp, &tail_parts);
+    if constexpr (std::is_same<Epi, StoreEpi>::value) {   // split tiles add into the output, which is zero then
+        const StorePlan plan = store_plan(M, NV, KB, num_sms);
+        ckb = plan.ckb;
+        clusters = plan.clusters;
+        dp = plan.dp;
+        tail_parts = plan.tail_parts;
+    }
     if constexpr (std::is_same<Epi, ModPEpi>::value) {
         if (epi.ld_m == 1 && epi.ld_b == M) ksplit = field_ksplit(tiles, n_tiles, (KB + ckb - 1) / ckb, pairs, (uint64_t)M * NV);
         if (ksplit > 1) {
@@ -786,8 +834,7 @@ static cudaError_t launch_pair_epi(int bn, const CUtensorMap &a_map, const PairB
     } else {
         if constexpr (std::is_same<Epi, StoreEpi>::value) {   // 256-wide plain tiles only
             if (bn != 256 || plane_chunks != 0) return cudaErrorInvalidValue;
-            return launch_pair_t<256, Epi, false>(a_map, bm, epi, M, NV, KB, store_chunk_kb(KB), 0, num_sms, status,
-                                                 stream);
+            return launch_pair_t<256, Epi, false>(a_map, bm, epi, M, NV, KB, 0, 0, num_sms, status, stream);
         } else if (plane_chunks == 0) {
             constexpr uint32_t ckb = pair_chunk_kb<Epi>();
             switch (bn) {
@@ -823,34 +870,6 @@ cudaError_t launch_limb_gemm_pair(const CUtensorMap &a_map, const PairBMaps &bm,
                                   uint32_t M, uint32_t NV, uint64_t K, int num_sms, int *status,
                                   cudaStream_t stream) {
     return launch_pair_epi(256, a_map, bm, StoreEpi{out, 1, M, sums}, M, NV, K, 0, num_sms, status, stream);
-}
-
-// Whether that launch splits tiles, and the time in us of a call, modelled as limb_gemm_tri.cu's is and fitted to the
-// same shapes, then raised by 5%: where the two are close, three limbs lose less when the model is wrong.
-static bool store_schedule(uint32_t M, uint32_t NV, uint64_t K, int num_sms, double *us) {
-    const uint64_t n_tiles = ((uint64_t)NV + 63) / 64, tiles = ((uint64_t)M + 2 * kPM - 1) / (2 * kPM) * n_tiles;
-    const uint32_t KB = static_cast<uint32_t>((K + kPK - 1) / kPK), ckb = store_chunk_kb(KB);
-    const int n = resident_pairs<256, StoreEpi, false>(num_sms);
-    const uint64_t pairs = n > 0 ? n : 1;
-    uint64_t clusters = 0;
-    uint32_t dp = 0, tail = 0;
-    const bool split = pair_split_schedule(tiles, n_tiles, (KB + ckb - 1) / ckb, pairs, &clusters, &dp, &tail);
-    const double waves = split ? static_cast<double>(dp) / pairs + static_cast<double>(tiles - dp) / (tail * n_tiles)
-                               : static_cast<double>((tiles + pairs - 1) / pairs);
-    *us = 6.2 + 1.86e-6 * K * NV + 0.298 * KB * waves + 2.94 * std::ceil(waves) +
-          (split ? 0.58 + 0.131e-6 * M * NV * tail : 0.0);
-    return split;
-}
-
-bool limb_gemm_pair_splits(uint32_t M, uint32_t NV, uint64_t K, int num_sms) {
-    double us;
-    return store_schedule(M, NV, K, num_sms, &us);
-}
-
-double limb_gemm_pair_us(uint32_t M, uint32_t NV, uint64_t K, int num_sms) {
-    double us;
-    store_schedule(M, NV, K, num_sms, &us);
-    return us;
 }
 
 cudaError_t launch_limb_gemm_pair_query(int bn, const CUtensorMap &a_map, const PairBMaps &bm,
