@@ -490,7 +490,7 @@ typedef struct qpadl_chor qpadl_chor;
 
 /* Binds a resident database (db_dev: rows x bits/32 uint32 words, caller-
  * owned, 16-byte aligned, kept until destroy) on the current device and
- * allocates the handle's scratch (32 bytes per row; for up to 2^18 rows at least 512, at most 16 MiB).
+ * allocates the handle's scratch (32 bytes per row; up to 2^18 rows 64 to 512, at most 16 MiB).
  * QPADL_EINVAL if rows
  * is 0 or >= 2^31, bits is not a positive multiple of 128, or db_dev is
  * NULL or misaligned. */
@@ -498,7 +498,7 @@ int qpadl_chor_setup(uint64_t rows, uint64_t bits, const uint32_t *db_dev, qpadl
                      qpadl_chor **out);
 
 /* Answers B queries (Q_dev: B x ceil(rows/32) words, query b in row b) in
- * one pass over the database per 128 to 1024 (tensor cores, as the scratch allows) or 256 (scan)
+ * one pass over the database per 128 to 1024 (tensor cores; fewer for more rows) or 256 (scan)
  * queries; out_dev: B x bits/32 words
  * (answer b in row b), overwritten.  Calls on one handle share its scratch:
  * issue them on one stream (or order them). */

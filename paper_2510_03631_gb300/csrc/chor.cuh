@@ -31,10 +31,12 @@ constexpr uint32_t kChorGemmUnitWords = 16;
 constexpr uint32_t kChorGemmTile = 128;
 // Rows per launch: bounds the expanded queries and, far below 2^22, the counts.
 constexpr uint64_t kChorGemmRows = 1ull << 18;
-// Queries per launch over `units` units: tiles whose expanded bits (128 bytes per query and unit) stay within
-// 16 MiB, one at 2^18 rows, at most 1024 queries.
+// Queries per launch over `units` units (128 bytes of expanded bits per query and unit): up to eight tiles in 1 MiB, which
+// cudaMalloc gives out of memory it holds (a larger piece takes a setup 100 us instead of 20), but at least two, or one
+// where two are more than 16 MiB.
 constexpr uint32_t chor_gemm_group(uint32_t units) {
-    return units <= 128 ? 1024u : (16u << 20) / (128u * kChorGemmTile * units) * kChorGemmTile;
+    const uint32_t tiles = (1u << 20) / (128u * kChorGemmTile * units);
+    return kChorGemmTile * (tiles > 8 ? 8 : (tiles >= 2 ? tiles : (units <= 512 ? 2 : 1)));
 }
 constexpr uint64_t chor_gemm_scratch(uint32_t units) { return 128ull * chor_gemm_group(units) * units; }
 // Up to this many units x column tiles, what a batch leaves for its last tile shares the launch of the others even when
