@@ -559,8 +559,12 @@ __global__ void __launch_bounds__(kSumCols / 8) vec_limbs_sums_kernel(const uint
 template <int LIMBS>
 __global__ void __launch_bounds__(256) mat_col_limbs_sums_kernel(const uint32_t *__restrict__ A, uint64_t C, uint32_t n,
                                                                  __half *__restrict__ L, uint64_t pitch,
-                                                                 uint32_t *__restrict__ sums) {
+                                                                 uint32_t *__restrict__ sums, uint32_t *__restrict__ Z,
+                                                                 uint64_t z_words) {
     griddep_launch_dependents();   // as in vec_limbs_sums_kernel
+    for (uint64_t i = ((uint64_t)blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x; i < z_words;
+         i += (uint64_t)gridDim.x * gridDim.y * blockDim.x)
+        Z[i] = 0u;
     __shared__ uint32_t tile[128][33];
     const uint64_t j0 = (uint64_t)blockIdx.x * 128;
     const uint32_t k0 = blockIdx.y * 32;
@@ -633,24 +637,25 @@ cudaError_t launch_vec_limbs_four(const uint32_t *X, uint64_t x_ld, uint32_t NV,
 
 template <int LIMBS>
 static cudaError_t launch_mat_col_limbs_sums(const uint32_t *A, uint64_t C, uint32_t n, __half *L, uint64_t pitch,
-                                             const VecSums &vs, cudaStream_t stream) {
+                                             const VecSums &vs, uint32_t *zero, uint64_t zero_words,
+                                             cudaStream_t stream) {
     if (n == 0 || C == 0 || pitch % 8 != 0) return cudaErrorInvalidValue;
     uint32_t *sums = const_cast<uint32_t *>(vs.words);
     const cudaError_t e = cudaMemsetAsync(sums, 0, 4ull * n, stream);
     if (e != cudaSuccess) return e;
     const dim3 grid(static_cast<unsigned>((C + 127) / 128), (n + 31) / 32);
-    mat_col_limbs_sums_kernel<LIMBS><<<grid, 256, 0, stream>>>(A, C, n, L, pitch, sums);
+    mat_col_limbs_sums_kernel<LIMBS><<<grid, 256, 0, stream>>>(A, C, n, L, pitch, sums, zero, zero ? zero_words : 0);
     return cudaGetLastError();
 }
 
 cudaError_t launch_mat_col_limbs_tri(const uint32_t *A, uint64_t C, uint32_t n, __half *L, uint64_t pitch,
-                                     cudaStream_t stream) {
-    return launch_mat_col_limbs_sums<3>(A, C, n, L, pitch, tri_sums(L, n, pitch, 1), stream);
+                                     uint32_t *zero, uint64_t zero_words, cudaStream_t stream) {
+    return launch_mat_col_limbs_sums<3>(A, C, n, L, pitch, tri_sums(L, n, pitch, 1), zero, zero_words, stream);
 }
 
 cudaError_t launch_mat_col_limbs_four(const uint32_t *A, uint64_t C, uint32_t n, __half *L, uint64_t pitch,
                                       cudaStream_t stream) {
-    return launch_mat_col_limbs_sums<4>(A, C, n, L, pitch, four_sums(L, n, pitch, 1), stream);
+    return launch_mat_col_limbs_sums<4>(A, C, n, L, pitch, four_sums(L, n, pitch, 1), nullptr, 0, stream);
 }
 
 template <int H>

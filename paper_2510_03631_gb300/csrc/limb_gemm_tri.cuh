@@ -32,7 +32,7 @@ cudaError_t launch_vec_limbs_four(const uint32_t *X, uint64_t x_ld, uint32_t NV,
                                   uint32_t *zero, uint64_t zero_words, cudaStream_t stream);
 // The three limbs, or four, of the columns of A (C x n row-major), and one sum each: vector k is column k.
 cudaError_t launch_mat_col_limbs_tri(const uint32_t *A, uint64_t C, uint32_t n, __half *L, uint64_t pitch,
-                                     cudaStream_t stream);
+                                     uint32_t *zero, uint64_t zero_words, cudaStream_t stream);
 cudaError_t launch_mat_col_limbs_four(const uint32_t *A, uint64_t C, uint32_t n, __half *L, uint64_t pitch,
                                       cudaStream_t stream);
 

@@ -792,8 +792,9 @@ int qpadl_pir_hint(qpadl_db *db, const uint32_t *A_dev, uint32_t *H_dev, qpadl_s
     if (!u8 && use_tri(db)) {
         const uint64_t R = db->prm.rows;
         const TriPlan plan = limb_gemm_tri_plan(static_cast<uint32_t>(R), n, db->prm.cols, db->num_sms);
-        if (plan.ranges > 1) QPADL_CU(cudaMemsetAsync(H_dev, 0, 4ull * n * R, s));
-        QPADL_CU(launch_mat_col_limbs_tri(A_dev, db->prm.cols, n, db->limbs, db->pitch, s));
+        // one launch makes the limbs and zeroes the hint that ranges add to, as in answer_f16
+        QPADL_CU(launch_mat_col_limbs_tri(A_dev, db->prm.cols, n, db->limbs, db->pitch, plan.ranges > 1 ? H_dev : nullptr,
+                                          (uint64_t)n * R, s));
         return run_tri_gemm(db, db->limbs, n, 1, H_dev, n, 1, plan, s);
     }
     if (!u8) {

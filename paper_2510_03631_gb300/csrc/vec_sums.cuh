@@ -22,7 +22,7 @@ struct VecSums {
     // programmatic dependent overlaps.
     __device__ __forceinline__ uint32_t centred(uint32_t v) const {
         uint32_t s = 0;
-#pragma unroll 4
+#pragma unroll 8
         for (uint32_t x = 0; x < parts; ++x) s += __ldcg(words + (uint64_t)x * nv + v);
         return kCentre * s;
     }
