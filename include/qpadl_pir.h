@@ -490,7 +490,7 @@ typedef struct qpadl_chor qpadl_chor;
 
 /* Binds a resident database (db_dev: rows x bits/32 uint32 words, caller-
  * owned, 16-byte aligned, kept until destroy) on the current device and
- * allocates the handle's scratch (32 bytes per row; up to 2^18 rows 64 to 512, at most 16 MiB).
+ * allocates the handle's scratch (32 bytes per row; up to 2^18 rows 64 or 128, and 256 KiB for few rows).
  * QPADL_EINVAL if rows
  * is 0 or >= 2^31, bits is not a positive multiple of 128, or db_dev is
  * NULL or misaligned. */

@@ -31,11 +31,11 @@ constexpr uint32_t kChorGemmUnitWords = 16;
 constexpr uint32_t kChorGemmTile = 128;
 // Rows per launch: bounds the expanded queries and, far below 2^22, the counts.
 constexpr uint64_t kChorGemmRows = 1ull << 18;
-// Queries per launch over `units` units (128 bytes of expanded bits per query and unit): up to eight tiles in 1 MiB, which
-// cudaMalloc gives out of memory it holds (a larger piece takes a setup 100 us instead of 20), but at least two, or one
+// Queries per launch over `units` units (128 bytes of expanded bits per query and unit): up to eight tiles in 256 KiB, which
+// cudaMalloc mostly gives out of memory it holds (else a setup takes 100 us instead of 20), but at least two, or one
 // where two are more than 16 MiB.
 constexpr uint32_t chor_gemm_group(uint32_t units) {
-    const uint32_t tiles = (1u << 20) / (128u * kChorGemmTile * units);
+    const uint32_t tiles = (256u << 10) / (128u * kChorGemmTile * units);
     return kChorGemmTile * (tiles > 8 ? 8 : (tiles >= 2 ? tiles : (units <= 512 ? 2 : 1)));
 }
 constexpr uint64_t chor_gemm_scratch(uint32_t units) { return 128ull * chor_gemm_group(units) * units; }

@@ -74,7 +74,7 @@ def test_option_reads_as_the_threshold_in_force():
 
 
 # several tiles of 128 queries in one launch, the last one whole, wide or narrow; more tiles than the scratch holds
-# (eight up to 2048 rows, two from 5500 and one from 2^17 on); a narrow rest in a launch of its own (more than 4096 units x column tiles)
+# (eight up to 512 rows, two from 1400 and one from 2^17 on); a narrow rest in a launch of its own (more than 4096 units x column tiles)
 @pytest.mark.parametrize("rows,bits,B", [(1, 128, 257), (300, 640, 129), (300, 640, 192), (300, 4096, 300), (2805, 1152, 190),
                                          (700, 1280, 726), (257, 512, 1025), (33000, 128, 300), (5000, 256, 700), (20000, 40960, 130), (1024, 16384, 129),
                                          ((1 << 18) + 700, 128, 140)])
