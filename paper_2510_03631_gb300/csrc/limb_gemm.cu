@@ -81,15 +81,6 @@ struct GemmCfg {
     static constexpr int kQPT = BN / 4;   // vectors per tile
 };
 
-__device__ __forceinline__ bool drain_wait_g(uint64_t *bar, uint32_t parity) {
-    if (mbar_test(bar, parity)) return true;
-    const uint64_t t0 = global_ns();
-    while (!mbar_test(bar, parity)) {
-        if (global_ns() - t0 > QPADL_WAIT_NS) return false;
-    }
-    return true;
-}
-
 // Work schedule of one CTA.  Tiles [0, dp_tiles) are whole-tile work dealt
 // round-robin (tile b, b + G, ...: neighbouring CTAs share the rows of D).
 // The remaining tiles are split stream-K style: their chunks (tile-major)
@@ -219,7 +210,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             }
             const uint32_t inflight = it < (uint32_t)kGemmStages ? it : (uint32_t)kGemmStages;
             for (uint32_t j = it - inflight; j < it; ++j)
-                if (!drain_wait_g(&full[j % kGemmStages], (j / kGemmStages) & 1u)) failed = true;
+                if (!mbar_drain(&full[j % kGemmStages], (j / kGemmStages) & 1u)) failed = true;
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer: the whole warp walks the loop (warp-uniform descriptors),
@@ -284,7 +275,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         if (issued) {
             if (elect_one()) umma_commit(mma_done);
             __syncwarp();
-            if (!drain_wait_g(mma_done, 0)) failed = true;
+            if (!mbar_drain(mma_done, 0)) failed = true;
         }
     } else {
         // ---------------- epilogue (warps 2..5; TMEM lane quarter = warp % 4)

@@ -90,15 +90,6 @@ struct PairCfg {
     static_assert(kStages >= 4, "pipeline depth");
 };
 
-__device__ __forceinline__ bool drain_wait_p(uint64_t *bar, uint32_t parity) {
-    if (mbar_test(bar, parity)) return true;
-    const uint64_t t0 = global_ns();
-    while (!mbar_test(bar, parity)) {
-        if (global_ns() - t0 > QPADL_WAIT_NS) return false;
-    }
-    return true;
-}
-
 // One piece of a cluster's work: chunks [c0, c1) of pair tile t.  Tiles below dp_tiles are dealt
 // whole, round-robin (tile c, c + nclusters, ...), so the clusters on the n_tiles tiles of one row
 // tile run together and share its rows through L2.  The remaining tiles (whole row tiles) are
@@ -289,7 +280,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
                 // the stages still owed bytes (both producers' and the peer's copies) must land before exit
                 const uint32_t inflight = it < (uint32_t)ST ? it : (uint32_t)ST;
                 for (uint32_t j = it - inflight; j < it; ++j)
-                    if (!drain_wait_p(&full[j % ST], (j / ST) & 1u)) failed = true;
+                    if (!mbar_drain(&full[j % ST], (j / ST) & 1u)) failed = true;
             }
         }
     } else if (warp == 1) {
@@ -352,7 +343,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
             if (issued) {
                 if (elect_one()) umma_commit_pair(mma_done, 1);
                 __syncwarp();
-                if (!drain_wait_p(mma_done, 0)) failed = true;
+                if (!mbar_drain(mma_done, 0)) failed = true;
             }
         }
     } else {

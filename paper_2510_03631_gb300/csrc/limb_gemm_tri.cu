@@ -73,15 +73,6 @@ struct TriCfg {
     static_assert(kStages >= 4, "a chunk's two stages and two in flight");
 };
 
-__device__ __forceinline__ bool drain_wait_t(uint64_t *bar, uint32_t parity) {
-    if (mbar_test(bar, parity)) return true;
-    const uint64_t t0 = global_ns();
-    while (!mbar_test(bar, parity)) {
-        if (global_ns() - t0 > QPADL_WAIT_NS) return false;
-    }
-    return true;
-}
-
 // A cluster's pieces: unit i is column range i / tiles of tile i % tiles, chunks [c0, c1).  The vector
 // tiles of a row tile are neighbours; which of them comes first turns from wave to wave, so a narrower
 // last one (fewer halves) does not always fall to the same clusters.
@@ -284,7 +275,7 @@ __global__ void __launch_bounds__(kTThreads, 1)
                     // the stages still owed bytes (both producers' and the peer's copies) must land before exit
                     const uint32_t inflight = it < (uint32_t)ST ? it : (uint32_t)ST;
                     for (uint32_t j = it - inflight; j < it; ++j)
-                        if (!drain_wait_t(&full[j % ST], (j / ST) & 1u)) failed = true;
+                        if (!mbar_drain(&full[j % ST], (j / ST) & 1u)) failed = true;
                 }
             }
         } else if (warp == 1) {
@@ -353,7 +344,7 @@ __global__ void __launch_bounds__(kTThreads, 1)
                 if (issued) {
                     if (elect_one()) umma_commit_pair(mma_done, 1);
                     __syncwarp();
-                    if (!drain_wait_t(mma_done, 0)) failed = true;
+                    if (!mbar_drain(mma_done, 0)) failed = true;
                 }
             }
         }

@@ -154,7 +154,7 @@ def main():
     ap.add_argument("--rows", type=int, default=8192)
     ap.add_argument("--cols", type=int, default=32768)
     ap.add_argument("--bits", type=int, default=262144, help="chor: bits per record")
-    ap.add_argument("--m4rm", type=int, default=-1, help="chor: smallest batch on the four-Russians kernel")
+    ap.add_argument("--m4rm", type=int, default=-1, help="chor: smallest batch on the tensor cores")
     ap.add_argument("--form", type=int, default=-1, help="chor: inner-loop form of the masked-XOR scan (0..3)")
     ap.add_argument("--batch", type=int, default=256)
     ap.add_argument("--n", type=int, default=1024)
