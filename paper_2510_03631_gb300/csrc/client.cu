@@ -14,7 +14,7 @@
 // before it (programmatic dependent launch); other n use one warp per row
 // and a shared-memory copy of the secret.
 // Batches are u32 GEMMs (Y = X * W^T over Z_{2^32}) on the CUDA cores in
-// panels of 32 rows whose warps split K.
+// panels of 32 rows whose warps split K, or in 128 x 128 tiles.
 #include <cstdint>
 #include <mutex>
 
@@ -407,6 +407,70 @@ __global__ void __launch_bounds__(kPanelThreads, 2)
     }
 }
 
+// The same product in 128 x 128 tiles, 8 x 8 outputs per thread, for many vectors whose rows allow copies of one or two
+// words only: a panel then spends its time on copy instructions, 32 words of each operand for 32 x 32 products, where
+// a tile of this size loads a quarter of them (32768 x 1023 by 1024 vectors: 2.95 ms, 5.33 in panels; rows of 630
+// words 1.99 and 2.47; rows of whole 16 bytes keep the panels, 2.85 for 1024 words).
+constexpr int kGT = 128, kGK = 8;
+template <class Epi>
+__global__ void __launch_bounds__(256) u32_gemm_nt_kernel(const uint32_t *__restrict__ X, uint64_t M,
+                                                          const uint32_t *__restrict__ W, uint32_t N, uint32_t K,
+                                                          Epi epi) {
+    __shared__ uint32_t xs[kGK][kGT];
+    __shared__ uint32_t ws[kGK][kGT];
+    const uint64_t i0 = (uint64_t)blockIdx.x * kGT;
+    const uint32_t b0 = blockIdx.y * kGT;
+    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+    uint32_t acc[8][8];
+#pragma unroll
+    for (int a = 0; a < 8; ++a)
+#pragma unroll
+        for (int c = 0; c < 8; ++c) acc[a][c] = 0u;
+    // loader mapping: 256 threads x 4 elements = one 128 x 8 tile
+    const int lr = threadIdx.x / 2;            // tile row 0..127
+    const int lk = (threadIdx.x % 2) * 4;      // k offset 0 or 4
+    for (uint32_t k0 = 0; k0 < K; k0 += kGK) {
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const uint32_t k = k0 + lk + t;
+            const uint64_t i = i0 + lr;
+            const uint32_t b = b0 + lr;
+            xs[lk + t][lr] = (i < M && k < K) ? X[i * K + k] : 0u;
+            ws[lk + t][lr] = (b < N && k < K) ? W[(uint64_t)b * K + k] : 0u;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int kk = 0; kk < kGK; ++kk) {
+            uint32_t xa[8], wb[8];
+#pragma unroll
+            for (int a = 0; a < 8; ++a) xa[a] = xs[kk][ty + 16 * a];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) wb[c] = ws[kk][tx + 16 * c];
+#pragma unroll
+            for (int a = 0; a < 8; ++a)
+#pragma unroll
+                for (int c = 0; c < 8; ++c) acc[a][c] += xa[a] * wb[c];
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+        const uint64_t i = i0 + ty + 16 * a;
+        if (i >= M) continue;
+        uint32_t pre_v[8];   // all loads of the row's outputs before any of its stores
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const uint32_t b = b0 + tx + 16 * c;
+            pre_v[c] = b < N ? epi.pre(i, b) : 0u;
+        }
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const uint32_t b = b0 + tx + 16 * c;
+            if (b < N) epi.put(i, b, acc[a][c], pre_v[c]);
+        }
+    }
+}
+
 // ------------------------------------------------------------------ host side
 template <int TC, class Epi>
 static cudaError_t launch_panel_t(const uint32_t *X, uint64_t M, const uint32_t *W, uint32_t N, uint32_t K, int vec,
@@ -419,13 +483,35 @@ static cudaError_t launch_panel_t(const uint32_t *X, uint64_t M, const uint32_t 
     return cudaGetLastError();
 }
 
-// The fewest panels of at most 32 vectors, each as narrow as covers the batch.
 template <class Epi>
-static cudaError_t launch_panel(const uint32_t *X, uint64_t M, const uint32_t *W, uint32_t N, uint32_t K,
+static cudaError_t launch_tiles(const uint32_t *X, uint64_t M, const uint32_t *W, uint32_t N, uint32_t K,
+                                const Epi &epi, cudaStream_t stream) {
+    const uint64_t rows = (M + kGT - 1) / kGT, cols = ((uint64_t)N + kGT - 1) / kGT;
+    if (rows >= (1ull << 31) || cols > 65535) return cudaErrorInvalidValue;
+    const dim3 grid(static_cast<unsigned>(rows), static_cast<unsigned>(cols));
+    u32_gemm_nt_kernel<Epi><<<grid, 256, 0, stream>>>(X, M, W, N, K, epi);
+    return cudaGetLastError();
+}
+
+// Whether 128 x 128 tiles are the faster form, from measured rates (us): a column of K costs 0.28 and 1.27e-3 per tile
+// in tiles, and one multiply-add per output at 6.4 (one-word copies) or 8.6 (two-word) million a us in panels; tiles
+// when they save 5%.  Measured, tiles against panels: 60000 rows of 999 words, 100 vectors 1067 / 1247; 8000 of 1023,
+// 512 vectors 669 / 714, 256 panels faster; 32768 of 630, 256 vectors panels faster, 512 1120 / 1243.
+static bool tiles_faster(uint64_t M, uint32_t N, uint32_t K, int vec) {
+    if (vec == 4) return false;
+    const double tiles = static_cast<double>((M + kGT - 1) / kGT) * static_cast<double>((N + kGT - 1) / kGT);
+    const double panels_us = static_cast<double>(M) * ((N + 31) / 32 * 32) * K / (vec == 2 ? 8.6e6 : 6.4e6);
+    return K * (0.28 + 1.27e-3 * tiles) < 0.95 * panels_us;
+}
+
+// Tiles, or the fewest panels of at most 32 vectors, each as narrow as covers the batch.
+template <class Epi>
+static cudaError_t launch_product(const uint32_t *X, uint64_t M, const uint32_t *W, uint32_t N, uint32_t K,
                                 const Epi &epi, cudaStream_t stream) {
     if (!client_status_word()) return cudaErrorUnknown;   // this device's kernel attributes
     const uintptr_t at = reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(W);
     const int vec = (K % 4 == 0 && at % 16 == 0) ? 4 : ((K % 2 == 0 && at % 8 == 0) ? 2 : 1);
+    if (tiles_faster(M, N, K, vec)) return launch_tiles(X, M, W, N, K, epi, stream);
     const uint32_t tiles = (N - 1) / 32 + 1, per = (N - 1) / tiles + 1;
     if (per <= 4) return launch_panel_t<1>(X, M, W, N, K, vec, epi, stream);
     if (per <= 8) return launch_panel_t<2>(X, M, W, N, K, vec, epi, stream);
@@ -448,7 +534,7 @@ cudaError_t launch_query(const uint32_t *A, uint64_t C, uint32_t n, const uint32
 cudaError_t launch_query_batch(const uint32_t *A, uint64_t C, uint32_t n, const uint32_t *S, const int32_t *E,
                                const uint32_t *cols, uint32_t B, uint32_t delta, uint32_t *Q, cudaStream_t stream) {
     QueryEpi epi{E, C, cols, 0, delta, Q, C};
-    return launch_panel(A, C, S, B, n, epi, stream);
+    return launch_product(A, C, S, B, n, epi, stream);
 }
 
 cudaError_t launch_recover(const uint32_t *ans, const uint32_t *H, uint64_t R, uint32_t n, const uint32_t *s,
@@ -460,7 +546,7 @@ cudaError_t launch_recover(const uint32_t *ans, const uint32_t *H, uint64_t R, u
 cudaError_t launch_recover_batch(const uint32_t *ans, const uint32_t *H, uint64_t R, uint32_t n, const uint32_t *S,
                                  uint32_t B, uint32_t shift, uint8_t *out, cudaStream_t stream) {
     RecoverEpi epi{ans, R, shift, out, R};
-    return launch_panel(H, R, S, B, n, epi, stream);
+    return launch_product(H, R, S, B, n, epi, stream);
 }
 
 cudaError_t prepare_client_kernels() { return client_status_word() ? cudaSuccess : cudaErrorUnknown; }
