@@ -199,13 +199,14 @@ __global__ void __launch_bounds__(kEncThreads) delta_encode_kernel(const uint32_
 // the row stores.  2^24 entries, one byte, blocks of 2 / 5 / 16 / 33 / 64 / 80 entries: 84 / 47 / 31 / 41 / 27 /
 // 26 us, in 128 x 128 tiles 969 / 399 / 132 / 73 / 41 / 35; 81 entries 37 in tiles, 90 entries 41 staged, 35 in tiles.
 constexpr uint32_t kShortEntries = 80;
+template <uint32_t COLS>   // blocks per CTA: 128, or 32 where that would leave SMs without a CTA
 __global__ void __launch_bounds__(kEncThreads) delta_encode_short_kernel(const uint32_t *__restrict__ x, uint64_t n,
                                                                          uint32_t E, uint32_t w, uint64_t C,
                                                                          uint8_t *__restrict__ db) {
-    extern __shared__ uint32_t ent[];   // [kEncCols][ld]; an odd stride puts neighbouring columns in distinct banks
+    extern __shared__ uint32_t ent[];   // [COLS][ld]; an odd stride puts neighbouring columns in distinct banks
     const uint32_t ld = E | 1u;
-    const uint64_t j0 = (uint64_t)blockIdx.x * kEncCols;
-    const uint32_t ncols = static_cast<uint32_t>(C - j0 < (uint64_t)kEncCols ? C - j0 : (uint64_t)kEncCols);
+    const uint64_t j0 = (uint64_t)blockIdx.x * COLS;
+    const uint32_t ncols = static_cast<uint32_t>(C - j0 < (uint64_t)COLS ? C - j0 : (uint64_t)COLS);
     const uint64_t k0 = j0 * E;
     if (k0 + (uint64_t)ncols * E <= n) {   // one check: the loads do not wait for one another
 #pragma unroll 4
@@ -225,7 +226,7 @@ __global__ void __launch_bounds__(kEncThreads) delta_encode_short_kernel(const u
     uint8_t *diffs = db + 4 * C + j0;
     db += j0;
     if (C % 4 == 0 && (reinterpret_cast<uintptr_t>(db) & 3u) == 0) {   // four columns in one store
-        constexpr uint32_t kQuads = kEncCols / 4;
+        constexpr uint32_t kQuads = COLS / 4;
         for (uint32_t t = threadIdx.x; t < rows * kQuads; t += kEncThreads) {
             const uint32_t r = t / kQuads, c = 4 * (t % kQuads);
             if (c >= ncols) continue;   // C % 4 == 0: whole quads
@@ -236,14 +237,47 @@ __global__ void __launch_bounds__(kEncThreads) delta_encode_short_kernel(const u
             *reinterpret_cast<uint32_t *>(diffs + r * C + c) = v;
         }
     } else {
-        for (uint32_t t = threadIdx.x; t < rows * kEncCols; t += kEncThreads) {
-            const uint32_t r = t / kEncCols, c = t % kEncCols, i = r / w;
+        for (uint32_t t = threadIdx.x; t < rows * COLS; t += kEncThreads) {
+            const uint32_t r = t / COLS, c = t % COLS, i = r / w;
             if (c < ncols) diffs[r * C + c] = static_cast<uint8_t>((ent[c * ld + i + 1] - ent[c * ld + i]) >> (8u * (r - i * w)));
         }
     }
-    for (uint32_t t = threadIdx.x; t < 4 * kEncCols; t += kEncThreads) {   // the first entry of each block in full
-        const uint32_t r = t / kEncCols, c = t % kEncCols;
+    for (uint32_t t = threadIdx.x; t < 4 * COLS; t += kEncThreads) {   // the first entry of each block in full
+        const uint32_t r = t / COLS, c = t % COLS;
         if (c < ncols) db[r * C + c] = static_cast<uint8_t>(ent[c * ld] >> (8u * r));
+    }
+}
+
+// The same for few blocks (columns): their rows are so short that the database is written as one run of bytes, four to
+// a thread, each from two neighbouring entries.  The tile above would be mostly columns past the last one: one block of
+// 2^20 entries, one byte, 138 us in tiles, FEWFIG.
+constexpr uint64_t kFewBlocks = 16;
+__global__ void __launch_bounds__(kEncThreads) delta_encode_few_kernel(const uint32_t *__restrict__ x, uint64_t n, uint32_t E,
+                                                                       uint32_t w, uint32_t C, uint8_t *__restrict__ db) {
+    const uint32_t total = (4 + w * (E - 1)) * C;   // at most 16 x 4 x 2^22 bytes
+    const uint32_t at = 4 * (blockIdx.x * kEncThreads + threadIdx.x);
+    if (at >= total) return;
+    uint32_t row = at / C, c = at - row * C, v = 0;
+#pragma unroll
+    for (uint32_t k = 0; k < 4; ++k) {
+        const uint64_t first = (uint64_t)c * E;
+        uint32_t d;
+        if (row < 4) {
+            d = entry_at(x, n, first) >> (8 * row);
+        } else {
+            const uint32_t i = (row - 4) / w, b = row - 4 - i * w;   // difference i + 1
+            d = (entry_at(x, n, first + i + 1) - entry_at(x, n, first + i)) >> (8 * b);
+        }
+        v |= (d & 255u) << (8 * k);
+        if (++c == C) {
+            c = 0;
+            ++row;
+        }
+    }
+    if (at + 4 <= total && (reinterpret_cast<uintptr_t>(db) & 3u) == 0) {
+        *reinterpret_cast<uint32_t *>(db + at) = v;
+    } else {
+        for (uint32_t k = 0; k < 4 && at + k < total; ++k) db[at + k] = static_cast<uint8_t>(v >> (8 * k));
     }
 }
 
@@ -373,9 +407,20 @@ int qpadl_pir_delta_encode(const uint32_t *entries_dev, uint64_t n, uint32_t E, 
     if (!entries_dev || !db_dev || !delta_shape_ok(n, E, w)) return QPADL_EINVAL;
     const uint64_t C = (n + E - 1) / E;
     if (E > kMaxEncodeEntries) return QPADL_EINVAL;
+    const cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     if (E <= kShortEntries) {
-        delta_encode_short_kernel<<<static_cast<unsigned>((C + kEncCols - 1) / kEncCols), kEncThreads, kEncCols * (E | 1u) * 4,
-                                    reinterpret_cast<cudaStream_t>(stream)>>>(entries_dev, n, E, w, C, db_dev);
+        const int sms = num_sms_current();
+        if (sms <= 0) return QPADL_ECUDA;
+        const uint32_t cols = C > (uint64_t)sms * kEncCols ? kEncCols : 32u;
+        const auto kernel = cols == 32u ? delta_encode_short_kernel<32> : delta_encode_short_kernel<kEncCols>;
+        kernel<<<static_cast<unsigned>((C + cols - 1) / cols), kEncThreads, cols * (E | 1u) * 4, s>>>(entries_dev, n, E, w, C,
+                                                                                                   db_dev);
+        return cudaGetLastError() == cudaSuccess ? QPADL_OK : QPADL_ECUDA;
+    }
+    if (C <= kFewBlocks) {
+        const uint64_t threads = ((4 + (uint64_t)w * (E - 1)) * C + 3) / 4;
+        delta_encode_few_kernel<<<static_cast<unsigned>((threads + kEncThreads - 1) / kEncThreads), kEncThreads, 0, s>>>(
+            entries_dev, n, E, w, static_cast<uint32_t>(C), db_dev);
         return cudaGetLastError() == cudaSuccess ? QPADL_OK : QPADL_ECUDA;
     }
     const int vec = (E % 4 == 0) && (reinterpret_cast<uintptr_t>(entries_dev) & 15u) == 0;

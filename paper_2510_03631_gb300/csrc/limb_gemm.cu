@@ -52,6 +52,7 @@
 // N = (4 - u) * BN/4 and the epilogue drains only those columns, adding
 // each shift times 2^{8t}.  That runs 10 of the 16 (plane, shift) blocks
 // with MMAs no narrower than BN/4.
+#include <algorithm>
 #include <cstdint>
 #include <type_traits>
 #include <cuda_fp16.h>
@@ -970,9 +971,13 @@ cudaError_t launch_mod_p_signed(uint32_t *x, uint64_t n, uint32_t p, int num_sms
 
 cudaError_t launch_centred_rows(const uint32_t *Q, uint32_t B, uint64_t C, uint32_t p, __half *L, uint64_t pitch,
                                 int num_sms, cudaStream_t stream, uint32_t *zero, uint64_t zero_words) {
-    (void)num_sms;
     if (B == 0 || C == 0 || B > 65535) return cudaErrorInvalidValue;   // callers pass chunks of at most 1024
-    const dim3 grid(static_cast<unsigned>((C + 2047) / 2048), B);
+    uint64_t nx = (C + 2047) / 2048;
+    // few columns make few blocks, but there can be many outputs to zero: enough blocks for four per SM, a thousand words
+    // each (100000 x 128, 5 queries: 26 us a call with five blocks, 19 so)
+    const uint64_t want = std::min<uint64_t>(4ull * num_sms, zero ? (zero_words + 1023) / 1024 : 0);
+    if (nx * B < want) nx = (want + B - 1) / B;
+    const dim3 grid(static_cast<unsigned>(nx), B);
     centred_rows_kernel<<<grid, 256, 0, stream>>>(Q, C, p, L, pitch, zero, zero_words);
     return cudaGetLastError();
 }
