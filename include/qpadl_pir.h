@@ -510,10 +510,12 @@ int qpadl_chor_answer_batch(qpadl_chor *h, const uint32_t *Q_dev, uint32_t B, ui
  *   256) of at least this many queries run on the tensor cores (exact parities
  *   of 4-bit products); smaller ones the masked-XOR scan.  257 disables the
  *   tensor cores.  Until it or QPADL_CHOR_OPT_SCAN_FORM is set, the library
- *   chooses by record length (1 below 512 words, 3 below 1024, else 9), also
+ *   chooses by record length (1 below 512 words, 3 below 1024, else 9, or 17
+ *   from 8192 words on up to 512 rows), also
  *   for what a larger batch leaves after its tiles of 128 queries (which a
  *   database of up to 64 MiB takes along), and the option reads as that
- *   number. */
+ *   number.  Up to 256 rows of at least 2048 words it
+ *   also answers batches of 33 and more by XOR tables of four rows. */
 #define QPADL_CHOR_OPT_M4RM_MIN_BATCH 1
 /* QPADL_CHOR_OPT_SCAN_FORM (-1..3, default -1): inner loop of the masked-XOR
  * scan.  Bit 1: each thread covers 8 database words per row (at most 16

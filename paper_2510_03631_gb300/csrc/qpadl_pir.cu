@@ -113,17 +113,21 @@ constexpr int kMaxN = 16384;
 // 1024 10.5 / 8.4 (two queries 11.4 / 9.0), 2048 x 2048 10.6 / 8.6 (10.9 / 9.4), 4096 x 4096 10.5 / 8.5 (12.2 /
 // 12.5), 6144 x 6144 12.4 / 12.4 (16.5 / 20.6), 8192 x 8192 14.4 / 16.5.
 constexpr uint64_t kRawCells = 16ull << 20, kRawCells2 = 4ull << 20, kRawCols = 4096;
-// Smallest Chor batch on the tensor cores for records of W words, unless the caller chose one.  Their
+// Smallest Chor batch on the tensor cores for `rows` records of W words, unless the caller chose one.  Their
 // time hardly depends on the batch up to 64 queries; the scan's grows with it and its column tiles
 // are 1024 words wide (one query; a narrower record leaves their threads idle).  Measured, scan
 // against tensor cores: 16 words (2^20 rows of 4: 536 against 83 us; 200,000 of 16: 111 / 20), 256
 // words (60,000 rows) 41 / 26 us at one query; 768 words (2^18 rows) 148 / 187 us at one, 159 / 189
-// at 2, 195 / 189 at 3; 8192 words (32,768 rows) 241 / 251 at 8 and 356 / 251 at 9.
-uint32_t chor_large_batch(uint32_t W) { return W < 512 ? 1u : (W < 1024 ? 3u : 9u); }
+// at 2, 195 / 189 at 3; 8192 words (32,768 rows) 241 / 251 at 8 and 356 / 251 at 9.  A tensor-core column tile
+// ends with a fixed cost, which few rows do not repay: 16384 words, 9 and 16 queries 9 and 11 us against 19
+// on 32 rows, 20 and 24 against 24 on 512, 30 and 34 against 31 on 1000.
+uint32_t chor_large_batch(uint64_t rows, uint32_t W) {
+    return W < 512 ? 1u : (W < 1024 ? 3u : (W >= 8192 && rows <= 512 ? 17u : 9u));
+}
 // Whether the caller's threshold applies (choosing a scan form asks for the scan below it), and the one in force.
 bool chor_min_batch_set(const qpadl_chor *h) { return h->large_set || h->scan_form >= 0; }
 uint32_t chor_min_batch(const qpadl_chor *h) {
-    return chor_min_batch_set(h) ? h->large_min_batch : chor_large_batch(h->words);
+    return chor_min_batch_set(h) ? h->large_min_batch : chor_large_batch(h->rows, h->words);
 }
 uint32_t chor_units(uint64_t rows) { return static_cast<uint32_t>((rows + kChorGemmUnitRows - 1) / kChorGemmUnitRows); }
 // Goldberg sums stay exact (|centred sum| < 2^31, unsigned sum < 2^32) below this many columns
@@ -1370,6 +1374,31 @@ int chor_answer_gemm(qpadl_chor *h, const uint32_t *Q, uint32_t B, uint32_t *out
     return QPADL_OK;
 }
 
+// B queries by four-row XOR tables, 256 at a time.
+int chor_answer_m4rm(qpadl_chor *h, const uint32_t *Q, uint32_t B, uint32_t *out, cudaStream_t s) {
+    CUtensorMap db_map;
+    if (!encode_2d(&db_map, CU_TENSOR_MAP_DATA_TYPE_UINT32, h->db, h->words, h->rows, 4ull * h->words, kChorM4TileWords,
+                   kChorM4BandRows, CU_TENSOR_MAP_SWIZZLE_NONE))
+        return QPADL_ECUDA;
+    for (uint32_t b0 = 0; b0 < B; b0 += kChorMaxBatch) {
+        const uint32_t Bc = std::min(B - b0, kChorMaxBatch);
+        QPADL_CU(launch_chor_words(Q + (uint64_t)b0 * h->qw, h->qw, Bc, h->rows, h->qt, h->num_sms, s));
+        QPADL_CU(launch_chor_m4rm(db_map, h->qt, h->rows, h->words, Bc, out + (uint64_t)b0 * h->words, h->num_sms,
+                                  h->d_status, s));
+    }
+    return QPADL_OK;
+}
+
+// Whether they are faster: at most one unit of rows, whose column tiles cost the tensor cores mostly their ends, long
+// records and more than a few queries.  Tensor cores against tables (us): 4096 words, 32 rows, 33 / 128 / 256 queries
+// 13 / 18 / 27 against 9 / 10 / 14, 256 rows 13 / 18 / 27 against 14 / 16 / 24; 16384 words, 256 rows 30 / 49 / 90 against
+// 32 / 36 / 54, 512 rows 35 / 56 / 102 against 55 / 60 / 89; 2048 words, 200 rows, 48 queries 9 / 9.
+bool chor_m4rm_faster(const qpadl_chor *h, uint32_t B) {
+    return !chor_min_batch_set(h) && h->rows <= kChorGemmUnitRows && h->words >= 2048 && B >= 33 &&
+           (uint64_t)h->words * B >= 131072;
+}
+
+
 // How many of a batch's queries, the first ones, take the tensor cores: a threshold set by the caller decides for every
 // chunk of 256 as a whole, the library's own for all tiles and for what is left after them, unless that shares
 // their launch (1024 rows of 512 words, 129 queries: 12 us so, 19 with a scan for the last).
@@ -1394,6 +1423,7 @@ int qpadl_chor_answer_batch(qpadl_chor *h, const uint32_t *Q_dev, uint32_t B, ui
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const uint64_t W = h->words;
     QPADL_CU(cudaMemsetAsync(out_dev, 0, 4ull * W * B, s));
+    if (chor_m4rm_faster(h, B)) return chor_answer_m4rm(h, Q_dev, B, out_dev, s);
     const uint32_t tensor = chor_tensor_queries(h, B);
     if (tensor) {
         const int rc = chor_answer_gemm(h, Q_dev, tensor, out_dev, s);

@@ -81,3 +81,11 @@ def test_option_reads_as_the_threshold_in_force():
 @pytest.mark.parametrize("min_batch", [None, 1])
 def test_tiles_of_one_launch(rows, bits, B, min_batch):
     _check(rows, bits, B, inputs.chor_db(rows, bits, seed=rows + B), inputs.chor_queries(B, rows, seed=B), min_batch)
+
+
+# few rows of long records: XOR tables of four rows (chunks of 256, a short last one), and the scan up to 16 queries
+@pytest.mark.parametrize("rows", [1, 63, 64, 65, 255, 256, 257])
+@pytest.mark.parametrize("bits,B", [(2048 * 32, 64), (2048 * 32 + 128, 129), (4096 * 32, 33), (4096 * 32, 290), (8192 * 32, 16),
+                                    (8192 * 32 + 1920, 17)])
+def test_few_rows_of_long_records(rows, bits, B):
+    _check(rows, bits, B, inputs.chor_db(rows, bits, seed=rows + B), inputs.chor_queries(B, rows, seed=bits), None)
