@@ -250,11 +250,13 @@ __global__ void __launch_bounds__(kEncThreads) delta_encode_short_kernel(const u
 
 // The same for few blocks (columns): their rows are so short that the database is written as one run of bytes, four to
 // a thread, each from two neighbouring entries.  The tile above would be mostly columns past the last one: one block of
-// 2^20 entries, one byte, 138 us in tiles, FEWFIG.
-constexpr uint64_t kFewBlocks = 16;
+// 2^20 entries, one byte, 138 us in tiles, 8 so.
+// A byte costs it the same whatever the rest, so wider digits leave it earlier: 2^24 entries, 25 blocks, one and four bytes
+// 94 and 220 us in tiles, 45 and 175 so; 41 blocks 60 and 136.
+constexpr uint64_t few_blocks(uint32_t w) { return w == 1 ? 40 : (w == 2 ? 32 : 28); }
 __global__ void __launch_bounds__(kEncThreads) delta_encode_few_kernel(const uint32_t *__restrict__ x, uint64_t n, uint32_t E,
                                                                        uint32_t w, uint32_t C, uint8_t *__restrict__ db) {
-    const uint32_t total = (4 + w * (E - 1)) * C;   // at most 16 x 4 x 2^22 bytes
+    const uint32_t total = (4 + w * (E - 1)) * C;   // at most 28 x 4 x 2^22 bytes
     const uint32_t at = 4 * (blockIdx.x * kEncThreads + threadIdx.x);
     if (at >= total) return;
     uint32_t row = at / C, c = at - row * C, v = 0;
@@ -417,7 +419,7 @@ int qpadl_pir_delta_encode(const uint32_t *entries_dev, uint64_t n, uint32_t E, 
                                                                                                    db_dev);
         return cudaGetLastError() == cudaSuccess ? QPADL_OK : QPADL_ECUDA;
     }
-    if (C <= kFewBlocks) {
+    if (C <= few_blocks(w)) {
         const uint64_t threads = ((4 + (uint64_t)w * (E - 1)) * C + 3) / 4;
         delta_encode_few_kernel<<<static_cast<unsigned>((threads + kEncThreads - 1) / kEncThreads), kEncThreads, 0, s>>>(
             entries_dev, n, E, w, static_cast<uint32_t>(C), db_dev);

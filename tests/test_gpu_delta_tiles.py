@@ -86,3 +86,27 @@ def test_decode_warps_per_block(E, w, B):
     exp = np.stack([oracle.delta_decode(digits[b], E, w) for b in range(B)])
     assert np.array_equal(got[:B * E].reshape(B, E), exp)
     assert (got[B * E:] == 0xFFFFFFFF).all()
+
+
+# few long blocks, written as one run of bytes: the first column counts past the line too, ragged last blocks, the database
+# on and off a 4-byte boundary
+@pytest.mark.parametrize("C", [1, 2, 3, 5, 16, 28, 29, 32, 33, 40, 41])
+@pytest.mark.parametrize("E,short", [(81, 0), (82, 80), (1001, 3), (4097, 4000)])
+@pytest.mark.parametrize("w", [1, 2, 3, 4])
+def test_encode_of_few_blocks(C, E, short, w):
+    n = C * E - short
+    C = -(-n // E)
+    x = inputs.uniform_u32(n, seed=n + w, tag=inputs.TAG_MISC)
+    for at in (0, 1):
+        buf = torch.full((pir.delta_rows(E, w) * C + at + 5,), 0xAB, dtype=torch.uint8, device="cuda")
+        end = buf.numel() - 5
+        pir.qpadl_pir_delta_encode(torch.from_numpy(x.view(np.int32)).cuda(), E, w, buf[at:end])
+        v = np.concatenate([x, np.full(C * E - n, x[-1], dtype=np.uint32)]).reshape(C, E)
+        d = v[:, 1:] - v[:, :-1]
+        exp = np.empty((4 + (E - 1) * w, C), dtype=np.uint8)
+        for k in range(4):
+            exp[k] = (v[:, 0] >> np.uint32(8 * k)) & 255
+        for k in range(w):
+            exp[4 + k::w] = ((d >> np.uint32(8 * k)) & 255).T
+        assert np.array_equal(buf[at:end].cpu().numpy().reshape(-1, C), exp)
+        assert (buf[end:] == 0xAB).all() and (at == 0 or int(buf[0]) == 0xAB)
