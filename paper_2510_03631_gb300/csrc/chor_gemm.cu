@@ -28,11 +28,11 @@
 // leave room for one plane, so each unit would be transposed four times), in one launch as far as the scratch
 // holds their expanded bits.
 //
-// Measured (2^18 records of 3 KB, 805 MB): 64 queries 195 us, 128 queries 303 us; the kernels it
+// Measured (2^18 records of 3 KB, 805 MB): 64 queries 195 us, 128 queries 300 us; the kernels it
 // replaced took 1,085 and 1,130 us there (four-Russians tables in shared memory) and 606 us at 32
 // queries (masked scan).  What bounds it: at 128 queries the tensor pipe is 59% and the ALUs 63% busy,
 // at 64 queries 45% and 63% (HBM floor 120 us): the chain transpose -> planes -> MMA, with about six
-// units in flight.  Tried on the way: one producer for both operand streams (396 us at 128: the query
+// units in flight.  At the 80 registers that 768 threads leave, the kernels for 32 and 64 queries spill 50 bytes.  Tried on the way: one producer for both operand streams (396 us at 128: the query
 // ring held the database back); one issuing warp (an MMA costs its lane about 42 cycles and each wait
 // 110); byte permutes instead of ldmatrix for step 1 (the ALUs' 64 lanes per clock); both steps in the
 // same warps (373 us).

@@ -22,7 +22,7 @@
 // to the bits that count and summed in exact packed FP32 steps (high_limbs).  32768 x 32768, 256 vectors, back
 // to back: four limbs 1308 us, this kernel 1190; single calls 1132 and 1024, of which 860 are left when the
 // drains do nothing (a timing copy) and 95 go when their conversions are left out.  Hint of 1024
-// columns 5336 -> 4677 us.  All three limbs through F2I 1670 us; sixteen epilogue warps 1160;
+// columns 5390 -> 4550 us.  All three limbs through F2I 1670 us; sixteen epilogue warps 1160;
 // a whole half's columns in registers first (setmaxnreg 208) 1090; one issue block per 64 columns
 // instead of per half 1140 (single calls).
 //
@@ -35,8 +35,8 @@
 // each stage, warp 2 the vector boxes, warp 1 of the leader issues the MMAs, warps 4..11 drain.
 //
 // Schedule.  Tiles are dealt round-robin, the vector tiles of one row tile to neighbouring clusters.
-// Where whole tiles leave the last wave too empty every tile is cut into the same few column ranges, dealt
-// range by range, whose parts add into a zeroed output (exact: addition mod 2^32 commutes).
+// Where whole tiles leave the last wave too empty, or clusters idle, every tile is cut into the same column ranges,
+// dealt range by range, whose parts add into a zeroed output (exact: addition mod 2^32 commutes).
 #include <cstdint>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
