@@ -5,8 +5,8 @@
 // q-bar queries against one database) and for the offline hint
 // H = D * A (X = columns of A; Sec. 5.3 offline precomputation).
 //
-// The matrix holds the digits minus 128 (one fp16 copy serves these tiles and the
-// CTA-pair ones); 128 times a vector's sum, made with its limbs, is added at the end.
+// The matrix holds the digits minus p / 2 (one fp16 copy serves these tiles and the
+// CTA-pair ones); p / 2 times a vector's sum, made with its limbs, is added at the end.
 //
 // Exactness.  Each X word is split into four balanced byte limbs
 // x = sum_k 2^{8k} c_k with c_k in [-128, 127] (low byte, minus 256 and a

@@ -20,7 +20,7 @@ cudaError_t prepare_limb_gemm_kernels();
 int limb_gemm_bn_for(uint32_t nv);
 
 // out[i * ld_m + v * ld_b] = sum_j D[i][j] X[v][j] mod 2^32, i < M, v < NV,
-// j < K; a_map covers D - 128 as fp16 (box 64 x 128), b_map the limbs (box 64 x bn), sums
+// j < K; a_map covers D - p / 2 as fp16 (box 64 x 128), b_map the limbs (box 64 x bn), sums
 // the vectors' sums.
 cudaError_t launch_limb_gemm(int bn, const CUtensorMap &a_map, const CUtensorMap &b_map, const VecSums &sums,
                              uint32_t *out, uint64_t ld_m, uint64_t ld_b, uint32_t M, uint32_t NV,

@@ -14,7 +14,7 @@
 // int32 after every exact chunk and recombined as sum_k 2^{8k} s_k in uint32
 // arithmetic.  The chunk depth follows the products' bound: digits times
 // centred field elements (magnitude <= 255 * 128) take 512-deep chunks, whose sums
-// stay below 2^24; limbs, or digits centred to d - 128, times limbs (client Query/Recover; Response;
+// stay below 2^24; limbs, or digits centred to d - p / 2, times limbs (client Query/Recover; Response;
 // magnitude <= 2^14) take 1024-deep chunks, whose partial sums never exceed 2^24 in magnitude.
 // Every integer of magnitude <= 2^24 is an fp32 value, so no partial sum is
 // ever rounded either way.

@@ -27,7 +27,7 @@ __host__ __device__ inline uint32_t pair_b_box_rows(int bn, bool planed, int u) 
 int limb_gemm_pair_bn_for(uint32_t nv);
 
 // out[v * M + i] = sum_j D[i][j] X[v][j] mod 2^32 (i < M, v < NV, j < K) on CTA pairs: a_map covers
-// D - 128 as fp16 (box 64 x 128), bm.m[0] four byte limbs per vector (box 64 x 128), sums the vectors' sums.
+// D - p / 2 as fp16 (box 64 x 128), bm.m[0] four byte limbs per vector (box 64 x 128), sums the vectors' sums.
 // Launched as the programmatic dependent of the kernel before it in the stream, which makes the limbs and, when
 // limb_gemm_pair_splits, zeroes out; everything earlier must have completed when that one starts.
 cudaError_t launch_limb_gemm_pair(const CUtensorMap &a_map, const PairBMaps &bm, const VecSums &sums, uint32_t *out,

@@ -5,10 +5,10 @@
 // often every digit is multiplied.  fp16 holds every integer up to 2048, so a limb may have 11 bits
 // (balanced: -1024 .. 1023) instead of 8, and 32 bits take three limbs (11 + 11 + 10) instead of
 // four: a quarter less tensor work and operand traffic.  The price is a shorter exact sum: digits centred to
-// d - 128 times limbs are at most 2^17 in magnitude, so fp32 sums are exact for 128 columns (2^24;
+// d - p / 2 (-128 .. 127) times limbs are at most 2^17 in magnitude, so fp32 sums are exact for 128 columns (2^24;
 // every integer of at most that magnitude is an fp32 value), and the accumulators are drained to
-// int32 every 128 columns.  Centring adds 128 sum_j X[b][j] to every output of vector b; that word
-// comes with the limbs.
+// int32 every 128 columns.  Centring takes p / 2 times sum_j X[b][j] from every output of vector b; the sums
+// come with the limbs.
 //
 // Tile.  256 rows x 64 H vectors over a pair of SMs (tcgen05 cta_group::2).  A half is 64 vectors
 // = 192 limb columns; the two accumulators of 192 TMEM columns take turns: with H = 2 half 0 and

@@ -14,11 +14,12 @@ constexpr uint32_t kTriGroup = 32;
 
 // Where the sums of NV vectors lie behind their limbs: three fp16 rows of `pitch` each (then the sums end within
 // 8 NV pitch bytes), or four byte limbs for limb_gemm_pair.cu and limb_gemm.cu (limb k of vector v in row 4 v + k).
-inline VecSums tri_sums(const __half *L, uint32_t nv, uint64_t pitch, uint32_t parts) {
-    return VecSums{reinterpret_cast<const uint32_t *>(L + 3ull * nv * pitch), nv, parts};
+// The GEMMs need the digits' centre beside them, the kernels that make them do not.
+inline VecSums tri_sums(const __half *L, uint32_t nv, uint64_t pitch, uint32_t parts, uint32_t centre = 0) {
+    return VecSums{reinterpret_cast<const uint32_t *>(L + 3ull * nv * pitch), nv, parts, centre};
 }
-inline VecSums four_sums(const __half *L, uint32_t nv, uint64_t pitch, uint32_t parts) {
-    return VecSums{reinterpret_cast<const uint32_t *>(L + 4ull * nv * pitch), nv, parts};
+inline VecSums four_sums(const __half *L, uint32_t nv, uint64_t pitch, uint32_t parts, uint32_t centre = 0) {
+    return VecSums{reinterpret_cast<const uint32_t *>(L + 4ull * nv * pitch), nv, parts, centre};
 }
 
 cudaError_t prepare_limb_gemm_tri_kernels();

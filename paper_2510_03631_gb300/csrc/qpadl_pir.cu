@@ -52,7 +52,7 @@ struct qpadl_db {
     int u8_kstep = 0;                // QPADL_OPT_U8_KSTEP (0 = per tile width default)
     int pair_gemm = 1;               // QPADL_OPT_PAIR_GEMM
     __half *d16 = nullptr;           // digits as fp16, R x pitch (Z_p handles)
-    __half *d16c = nullptr;          // digits minus 128 as fp16, R x pitch (lattice handles, either tile form)
+    __half *d16c = nullptr;          // digits minus p / 2 as fp16, R x pitch (lattice handles, either tile form)
     uint64_t pitch = 0;              // roundup(C, 8)
     CUtensorMap a_map, ac_map;       // over d16, d16c
     __half *limbs = nullptr;         // limb scratch
@@ -263,7 +263,7 @@ bool use_tri(const qpadl_db *db) { return db->pair_gemm && db->num_sms >= 2; }
 // The fp16 copy that batches and hints of a lattice handle read, whatever its tile option says: a change
 // of the option after qpadl_pir_reserve builds nothing.
 int ensure_batch_copy(qpadl_db *db, cudaStream_t stream) {
-    return build_f16_copy(db, &db->d16c, &db->ac_map, kCentre, stream);
+    return build_f16_copy(db, &db->d16c, &db->ac_map, static_cast<int>(digit_centre(db->prm.p)), stream);
 }
 
 int ensure_limbs(qpadl_db *db, uint64_t bytes) {
@@ -303,7 +303,7 @@ int run_tri_gemm(qpadl_db *db, const __half *limbs, uint32_t NV, uint32_t parts,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return QPADL_ECUDA;
-    QPADL_CU(launch_limb_gemm_tri(db->ac_map, b_map, tri_sums(limbs, NV, db->pitch, parts), out, ld_m, ld_b,
+    QPADL_CU(launch_limb_gemm_tri(db->ac_map, b_map, tri_sums(limbs, NV, db->pitch, parts, digit_centre(db->prm.p)), out, ld_m, ld_b,
                                   static_cast<uint32_t>(db->prm.rows), NV, C, plan, db->num_sms, db->d_status, stream));
     return QPADL_OK;
 }
@@ -315,7 +315,7 @@ int run_limb_gemm(qpadl_db *db, const __half *limbs, uint32_t NV, uint32_t parts
     if (!encode_2d(&b_map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, limbs, db->prm.cols, 4ull * NV, db->pitch * 2,
                    kLimbBoxK, static_cast<uint32_t>(bn), CU_TENSOR_MAP_SWIZZLE_128B))
         return QPADL_ECUDA;
-    QPADL_CU(launch_limb_gemm(bn, db->ac_map, b_map, four_sums(limbs, NV, db->pitch, parts), out, ld_m, ld_b,
+    QPADL_CU(launch_limb_gemm(bn, db->ac_map, b_map, four_sums(limbs, NV, db->pitch, parts, digit_centre(db->prm.p)), out, ld_m, ld_b,
                               static_cast<uint32_t>(db->prm.rows), NV, db->prm.cols, db->num_sms, db->d_status, stream));
     return QPADL_OK;
 }
@@ -351,7 +351,7 @@ int answer_f16(qpadl_db *db, const uint32_t *Q, uint32_t B, uint32_t *ans, __hal
         if (!encode_2d(&bm.m[0], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, limbs, C, 4ull * B, db->pitch * 2, kLimbBoxK,
                        pair_b_box_rows(256, false, 0), CU_TENSOR_MAP_SWIZZLE_128B))
             return QPADL_ECUDA;
-        QPADL_CU(launch_limb_gemm_pair(db->ac_map, bm, four_sums(limbs, B, db->pitch, parts), ans,
+        QPADL_CU(launch_limb_gemm_pair(db->ac_map, bm, four_sums(limbs, B, db->pitch, parts, digit_centre(db->prm.p)), ans,
                                        static_cast<uint32_t>(R), B, C, db->num_sms, db->d_status, stream));
         return QPADL_OK;
     }

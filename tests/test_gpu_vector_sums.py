@@ -35,3 +35,26 @@ def test_blocks_of_columns(C, B, pair):
     assert pir.qpadl_pir_status(db) == pir.QPADL_OK
     assert np.array_equal(pir.as_u32(out).reshape(B, R), oracle.answer_batch(D, Q, threads=oracle.max_threads()))
     db.close()
+
+
+@pytest.mark.parametrize("pair", [1, 0])
+@pytest.mark.parametrize("B", [3, 66, 150])
+@pytest.mark.parametrize("p", [2, 4, 16, 128])   # digits are centred by p / 2
+@pytest.mark.parametrize("largest", [False, True])
+def test_centre_follows_p(p, B, pair, largest):
+    R, C = 270, 2100
+    D = np.full((R, C), p - 1, dtype=np.uint8) if largest else inputs.db_digits(R, C, p, seed=p)
+    Q = inputs.uniform_u32(B * C, seed=p + B, tag=inputs.TAG_MISC).reshape(B, C)
+    db = pir.qpadl_pir_setup(pir.params(R, C, B, p=p), torch.from_numpy(D).cuda())
+    pir.qpadl_pir_set_option(db, pir.QPADL_OPT_PAIR_GEMM, pair)
+    pir.qpadl_pir_set_option(db, pir.QPADL_OPT_U8_MAX_BATCH, 0)
+    out = torch.empty(B * R, dtype=torch.int32, device="cuda")
+    pir.qpadl_pir_answer_batch(db, pir.from_u32(Q.reshape(-1)), out, path=1)
+    H = torch.empty(R * B, dtype=torch.int32, device="cuda")
+    pir.qpadl_pir_hint(db, pir.from_u32(np.ascontiguousarray(Q.T).reshape(-1)), H)
+    torch.cuda.synchronize()
+    assert pir.qpadl_pir_status(db) == pir.QPADL_OK
+    exp = oracle.answer_batch(D, Q, threads=oracle.max_threads())
+    assert np.array_equal(pir.as_u32(out).reshape(B, R), exp)
+    assert np.array_equal(pir.as_u32(H).reshape(R, B), exp.T)
+    db.close()
